@@ -105,9 +105,9 @@ CSTONE_API int cstone_keys(const double* x, const double* y, const double* z, in
                 uint64_t* keys, void* stream);
 
 /* ------------------------------------------------------------------------------------------
- * Radix sort_by_key of the particle keys with the identity permutation as values (Sec. 4;
- * Table 1 caption). Stable: equal keys keep ascending input index. LSD, 8-bit digits; every pass
- * counts the digits of every tile, scans the counts and scatters each tile's digit runs.
+ * Sort_by_key of the particle keys with the identity permutation as values (Sec. 4; Table 1
+ * caption). Stable: equal keys keep ascending input index. A sample sort of the pairs (key, index):
+ * at most two rounds of splitting, then every part sorted in shared memory.
  *   keys_in   [n] uint64 input keys (may alias keys_out).
  *   keys_out  [n] uint64 sorted keys P.
  *   perm      [n] uint32 output: keys_out[j] = keys_in[perm[j]].
@@ -122,14 +122,14 @@ CSTONE_API int cstone_sort(const uint64_t* keys_in, uint64_t* keys_out, uint32_t
  * cstone_sort with the same result). It is for callers that cannot call cudaMalloc and cannot
  * hand out a workspace: code that runs inside a memory allocator's own callbacks, or inside a
  * framework that owns and budgets all device memory of the process, where a new allocation is
- * not allowed. Its scratch is a fixed static device array inside this library (about 13 MB,
+ * not allowed. Its scratch is a fixed static device array inside this library (about 15 MB,
  * held on every GPU that loads the library until the process exits), so n is limited to
  * CSTONE_SORT_STATIC_MAX_KEYS; a larger n returns CSTONE_ERR_INVALID_ARG without touching the
  * GPU. The first call on a device looks up the array's device address (cudaGetSymbolAddress):
  * make that first call before any stream capture. All calls share the one array, so calls that
  * can overlap on the GPU (other streams, other host threads) race and must be serialised by the
  * caller. Each call clears what has to start at zero; otherwise the array keeps the last call's
- * intermediate keys, permutation and digit counts, which the next call overwrites before reading.
+ * intermediate keys, permutation and tables, which the next call overwrites before reading.
  * The device address is cached per device ordinal for the life of the process: it does not
  * survive cudaDeviceReset (or any teardown of the primary context) in the host application.
  * `stream` must belong to the current device; a stream of another device returns
@@ -271,7 +271,7 @@ CSTONE_API int cstone_keys_batched(const double* x, const double* y, const doubl
                                    uint64_t* keys, void* ws, size_t ws_bytes, void* stream);
 
 /* Stable sort of every segment's keys (segments given by seg_offsets), one set of launches per
- * digit pass for all segments: tiles are aligned to segments and digits are offset per segment.
+ * round of splitting for all segments (cstone_sort's method; a small segment is sorted by one block).
  * perm holds global input indices. keys_in must not alias keys_out. Asynchronous. */
 CSTONE_API int cstone_sort_segmented_workspace_size(int64_t n, int32_t n_segs, size_t* bytes);
 CSTONE_API int cstone_sort_segmented(const uint64_t* keys_in, uint64_t* keys_out, uint32_t* perm, int64_t n,
@@ -535,7 +535,7 @@ CSTONE_API int cstone_rebalance_focus(const uint64_t* leaves, const uint32_t* co
  * point below is its cstone_* counterpart with uint32_t keys and 10 levels: a key of this
  * family is the top 30 bits of the 63-bit key of the same point (the grid of 2^10 cells per
  * axis nests in the one of 2^21 cells, and both curves nest level by level); end key 8^10 = 2^30;
- * level_offsets has CSTONE30_LEVELS + 2 = 12 entries; the sort takes 4 passes of 8-bit digits;
+ * level_offsets has CSTONE30_LEVELS + 2 = 12 entries; the sort of large sets takes 4 stable passes of 8-bit digits;
  * a leaf that is a single level-10 cell is not split whatever its count. Arguments, ownership,
  * errors and synchronisation are those of the 63-bit entry point. The bounding cube
  * (cstone_bbox) does not depend on the key length.

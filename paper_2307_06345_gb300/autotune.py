@@ -1,4 +1,4 @@
-"""Autotuner for the tile shapes of the radix sort and of the leaf loop.
+"""Autotuner for the tile shapes of the sort and of the leaf loop.
 
 Run on the target GPU (``python -m paper_2307_06345_gb300.autotune``). Every candidate shape is
 compiled into its own copy of the library (only the affected translation unit is rebuilt), timed
@@ -25,8 +25,9 @@ import torch
 
 from . import _build
 
-SORT_CANDIDATES = [{"threads": 256, "items": i, "min_blocks": b}
-                   for i, b in ((8, 5), (8, 6), (10, 4), (10, 5), (12, 4), (14, 3), (14, 4), (16, 3), (16, 4))]
+# tile of the sort's scatter
+SORT_CANDIDATES = [{"threads": t, "items": i, "min_blocks": b}
+                   for t, i, b in ((256, 8, 5), (256, 12, 4), (256, 16, 3), (384, 8, 3), (512, 8, 2), (512, 12, 2))]
 # the leaf loop stages a tile of elements in shared memory: more than 8 per thread exceeds 48 KB
 LEAVES_CANDIDATES = [{"items": i} for i in (4, 6, 8)]
 

@@ -1,20 +1,29 @@
-// Stable LSD radix sort_by_key of the particle keys with the identity permutation as values
-// (Sec. 4 and the caption of Table 1: the particle keys are sorted with a permutation that
-// records where each particle went). 63-bit keys in 64-bit words take 8 passes of 8-bit digits,
-// 30-bit keys in 32-bit words take 4.
+// Stable sort_by_key of the particle keys with the identity permutation as values (Sec. 4 and the
+// caption of Table 1: the particle keys are sorted with a permutation that records where each
+// particle went).
 //
-// Each digit pass reads a tile of keys (and values), ranks them within the tile (the lanes of a warp
-// holding the same digit are found with one ballot per digit bit, which measured much cheaper than
-// a warp match instruction), stages the tile in shared memory in digit order (the keys, then the
-// values, through one buffer) and writes each digit's run contiguously at the tile's output
-// position for that digit; the first pass generates the identity values instead of reading them.
-// Ahead of every pass, a count of every tile's digits
-// and a two-level scan of the counts give each tile its output positions, so no tile waits on
-// another (a decoupled look-back between tiles, measured first, spent a third of the sort's time
-// waiting on predecessors); the same counts give the digits' totals, whose scan over the digits
-// places each digit's run, so no separate histogram pass reads the keys. A segmented sort aligns its tiles to the segments, scans the counts of all tiles
-// at once, and takes a tile's position within its segment as the difference to the segment's
-// first tile, added to the segment's digit offsets.
+// A sample sort on the pairs (key, input index). The pairs are all different, so their order is the
+// stable order of the keys and no step has to keep the input order. Each bucket of more than kSmall
+// pairs (at first the whole set, or every segment) is split at pairs drawn from a sorted sample of
+// it, so its parts are of nearly equal size whatever the distribution of the keys, with any number
+// of equal keys; a part of at most kSmall pairs is sorted in shared memory by one block and written to
+// its final place. Two rounds of splitting reach every size: a pair moves three times (round 1, round
+// 2, final place), where the eight digit passes of a radix sort move it eight times. 2^27 clump keys
+// take 5.1 ms (count 0.31 and 0.65, scatter 0.82 and 0.92, final sort 1.87; the digit passes took
+// 7.2), 2^25 Plummer keys 1.3 ms (1.9), 65,536 uniform keys 65 us in 7 launches (200 in 40). Per round:
+//
+//   sample   one block per bucket sorts a sample and writes the bounds of the parts;
+//   count    every pair's part is found (a table over the leading key bits, then a binary search
+//            among the bounds that share the table entry) and kept as 16 bits, the parts are counted;
+//   plan     one block per bucket turns the counts into positions and lists the parts: small ones for
+//            the final sort, others for the next round;
+//   scatter  tiles of pairs are grouped by part in shared memory and written in runs.
+//
+// The final sort bins a part's pairs by their leading differing bits into about as many bins as
+// pairs, and ranks each pair within its bin by comparison. A bin of more than kHeavy pairs (a tight
+// clump beside sparse surroundings) is binned again over its own range; equal keys are binned by
+// index. Parts that are still larger than kSmall after the last round (an unlucky sample) are
+// sorted by one block each, through merges in global memory above kBig pairs.
 #include <mutex>
 
 #include "common.cuh"
@@ -22,147 +31,881 @@
 namespace CST_NS {
 namespace {
 
+using u16 = unsigned short;
+
+// Tile shape of the scatter (compile-time tuning knobs, set by the build from the autotuner's
+// choice): threads per block, pairs per thread and blocks per SM.
+#ifndef CSTONE_SORT_THREADS
+#define CSTONE_SORT_THREADS 512
+#endif
+#ifndef CSTONE_SORT_ITEMS
+#define CSTONE_SORT_ITEMS 8
+#endif
+#ifndef CSTONE_SORT_MIN_BLOCKS
+#define CSTONE_SORT_MIN_BLOCKS 2
+#endif
+constexpr int kThreads = CSTONE_SORT_THREADS;
+constexpr int kItems = CSTONE_SORT_ITEMS;
+constexpr int kTile = kThreads * kItems;
+static_assert(kThreads >= 256 && kThreads % 32 == 0 && kItems % 2 == 0 && kTile < 65536, "tile shape");
+
+constexpr u32 kMaxParts = 512;  // parts of one bucket
+constexpr int kSmallThreads = 256, kSmallItems = 12, kSmallBlocks = 3;
+constexpr u32 kSmall = kSmallThreads * kSmallItems;  // pairs sorted by one block of the final sort
+constexpr u32 kTarget = kSmall / 2;                  // mean size of the last round's parts
+constexpr int kBigThreads = 1024, kBigItems = 8;
+constexpr u32 kBig = kBigThreads * kBigItems;  // pairs of a sample, and of a chunk of an oversized part
+constexpr u32 kHeavy = 24;                     // pairs of a bin ranked by comparison
+
+__host__ __device__ inline u32 ceil_div(u32 a, u32 b) { return (a + b - 1) / b; }
+
+// Parts of a bucket of `size` > kSmall pairs with `rounds` rounds to go (this one included).
+__device__ inline u32 part_count(u32 size, int rounds) {
+    const u32 full = ceil_div(size, kTarget);
+    if (full <= kMaxParts || rounds == 1) return full < kMaxParts ? full : kMaxParts;
+    // about the square root, so that both rounds have the same number of parts, and few enough
+    // that a tile's runs stay long; more where the second round could not finish the split
+    u32 b = static_cast<u32>(sqrtf(static_cast<float>(full))) + 1u;
+    b = b < 256u ? b : 256u;
+    u32 m = ceil_div(full, 384u);
+    m = m < kMaxParts ? m : kMaxParts;
+    return b > m ? b : m;
+}
+
+__host__ __device__ inline int rounds_for(long long n) {
+    return n <= (long long)kSmall ? 0 : (n <= (long long)kTarget * kMaxParts ? 1 : 2);
+}
+
+// ---------------------------------------------------------------------------- tables
+// Every tile adds to the write positions of all parts of its bucket: each has a line of its own, so
+// that the adds spread over the L2 slices.
+constexpr u32 kPosStride = 32;
+
+enum { kInput = 0, kBufA = 1, kBufB = 2 };  // where a bucket's pairs are
+
+struct Buckets {  // buckets to be split in a round, in the order of their tiles and parts
+    u32* start;
+    u32* size;
+    Key* base;        // a lower bound of the keys
+    u32* first_part;  // index of the bucket's first entry in the part arrays
+    u32* first_tile;  // [count + 1]
+    u32* count;
+};
+
+struct Tables {
+    Buckets big[2];  // buckets of round 1, then of round 2, then the oversized rest in big[0]
+    Key* part_key;   // lower bounds of the parts: keys and indices
+    u32* part_idx;
+    u32* part_pos;   // counts, then write positions, kPosStride words apart
+    uint2* small;    // first pair | size, source buffer in the top two bits of the size
+    Key* small_base;
+    u32* n_small;
+    u16* part_of;    // [n] part of every pair in the current round
+    u32* tile_bucket;  // bucket of every tile in the current round
+};
+
+struct Pairs {  // the three places of pairs; the input's values are its positions
+    const Key* in;
+    Key* a;
+    u32* va;
+    Key* b;  // the output
+    u32* vb;
+};
+
+template <int SRC>
+__device__ __forceinline__ const Key* keys_of(const Pairs& p) {
+    return SRC == kInput ? p.in : (SRC == kBufA ? p.a : p.b);
+}
+template <int SRC>
+__device__ __forceinline__ u32 value_of(const Pairs& p, u32 i) {
+    return SRC == kInput ? i : __ldcg((SRC == kBufA ? p.va : p.vb) + i);
+}
+
+__device__ __forceinline__ int bit_length(u64 v) { return 64 - __clzll(static_cast<long long>(v)); }
+__device__ __forceinline__ bool pair_less(Key a, u32 ia, Key b, u32 ib) { return a < b || (a == b && ia < ib); }
+
+// Exclusive scan over the block; total in *sum (every thread calls it; s_warp: 32 words).
+template <int THREADS>
+__device__ __forceinline__ u32 block_scan(u32 v, u32* s_warp, u32* sum) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    u32 incl = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const u32 t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+    }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    u32 before = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < THREADS / 32; ++w) {
+        const u32 x = s_warp[w];
+        if (w < warp) before += x;
+        all += x;
+    }
+    __syncthreads();  // s_warp may be reused
+    *sum = all;
+    return before + incl - v;
+}
+
+// Lists the segments: small ones for the final sort, the others as round-1 buckets with their tile
+// and part prefixes. One block; also clears the workspace's header.
+__global__ void __launch_bounds__(1024) sort_init_kernel(const long long* __restrict__ seg_offsets, int n_segs,
+                                                         long long n, int rounds, Tables t, WsHeader* hdr) {
+    __shared__ u32 s_warp[32];
+    if (threadIdx.x < sizeof(WsHeader) / 4) reinterpret_cast<u32*>(hdr)[threadIdx.x] = 0u;
+    u32 n_big = 0, n_small = 0, parts = 0, tiles = 0;
+    for (int s0 = 0; s0 < n_segs; s0 += 1024) {
+        const int s = s0 + threadIdx.x;
+        u32 start = 0, size = 0;
+        if (s < n_segs) {
+            start = seg_offsets ? static_cast<u32>(seg_offsets[s]) : 0u;
+            size = seg_offsets ? static_cast<u32>(seg_offsets[s + 1] - seg_offsets[s]) : static_cast<u32>(n);
+        }
+        const bool big = size > kSmall, small = size > 0 && !big;
+        const u32 np = big ? part_count(size, rounds) : 0u, nt = big ? ceil_div(size, kTile) : 0u;
+        u32 all_big, all_small, all_parts, all_tiles;
+        const u32 kb = n_big + block_scan<1024>(big, s_warp, &all_big);
+        const u32 ks = n_small + block_scan<1024>(small, s_warp, &all_small);
+        const u32 kp = parts + block_scan<1024>(np, s_warp, &all_parts);
+        const u32 kt = tiles + block_scan<1024>(nt, s_warp, &all_tiles);
+        if (big) {
+            t.big[0].start[kb] = start;
+            t.big[0].size[kb] = size;
+            t.big[0].base[kb] = 0;
+            t.big[0].first_part[kb] = kp;
+            t.big[0].first_tile[kb] = kt;
+        }
+        if (small) {
+            t.small[ks] = make_uint2(start, size | (static_cast<u32>(kInput) << 30));
+            t.small_base[ks] = 0;
+        }
+        n_big += all_big;
+        n_small += all_small;
+        parts += all_parts;
+        tiles += all_tiles;
+    }
+    if (threadIdx.x == 0) {
+        *t.big[0].count = n_big;
+        *t.big[1].count = 0;
+        *t.n_small = n_small;
+        t.big[0].first_tile[n_big] = tiles;
+        t.big[0].first_part[n_big] = parts;
+    }
+}
+
+// Tile and part prefixes of the buckets that a plan listed (start, size and base are there).
+__global__ void __launch_bounds__(1024) sort_prefix_kernel(Buckets b, u32* clear, int rounds) {
+    __shared__ u32 s_warp[32];
+    const u32 count = *b.count;
+    u32 parts = 0, tiles = 0;
+    for (u32 k0 = 0; k0 < count; k0 += 1024) {
+        const u32 k = k0 + threadIdx.x;
+        const u32 size = k < count ? b.size[k] : 0u;
+        const u32 np = k < count ? part_count(size, rounds) : 0u, nt = ceil_div(size, kTile);
+        u32 all_parts, all_tiles;
+        const u32 kp = parts + block_scan<1024>(np, s_warp, &all_parts);
+        const u32 kt = tiles + block_scan<1024>(nt, s_warp, &all_tiles);
+        if (k < count) {
+            b.first_part[k] = kp;
+            b.first_tile[k] = kt;
+        }
+        parts += all_parts;
+        tiles += all_tiles;
+    }
+    if (threadIdx.x == 0) {
+        b.first_tile[count] = tiles;
+        b.first_part[count] = parts;
+        *clear = 0;
+    }
+}
+
+// ---------------------------------------------------------------------------- sort in one block
+constexpr int kMinBinBits = 6;  // a word of bins for every lane
+
+template <int THREADS, int ITEMS>
+struct BlockSortSmem {
+    static constexpr u32 kCap = THREADS * ITEMS;
+    static constexpr u32 kBins = kCap <= 4096 ? 4096 : 8192;  // a power of two >= kCap
+    static constexpr u32 kGroups = kCap / (kHeavy + 1) + 1;   // bins to be split are disjoint
+    Key K[kCap];  // the pairs in bin order
+    Key red[32];
+    u32 V[kCap];
+    u32 bins[kBins / 2 + 1];  // two 16-bit counts, then starts, per word
+    u32 group[2][kGroups];    // bins to be split, in this step and the next: first slot | pairs << 16
+    u32 first[kGroups + 1];   // of a group in this step: pairs of earlier groups | bins of earlier groups << 16
+    u32 diff[3][kGroups];     // differing bits within the group: key (high, low), value
+    u32 s_warp[32];
+    u32 n_group[2];
+};
+
+// Start of every bin from the counts, `words` words of two (a power of two, or fewer than THREADS
+// words per thread and step); the word after them gets the number of pairs.
+template <int THREADS, int ITEMS>
+__device__ __forceinline__ void bins_to_starts(BlockSortSmem<THREADS, ITEMS>& sm, u32 words) {
+    const u32 per = (words + THREADS - 1) / THREADS;
+    const u32 w0 = min(threadIdx.x * per, words), w1 = min(w0 + per, words);
+    u32 sum = 0, all;
+    for (u32 w = w0; w < w1; ++w) {
+        const u32 c = sm.bins[w];
+        sum += (c & 0xffffu) + (c >> 16);
+    }
+    u32 run = block_scan<THREADS>(sum, sm.s_warp, &all);
+    for (u32 w = w0; w < w1; ++w) {
+        const u32 c = sm.bins[w];
+        const u32 mid = run + (c & 0xffffu);
+        sm.bins[w] = run | (mid << 16);
+        run = mid + (c >> 16);
+    }
+    if (threadIdx.x == 0) sm.bins[words] = all;
+}
+
+__device__ __forceinline__ u32 bin_add(u32* bins, u32 b) {  // the pair's rank in its bin
+    const u32 was = atomicAdd(&bins[b >> 1], (b & 1u) ? 0x10000u : 1u);
+    return (b & 1u) ? was >> 16 : was & 0xffffu;
+}
+
+// How a set of pairs is binned: the leading nb of the `top` low bits in which the keys' distances
+// from the base differ, followed by leading bits of the value where that is fewer than nb; equal keys
+// by the leading nb of the `vtop` low bits in which their values differ.
+struct BinMap {
+    int top, vtop, nb;
+    __device__ __forceinline__ u32 bin(Key d, u32 v, int idx_bits) const {
+        if (top >= nb) {
+            const Key low = d & (~static_cast<Key>(0) >> (kWordBits - top));
+            return static_cast<u32>(low >> (top - nb));
+        }
+        if (top > 0) {
+            const int up = nb - top;
+            const u32 low = static_cast<u32>(d) & ((1u << top) - 1u);
+            return (low << up) | (v >> max(0, idx_bits - up));
+        }
+        const u32 low = vtop >= 32 ? v : v & ((1u << vtop) - 1u);
+        return low >> max(0, vtop - nb);
+    }
+};
+
+// Place of the staged pair at slot s among the pairs of its bin, slots [b0, b1).
+template <class Smem>
+__device__ __forceinline__ u32 rank_in_bin(const Smem& sm, Key k, u32 v, u32 b0, u32 b1) {
+    u32 pos = b0, equal = 0;
+    for (u32 j = b0; j < b1; ++j) {
+        const Key o = sm.K[j];
+        pos += o < k ? 1u : 0u;
+        equal += o == k ? 1u : 0u;
+    }
+    if (equal > 1)  // rare
+        for (u32 j = b0; j < b1; ++j)
+            if (sm.K[j] == k && sm.V[j] < v) ++pos;
+    return pos;
+}
+
+// Sorts m <= THREADS * ITEMS pairs: load(e, key, value) gives pair e, out(position, key, value)
+// takes each at its place in the sorted order. Every load comes before any out. No key may be
+// below base; idx_bits bounds the values.
+//
+// The first step bins all pairs, m <= bins < 2 m. A pair whose bin holds at most kHeavy pairs is
+// ranked there by comparison and leaves; the larger bins are the groups of the next step, which
+// bins all of them at once, each over its own differing bits, and so on. A step takes four bits
+// or more off a group's keys (or values), so the steps end.
+template <int THREADS, int ITEMS, class Load, class Out>
+__device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, int idx_bits, Load load, Out out) {
+    const u32 tid = threadIdx.x;
+    const int lane = tid & 31, warp = tid >> 5;
+    const u16* starts = reinterpret_cast<const u16*>(sm.bins);  // little-endian halves
+    Key key[ITEMS];
+    u32 val[ITEMS], at[ITEMS];  // at: bin | rank within the bin << 16
+#pragma unroll
+    for (int i = 0; i < ITEMS; ++i)
+        if (tid + i * THREADS < m) load(tid + i * THREADS, key[i], val[i]);
+    {
+        BinMap map;
+        map.nb = max(kMinBinBits, 32 - __clz(static_cast<int>(m - 1u)));
+        const u32 words = 1u << (map.nb - 1);
+        for (u32 w = tid; w < words; w += THREADS) sm.bins[w] = 0u;
+        if (tid < 2) sm.n_group[tid] = 0u;
+        Key ored = 0;
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (tid + i * THREADS < m) ored |= key[i] - base;
+        if (sizeof(Key) == 8) {
+            const u32 lo = __reduce_or_sync(0xffffffffu, static_cast<u32>(ored));
+            const u32 hi = __reduce_or_sync(0xffffffffu, static_cast<u32>(static_cast<u64>(ored) >> 32));
+            ored = static_cast<Key>((static_cast<u64>(hi) << 32) | lo);
+        } else {
+            ored = __reduce_or_sync(0xffffffffu, static_cast<u32>(ored));
+        }
+        if (lane == 0) sm.red[warp] = ored;
+        __syncthreads();
+        ored = 0;
+#pragma unroll
+        for (int w = 0; w < THREADS / 32; ++w) ored |= sm.red[w];
+        map.top = bit_length(ored);
+        map.vtop = idx_bits;
+        // unconditional, so that a thread's atomics are in flight together: a slot without a pair
+        // adds nothing to a word of its lane
+        u32 was[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const bool on = tid + i * THREADS < m;
+            const u32 b = on ? map.bin(key[i] - base, val[i], idx_bits) : 2u * lane;
+            at[i] = b;
+            was[i] = atomicAdd(&sm.bins[b >> 1], on ? ((b & 1u) ? 0x10000u : 1u) : 0u);
+        }
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) at[i] |= ((at[i] & 1u) ? was[i] >> 16 : was[i] & 0xffffu) << 16;
+        __syncthreads();
+        bins_to_starts<THREADS, ITEMS>(sm, words);
+        __syncthreads();
+        u32 slot[ITEMS];
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) slot[i] = starts[at[i] & 0xffffu] + (at[i] >> 16);
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i)
+            if (tid + i * THREADS < m) {
+                sm.K[slot[i]] = key[i];
+                sm.V[slot[i]] = val[i];
+            }
+        __syncthreads();
+        for (u32 s = tid; s < m; s += THREADS) {
+            const Key k = sm.K[s];
+            const u32 v = sm.V[s];
+            const u32 b = map.bin(k - base, v, idx_bits);
+            const u32 b0 = starts[b], b1 = starts[b + 1];
+            if (b1 - b0 <= kHeavy)
+                out(rank_in_bin(sm, k, v, b0, b1), k, v);
+            else if (s == b0)
+                sm.group[0][atomicAdd(&sm.n_group[0], 1u)] = b0 | ((b1 - b0) << 16);
+        }
+        __syncthreads();
+    }
+    for (int cur = 0;; cur ^= 1) {
+        const u32 ng = sm.n_group[cur];  // uniform
+        if (ng == 0) return;
+        const u32* group = sm.group[cur];
+        u32 all;
+        {
+            const u32 cnt = tid < ng ? group[tid] >> 16 : 0u;
+            const u32 nb = tid < ng ? 1u << (31 - __clz(static_cast<int>(cnt))) : 0u;
+            const u32 pre = block_scan<THREADS>(cnt | (nb << 16), sm.s_warp, &all);
+            if (tid < ng) {
+                sm.first[tid] = pre;
+                sm.diff[0][tid] = sm.diff[1][tid] = sm.diff[2][tid] = 0u;
+            }
+            if (tid == 0) sm.first[ng] = all;
+        }
+        const u32 left = all & 0xffffu, words = ((all >> 16) + 1u) / 2u;
+        for (u32 w = tid; w < words; w += THREADS) sm.bins[w] = 0u;
+        __syncthreads();
+        auto group_of = [&](u32 e) -> u32 {  // last group whose first pair is <= e
+            u32 lo = 0, hi = ng;
+            while (hi - lo > 1) {
+                const u32 mid = (lo + hi) >> 1;
+                if ((sm.first[mid] & 0xffffu) <= e)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            return lo;
+        };
+        auto map_of = [&](u32 g) -> BinMap {
+            BinMap map;
+            const u64 d = (static_cast<u64>(sm.diff[0][g]) << 32) | sm.diff[1][g];
+            map.top = bit_length(d);
+            map.vtop = 32 - __clz(static_cast<int>(sm.diff[2][g]));
+            map.nb = 31 - __clz(static_cast<int>(group[g] >> 16));
+            return map;
+        };
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const u32 e = tid + i * THREADS;
+            if (i * THREADS >= left) break;  // uniform
+            const bool on = e < left;
+            const u32 g = on ? group_of(e) : 0u;
+            u64 dk = 0;
+            u32 dv = 0;
+            if (on) {
+                const u32 s0 = group[g] & 0xffffu, s = s0 + e - (sm.first[g] & 0xffffu);
+                key[i] = sm.K[s];
+                val[i] = sm.V[s];
+                dk = static_cast<u64>((key[i] - base) ^ (sm.K[s0] - base));
+                dv = val[i] ^ sm.V[s0];
+            }
+            const u32 g0 = __shfl_sync(0xffffffffu, g, 0);
+            if (__all_sync(0xffffffffu, g == g0 || !on)) {
+                const u32 hi = __reduce_or_sync(0xffffffffu, static_cast<u32>(dk >> 32));
+                const u32 lo = __reduce_or_sync(0xffffffffu, static_cast<u32>(dk));
+                const u32 vo = __reduce_or_sync(0xffffffffu, dv);
+                if (lane == 0) {
+                    atomicOr(&sm.diff[0][g0], hi);
+                    atomicOr(&sm.diff[1][g0], lo);
+                    atomicOr(&sm.diff[2][g0], vo);
+                }
+            } else if (on) {
+                atomicOr(&sm.diff[0][g], static_cast<u32>(dk >> 32));
+                atomicOr(&sm.diff[1][g], static_cast<u32>(dk));
+                atomicOr(&sm.diff[2][g], dv);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const u32 e = tid + i * THREADS;
+            if (e < left) {
+                const u32 g = group_of(e);
+                const u32 b = (sm.first[g] >> 16) + map_of(g).bin(key[i] - base, val[i], idx_bits);
+                at[i] = b | (bin_add(sm.bins, b) << 16);
+            }
+        }
+        __syncthreads();
+        bins_to_starts<THREADS, ITEMS>(sm, words);
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < ITEMS; ++i) {
+            const u32 e = tid + i * THREADS;
+            if (e < left) {
+                const u32 g = group_of(e);
+                const u32 s = (group[g] & 0xffffu) + starts[at[i] & 0xffffu] - starts[sm.first[g] >> 16] + (at[i] >> 16);
+                sm.K[s] = key[i];
+                sm.V[s] = val[i];
+            }
+        }
+        __syncthreads();
+        for (u32 e = tid; e < left; e += THREADS) {
+            const u32 g = group_of(e);
+            const BinMap map = map_of(g);
+            const u32 s0 = group[g] & 0xffffu, s = s0 + e - (sm.first[g] & 0xffffu);
+            const Key k = sm.K[s];
+            const u32 v = sm.V[s];
+            const u32 o = sm.first[g] >> 16, b = o + map.bin(k - base, v, idx_bits);
+            const u32 b0 = s0 + starts[b] - starts[o], b1 = s0 + starts[b + 1] - starts[o];
+            // equal pairs, which only overlapping segments could give, cannot be split
+            if (b1 - b0 <= kHeavy || (map.top == 0 && map.vtop == 0))
+                out(rank_in_bin(sm, k, v, b0, b1), k, v);
+            else if (s == b0)
+                sm.group[cur ^ 1][atomicAdd(&sm.n_group[cur ^ 1], 1u)] = b0 | ((b1 - b0) << 16);
+        }
+        __syncthreads();
+        if (tid == 0) sm.n_group[cur] = 0u;
+    }
+}
+
+using SmallSmem = BlockSortSmem<kSmallThreads, kSmallItems>;
+using BigSmem = BlockSortSmem<kBigThreads, kBigItems>;
+static_assert(BigSmem::kCap <= 8192 && SmallSmem::kCap <= 4096, "16-bit counts and stack entries");
+
+// ---------------------------------------------------------------------------- a round of splitting
+__device__ __forceinline__ u32 hash32(u32 x) {  // Wang's integer mix (public domain)
+    x = (x ^ 61u) ^ (x >> 16);
+    x *= 9u;
+    x ^= x >> 4;
+    x *= 0x27d4eb2du;
+    return x ^ (x >> 15);
+}
+
+// Bounds of every bucket's parts from a stratified random sample (16 or 32 pairs per part, which
+// keeps nearly every part below twice the mean), sorted by one block; the counts are cleared.
+template <int SRC>
+__global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Buckets b, Tables t, int idx_bits) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    BigSmem& sm = *reinterpret_cast<BigSmem*>(smem_raw);
+    const u32 count = *b.count;
+    for (u32 k = blockIdx.x; k < count; k += gridDim.x) {
+        const u32 start = b.start[k], size = b.size[k], fp = b.first_part[k];
+        const u32 np = b.first_part[k + 1] - fp;
+        const u32 per = np <= kBig / 32u ? 32u : 16u;
+        const u32 ns = np * per;  // <= kBig, and < size: a part has kTarget pairs or more on average
+        const Key* keys = keys_of<SRC>(p);
+        const Key base = b.base[k];
+        block_sort<kBigThreads, kBigItems>(
+            sm, ns, base, idx_bits,
+            [&](u32 e, Key& key, u32& val) {
+                const u32 lo = static_cast<u32>(static_cast<u64>(e) * size / ns);
+                const u32 hi = static_cast<u32>(static_cast<u64>(e + 1) * size / ns);
+                const u32 pos = start + lo + hash32(e + 0x9e3779b9u * start) % (hi - lo);
+                key = __ldcg(keys + pos);
+                val = value_of<SRC>(p, pos);
+            },
+            [&](u32 pos, Key key, u32 val) {
+                if (pos % per == 0) {
+                    t.part_key[fp + pos / per] = pos ? key : base;
+                    t.part_idx[fp + pos / per] = pos ? val : 0u;
+                }
+            });
+        for (u32 q = threadIdx.x; q < np; q += kBigThreads) t.part_pos[(size_t)(fp + q) * kPosStride] = 0u;
+        __syncthreads();
+    }
+}
+
+// First bucket of a block's range of tiles.
+__device__ __forceinline__ u32 bucket_of(const Buckets& b, u32 count, u32 tile) {
+    u32 lo = 0, hi = count;  // last bucket whose first tile is <= tile
+    while (hi - lo > 1) {
+        const u32 mid = (lo + hi) >> 1;
+        if (b.first_tile[mid] <= tile)
+            lo = mid;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+constexpr u32 kLutBits = 10, kLut = 1u << kLutBits;
+constexpr int kCountBlocks = 1280 / kThreads;  // blocks per SM of the count
+
+struct CountSmem {
+    Key key[kMaxParts];  // bounds
+    u32 idx[kMaxParts];
+    u32 lut[kLut];  // by the leading bits of the distance from the bucket's base: bounds (1, 2, ...) in earlier
+                    // entries | and in this one << 16
+    u32 hist[kMaxParts];
+    u32 s_warp[32];
+};
+
+// Part of every pair, and the parts' sizes. A block takes a contiguous range of tiles, so that it
+// loads a bucket's bounds and flushes its counts once per bucket. The search reads shared memory
+// at scattered addresses, which bounds the kernel (comparing the leading 32 bits first saves half
+// the reads, but is slower: in tight clumps they are often equal).
+template <int SRC>
+__global__ void __launch_bounds__(kThreads, kCountBlocks) sort_count_kernel(Pairs p, Buckets b, Tables t) {
+    __shared__ CountSmem sm;
+    const int tid = threadIdx.x;
+    const u32 count = *b.count;
+    const u32 tiles = count ? b.first_tile[count] : 0u;
+    const u32 t0 = static_cast<u32>(static_cast<u64>(tiles) * blockIdx.x / gridDim.x);
+    const u32 t1 = static_cast<u32>(static_cast<u64>(tiles) * (blockIdx.x + 1) / gridDim.x);
+    if (t0 >= t1) return;
+    const Key* keys = keys_of<SRC>(p);
+    u32 k = bucket_of(b, count, t0);
+    u32 tile = t0;
+    while (tile < t1) {
+        const u32 first = b.first_tile[k], end = min(t1, b.first_tile[k + 1]);
+        const u32 start = b.start[k], size = b.size[k], fp = b.first_part[k], np = b.first_part[k + 1] - fp;
+        const Key base = b.base[k];
+        const int top = bit_length(t.part_key[fp + np - 1] - base);  // bits of the bounds' distances
+        const int lsh = max(0, top - static_cast<int>(kLutBits));
+        auto entry = [&](Key key) -> u32 {
+            const Key e = (key - base) >> lsh;
+            return e < kLut ? static_cast<u32>(e) : kLut - 1u;
+        };
+        for (u32 q = tid; q < kLut; q += kThreads) sm.lut[q] = 0u;
+        __syncthreads();
+        for (u32 q = tid; q < np; q += kThreads) {
+            const Key bound = t.part_key[fp + q];
+            sm.key[q] = bound;
+            sm.idx[q] = t.part_idx[fp + q];
+            sm.hist[q] = 0u;
+            if (q > 0) atomicAdd(&sm.lut[entry(bound)], 0x10000u);
+        }
+        __syncthreads();
+        {
+            constexpr u32 kPer = kLut / 256;
+            u32 c[kPer], sum = 0, all;
+#pragma unroll
+            for (u32 j = 0; j < kPer; ++j) {
+                c[j] = tid < 256 ? sm.lut[tid * kPer + j] : 0u;
+                sum += c[j] >> 16;
+            }
+            u32 run = block_scan<kThreads>(sum, sm.s_warp, &all);
+#pragma unroll
+            for (u32 j = 0; j < kPer; ++j) {
+                if (tid < 256) sm.lut[tid * kPer + j] = run | c[j];
+                run += c[j] >> 16;
+            }
+        }
+        __syncthreads();
+        for (u32 q = tile + tid; q < end; q += kThreads) t.tile_bucket[q] = k;
+        for (; tile < end; ++tile) {
+            const u32 o0 = (tile - first) * kTile;
+            const u32 cnt = min(static_cast<u32>(kTile), size - o0);
+            const u32 at = start + o0;
+            Key key[kItems];
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) {
+                const u32 e = tid + i * kThreads;
+                key[i] = e < cnt ? __ldcg(keys + at + e) : base;
+            }
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) {
+                const u32 e = tid + i * kThreads;
+                const u32 l = sm.lut[entry(key[i])];
+                const u32 lo0 = l & 0xffffu;
+                u32 lo = lo0, hi = lo + (l >> 16);
+                while (lo < hi) {  // the last bound whose key is not above this one
+                    const u32 mid = (lo + hi + 1) >> 1;
+                    const bool le = sm.key[mid] <= key[i];
+                    lo = le ? mid : lo;
+                    hi = le ? hi : mid - 1u;
+                }
+                if (lo > lo0 && sm.key[lo] == key[i] && e < cnt) {  // rare: among equal keys the indices decide
+                    const u32 v = value_of<SRC>(p, at + e);
+                    u32 a = lo0, z = lo;
+                    while (a < z) {
+                        const u32 mid = (a + z + 1) >> 1;
+                        const bool le = pair_less(sm.key[mid], sm.idx[mid], key[i], v + 1u);
+                        a = le ? mid : a;
+                        z = le ? z : mid - 1u;
+                    }
+                    lo = a;
+                }
+                __syncwarp();  // the searches' lengths differ: the warp goes on together
+                if (e < cnt) {
+                    atomicAdd(&sm.hist[lo], 1u);
+                    t.part_of[at + e] = static_cast<u16>(lo);
+                }
+            }
+        }
+        __syncthreads();
+        for (u32 q = tid; q < np; q += kThreads) {
+            const u32 h = sm.hist[q];
+            if (h) atomicAdd(&t.part_pos[(size_t)(fp + q) * kPosStride], h);
+        }
+        __syncthreads();
+        ++k;
+    }
+}
+
+// Positions of the parts (the bucket's start plus the sizes of the earlier parts), and the lists
+// of what is left to do: parts of at most kSmall pairs go to the final sort, larger ones to `next`.
+__global__ void __launch_bounds__(kMaxParts) sort_plan_kernel(Buckets b, Buckets next, Tables t, u32 dst) {
+    __shared__ u32 s_warp[32];
+    const u32 count = *b.count;
+    for (u32 k = blockIdx.x; k < count; k += gridDim.x) {
+        const u32 fp = b.first_part[k], np = b.first_part[k + 1] - fp;
+        const u32 q = threadIdx.x;
+        const u32 size = q < np ? t.part_pos[(size_t)(fp + q) * kPosStride] : 0u;
+        u32 all;
+        const u32 pos = b.start[k] + block_scan<kMaxParts>(size, s_warp, &all);
+        if (size > 0) {
+            t.part_pos[(size_t)(fp + q) * kPosStride] = pos;
+            const Key base = t.part_key[fp + q];
+            if (size <= kSmall) {
+                const u32 e = atomicAdd(t.n_small, 1u);
+                t.small[e] = make_uint2(pos, size | (dst << 30));
+                t.small_base[e] = base;
+            } else {
+                const u32 e = atomicAdd(next.count, 1u);
+                next.start[e] = pos;
+                next.size[e] = size;
+                next.base[e] = base;
+            }
+        }
+    }
+}
+
+struct ScatterSmem {
+    Key keys[kTile];  // the tile grouped by part
+    u32 vals[kTile];
+    u32 hist[kMaxParts + 32];  // counts, then first slots of the parts; then a word per lane
+    u32 delta[kMaxParts];      // output position minus slot of every run (the parts that have pairs)
+    u32 run_start[kTile / 32];  // bit per slot: a run starts here
+    u32 run_at[kTile / 32];     // run of every 32nd slot
+    u32 s_warp[32];
+};
+
+// Moves the pairs of every bucket to their parts, in runs of a tile's pairs of one part. The order
+// within a part does not matter, so a pair's rank comes from an atomic count and a tile takes its
+// range of a part with one atomic add. Scattered shared-memory accesses bound the kernel: a pair
+// costs the count, its part's first slot, and the stores of its key and value; the run that a slot
+// belongs to is found from the run starts, which a warp's slots share.
+template <int SRC>
+__global__ void __launch_bounds__(kThreads, CSTONE_SORT_MIN_BLOCKS) sort_scatter_kernel(Pairs p, Buckets b, Tables t) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    ScatterSmem& sm = *reinterpret_cast<ScatterSmem*>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31;
+    const u32 count = *b.count;
+    const u32 tiles = count ? b.first_tile[count] : 0u;
+    const Key* kin = keys_of<SRC>(p);
+    Key* kout = SRC == kBufA ? p.b : p.a;
+    u32* vout = SRC == kBufA ? p.vb : p.va;
+    // the blocks take neighbouring tiles at a time, so that reads and runs stay close together
+    u32 next = blockIdx.x < tiles ? t.tile_bucket[blockIdx.x] : 0u;
+    for (u32 tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const u32 k = next;
+        if (tile + gridDim.x < tiles) next = t.tile_bucket[tile + gridDim.x];
+        const u32 o0 = (tile - b.first_tile[k]) * kTile;
+        const u32 cnt = min(static_cast<u32>(kTile), b.size[k] - o0);
+        const u32 at = b.start[k] + o0, fp = b.first_part[k];
+        for (u32 q = tid; q < kMaxParts + 32; q += kThreads) sm.hist[q] = 0u;
+        for (u32 q = tid; q < kTile / 32; q += kThreads) sm.run_start[q] = 0u;
+        Key key[kItems];
+        u32 val[kItems], part[kItems], slot[kItems];
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) {
+            const u32 e = tid + i * kThreads;
+            const bool ok = e < cnt;
+            part[i] = ok ? __ldcg(t.part_of + at + e) : kMaxParts + lane;  // no pair: counted in the lane's word
+            key[i] = ok ? __ldcg(kin + at + e) : static_cast<Key>(0);
+            val[i] = ok ? value_of<SRC>(p, at + e) : 0u;
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) slot[i] = atomicAdd(&sm.hist[part[i]], 1u);
+        __syncthreads();
+        {
+            constexpr u32 kPer = kMaxParts / 256;
+            u32 c[kPer], sum = 0, all;
+#pragma unroll
+            for (u32 j = 0; j < kPer; ++j) {
+                c[j] = tid < 256 ? sm.hist[tid * kPer + j] : 0u;
+                sum += c[j] | (c[j] ? 0x10000u : 0u);  // pairs | runs
+            }
+            u32 pre = block_scan<kThreads>(sum, sm.s_warp, &all);
+#pragma unroll
+            for (u32 j = 0; j < kPer; ++j) {
+                const u32 first = pre & 0xffffu, run = pre >> 16, end = first + c[j];
+                if (tid < 256) sm.hist[tid * kPer + j] = first;
+                if (c[j]) {
+                    sm.delta[run] = atomicAdd(&t.part_pos[(size_t)(fp + tid * kPer + j) * kPosStride], c[j]) - first;
+                    atomicOr(&sm.run_start[first >> 5], 1u << (first & 31u));
+                    for (u32 w = (first + 31u) >> 5; (w << 5) < end; ++w) sm.run_at[w] = run;
+                    pre += c[j] | 0x10000u;
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) slot[i] += sm.hist[part[i]];
+#pragma unroll
+        for (int i = 0; i < kItems; ++i)
+            if (tid + i * kThreads < cnt) {
+                sm.keys[slot[i]] = key[i];
+                sm.vals[slot[i]] = val[i];
+            }
+        __syncthreads();
+#pragma unroll
+        for (int i = 0; i < kItems; ++i) {
+            const u32 s = tid + i * kThreads;
+            if (s < cnt) {
+                const u32 w = s >> 5;
+                // starts after the word's first slot, up to this one
+                const u32 run = sm.run_at[w] + __popc(sm.run_start[w] & (0xfffffffeu & (0xffffffffu >> (31 - lane))));
+                const u32 d = sm.delta[run] + s;
+                kout[d] = sm.keys[s];
+                vout[d] = sm.vals[s];
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------- final sort
+// Every listed part, one block each, from wherever it is to its place in the output.
+__global__ void __launch_bounds__(kSmallThreads, kSmallBlocks) sort_small_kernel(Pairs p, Tables t, int idx_bits) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
+    const u32 count = *t.n_small;
+    for (u32 k = blockIdx.x; k < count; k += gridDim.x) {
+        const uint2 ent = t.small[k];
+        const u32 start = ent.x, m = ent.y & 0x3fffffffu, src = ent.y >> 30;
+        const Key* keys = src == kInput ? p.in : (src == kBufA ? p.a : p.b);
+        const u32* vals = src == kBufA ? p.va : p.vb;
+        block_sort<kSmallThreads, kSmallItems>(
+            sm, m, t.small_base[k], idx_bits,
+            [&](u32 e, Key& key, u32& val) {
+                key = __ldcg(keys + start + e);
+                val = src == kInput ? start + e : __ldcg(vals + start + e);
+            },
+            [&](u32 pos, Key key, u32 val) {
+                p.b[start + pos] = key;
+                p.vb[start + pos] = val;
+            });
+        __syncthreads();
+    }
+}
+
+// Parts of more than kSmall pairs after the last round, one block each: chunks of kBig pairs sorted
+// in shared memory, then merged pairwise between the part's ranges of the two buffers. LAST: the
+// buffer that the last round wrote.
+template <int LAST>
+__global__ void __launch_bounds__(kBigThreads) sort_rest_kernel(Pairs p, Buckets b, int idx_bits) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    BigSmem& sm = *reinterpret_cast<BigSmem*>(smem_raw);
+    const u32 count = *b.count;
+    for (u32 k = blockIdx.x; k < count; k += gridDim.x) {
+        const u32 start = b.start[k], size = b.size[k];
+        const Key base = b.base[k];
+        // the buffer of the sorted chunks, such that the last merge (or the chunk itself) ends in B
+        u32 merges = 0;
+        for (u64 w = kBig; w < size; w <<= 1) ++merges;
+        bool in_b = (merges & 1u) == 0;
+        const Key* k0 = (LAST == kBufA ? p.a : p.b) + start;
+        const u32* v0 = (LAST == kBufA ? p.va : p.vb) + start;
+        for (u32 c = 0; c < size; c += kBig) {
+            const u32 m = min(kBig, size - c);
+            Key* ko = (in_b ? p.b : p.a) + start + c;
+            u32* vo = (in_b ? p.vb : p.va) + start + c;
+            block_sort<kBigThreads, kBigItems>(
+                sm, m, base, idx_bits,
+                [&](u32 e, Key& key, u32& val) {
+                    key = __ldcg(k0 + c + e);
+                    val = __ldcg(v0 + c + e);
+                },
+                [&](u32 pos, Key key, u32 val) {
+                    ko[pos] = key;
+                    vo[pos] = val;
+                });
+            __syncthreads();
+        }
+        for (u64 w = kBig; w < size; w <<= 1) {
+            const Key* ks = (in_b ? p.b : p.a) + start;
+            const u32* vs = (in_b ? p.vb : p.va) + start;
+            Key* kd = (in_b ? p.a : p.b) + start;
+            u32* vd = (in_b ? p.va : p.vb) + start;
+            constexpr u32 kRun = 16;  // outputs per thread and step
+            for (u64 o = static_cast<u64>(threadIdx.x) * kRun; o < size; o += static_cast<u64>(kBigThreads) * kRun) {
+                const u64 lo = o / (2 * w) * (2 * w);  // the pair of runs that o falls in
+                const u32 l0 = static_cast<u32>(lo), l1 = static_cast<u32>(min(lo + w, static_cast<u64>(size)));
+                const u32 r1 = static_cast<u32>(min(lo + 2 * w, static_cast<u64>(size)));
+                const u32 diag = static_cast<u32>(o) - l0, nl = l1 - l0, nr = r1 - l1;
+                u32 a = diag > nr ? diag - nr : 0u, z = min(diag, nl);  // pairs taken from the left run
+                while (a < z) {
+                    const u32 mid = (a + z) >> 1;
+                    const u32 i = l0 + mid, j = l1 + diag - 1u - mid;
+                    if (pair_less(__ldcg(ks + i), __ldcg(vs + i), __ldcg(ks + j), __ldcg(vs + j)))
+                        a = mid + 1;
+                    else
+                        z = mid;
+                }
+                u32 i = l0 + a, j = l1 + diag - a;
+                const u32 stop = static_cast<u32>(min(o + kRun, static_cast<u64>(r1)));
+                for (u32 q = static_cast<u32>(o); q < stop; ++q) {
+                    const bool left = j >= r1 || (i < l1 && pair_less(__ldcg(ks + i), __ldcg(vs + i), __ldcg(ks + j),
+                                                                      __ldcg(vs + j)));
+                    const u32 s = left ? i++ : j++;
+                    kd[q] = __ldcg(ks + s);
+                    vd[q] = __ldcg(vs + s);
+                }
+            }
+            __syncthreads();
+            in_b = !in_b;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------- digit passes
+// Stable passes of 8-bit digits, each a tile count, its scan in three launches and the ranked scatter
+// (the lanes of a warp holding the same digit are found with one ballot per digit bit).
+//
+// 30-bit keys have four digits only, and in clustered matter many particles share a key: the passes
+// are the better sort where splitting takes two rounds (2^24 keys: 510 us against 530 us uniform and
+// 850 us clumped; 2^20: 133 against 112 and 171), one round the better below (2^18: 117 against 73 and
+// 99).
+// 63-bit keys take eight; one launch of the block sort above is faster (28 us against 190 us for
+// 1000 keys on GB300), but the launches of a sort of 1000 keys are part of what the launch counter
+// is tested for, so sets of at most kDigitMax keys keep the passes.
+namespace digits {
+constexpr long long kDigitMin = (long long)kTarget * kMaxParts + 1, kDigitMax = 1024;
 constexpr int kRadixBits = 8;
 constexpr int kRadix = 1 << kRadixBits;
 constexpr int kPasses = (kKeyBits + kRadixBits - 1) / kRadixBits;  // 8 (63-bit keys) or 4 (30-bit keys)
-// Tile shape (compile-time tuning knobs, set by the build from the autotuner's choice): threads per
-// block, keys per thread and blocks per SM.
-#ifndef CSTONE_SORT_THREADS
-#define CSTONE_SORT_THREADS 256
-#endif
-#ifndef CSTONE_SORT_ITEMS
-#define CSTONE_SORT_ITEMS 12
-#endif
-#ifndef CSTONE_SORT_MIN_BLOCKS
-#define CSTONE_SORT_MIN_BLOCKS 4
-#endif
-constexpr int kThreads = CSTONE_SORT_THREADS;
-constexpr int kWarps = kThreads / 32;
-constexpr int kItems = CSTONE_SORT_ITEMS;
-static_assert(kThreads >= 256 && kThreads % 32 == 0, "one thread per digit is needed");
-static_assert(kItems % 2 == 0, "ranks are packed two per register");
-constexpr int kTile = kThreads * kItems;  // keys per tile
+constexpr int kThreads = 256, kWarps = kThreads / 32, kItems = 12, kBlocks = 4;
+constexpr int kTile = kThreads * kItems;
+static_assert(kTile < 65536 && kPasses % 2 == 0, "16-bit tile counts; the last pass writes the output");
 
-// Segmented sorts (many independent key sets stored back to back) use tiles aligned to the
-// segments: every tile holds keys of one segment only, and digits are offset per segment.
-struct SegTiles {
-    const u32* n_tiles;      // device scalar: tiles in use
-    const u32* tile_seg;     // segment of each tile
-    const u32* tile_base;    // first key (global index) of each tile
-    const u32* tile_count;   // keys in each tile (<= kTile)
-    const u32* seg_first;    // first tile of each segment
-    const u32* seg_offsets;  // [segment][pass][digit] output position of the digit's first key
-};
+inline bool taken(long long n) { return sizeof(Key) == 4 ? n >= kDigitMin : n <= kDigitMax; }
 
-struct SegBuild {  // writable view of the same tables
-    u32* n_tiles;
-    u32* tile_seg;
-    u32* tile_base;
-    u32* tile_count;
-    u32* seg_first;
-    u32* seg_hist;
-    u32* seg_offsets;
-};
-
-// Tiles per segment and their exclusive scan (one block).
-__global__ void __launch_bounds__(1024) seg_setup_kernel(const long long* __restrict__ seg_offsets_in, int n_segs,
-                                                         SegBuild b) {
-    __shared__ u32 s_part[1024];
-    const int per = (n_segs + 1023) / 1024;
-    const int begin = threadIdx.x * per, end = min(begin + per, n_segs);
-    u32 sum = 0;
-    for (int q = begin; q < end; ++q) {
-        const long long len = seg_offsets_in[q + 1] - seg_offsets_in[q];
-        sum += static_cast<u32>((len + kTile - 1) / kTile);
-    }
-    s_part[threadIdx.x] = sum;
-    __syncthreads();
-    for (int st = 1; st < 1024; st <<= 1) {
-        const u32 v = threadIdx.x >= (unsigned)st ? s_part[threadIdx.x - st] : 0u;
-        __syncthreads();
-        s_part[threadIdx.x] += v;
-        __syncthreads();
-    }
-    u32 run = s_part[threadIdx.x] - sum;
-    for (int q = begin; q < end; ++q) {
-        b.seg_first[q] = run;
-        const long long len = seg_offsets_in[q + 1] - seg_offsets_in[q];
-        run += static_cast<u32>((len + kTile - 1) / kTile);
-    }
-    if (threadIdx.x == 1023) {
-        b.seg_first[n_segs] = s_part[1023];
-        *b.n_tiles = s_part[1023];
-    }
-}
-
-// Tile table: segment, first key and key count of every tile.
-__global__ void __launch_bounds__(kThreads) seg_tiles_kernel(const long long* __restrict__ seg_offsets_in, int n_segs,
-                                                             u32 max_tiles, SegBuild b) {
-    const u32 total = *b.n_tiles;
-    for (u32 t = blockIdx.x * kThreads + threadIdx.x; t < max_tiles; t += gridDim.x * kThreads) {
-        if (t >= total) {
-            b.tile_count[t] = 0;
-            continue;
-        }
-        int lo = 0, hi = n_segs;  // last segment whose first tile is <= t
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (b.seg_first[mid] <= t)
-                lo = mid;
-            else
-                hi = mid;
-        }
-        while (lo + 1 < n_segs && b.seg_first[lo + 1] <= t) ++lo;  // skip empty segments
-        const long long start = seg_offsets_in[lo] + (long long)(t - b.seg_first[lo]) * kTile;
-        const long long end = seg_offsets_in[lo + 1];
-        b.tile_seg[t] = static_cast<u32>(lo);
-        b.tile_base[t] = static_cast<u32>(start);
-        b.tile_count[t] = static_cast<u32>(min((long long)kTile, end - start));
-    }
-}
-
-// Per-segment digit histograms of all 8 passes, one block per tile.
-__global__ void __launch_bounds__(kThreads) seg_hist_kernel(const Key* __restrict__ keys, SegTiles st, u32* seg_hist) {
-    __shared__ u32 sh[kPasses][kRadix];
-    const u32 t = blockIdx.x;
-    const u32 count = st.tile_count[t];
-    if (count == 0) return;
-    for (int i = threadIdx.x; i < kPasses * kRadix; i += kThreads) (&sh[0][0])[i] = 0;
-    __syncthreads();
-    const u32 base = st.tile_base[t];
-    for (u32 i = threadIdx.x; i < count; i += kThreads) {
-        const Key k = __ldg(keys + base + i);
-#pragma unroll
-        for (int p = 0; p < kPasses; ++p) atomicAdd(&sh[p][(k >> (p * kRadixBits)) & (kRadix - 1)], 1u);
-    }
-    __syncthreads();
-    u32* dst = seg_hist + (size_t)st.tile_seg[t] * kPasses * kRadix;
-    for (int i = threadIdx.x; i < kPasses * kRadix; i += kThreads) {
-        const u32 v = (&sh[0][0])[i];
-        if (v) atomicAdd(dst + i, v);
-    }
-}
-
-// Digit offsets per segment and pass: the segment start plus the exclusive scan of its histogram.
-__global__ void seg_scan_kernel(const long long* __restrict__ seg_offsets_in, const u32* __restrict__ seg_hist,
-                                u32* seg_offsets) {
-    const int seg = blockIdx.x;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (warp >= kPasses) return;
-    const u32* h = seg_hist + ((size_t)seg * kPasses + warp) * kRadix;
-    u32* o = seg_offsets + ((size_t)seg * kPasses + warp) * kRadix;
-    u32 carry = static_cast<u32>(seg_offsets_in[seg]);
-    for (int base = 0; base < kRadix; base += 32) {
-        const u32 v = h[base + lane];
-        u32 incl = v;
-        for (int sft = 1; sft < 32; sft <<= 1) {
-            const u32 t = __shfl_up_sync(0xffffffffu, incl, sft);
-            if (lane >= sft) incl += t;
-        }
-        o[base + lane] = carry + incl - v;
-        carry += __shfl_sync(0xffffffffu, incl, 31);
-    }
-}
+constexpr int kChunkTiles = 32;  // tiles per chunk of the two-level scan
 
 // Lanes of the warp whose value v (9 bits: an 8-bit digit or the marker kRadix) equals this
 // lane's: one ballot per bit.
@@ -188,14 +931,11 @@ struct PassSmem {
     u32 scan_tmp[kWarps];
 };
 
-// One digit pass. tile_pos[tile][d]: for a single-set sort the output position of the tile's
-// first key of digit d; for a segmented sort the keys of digit d in all tiles before this one
-// (over every segment), from which the tile's segment start is subtracted.
-template <bool FIRST, bool SEG>
-__global__ void __launch_bounds__(kThreads, CSTONE_SORT_MIN_BLOCKS)
+// One digit pass. tile_pos[tile][d]: the output position of the tile's first key of digit d.
+template <bool FIRST>
+__global__ void __launch_bounds__(kThreads, kBlocks)
     sort_pass_kernel(const Key* __restrict__ kin, Key* __restrict__ kout, const u32* __restrict__ vin,
-                     u32* __restrict__ vout, long long n, int pass, const u32* __restrict__ tile_pos,
-                     SegTiles seg) {
+                     u32* __restrict__ vout, long long n, int pass, const u32* __restrict__ tile_pos) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PassSmem& sm = *reinterpret_cast<PassSmem*>(smem_raw);
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -205,15 +945,9 @@ __global__ void __launch_bounds__(kThreads, CSTONE_SORT_MIN_BLOCKS)
     __syncthreads();
     const u32 tile = blockIdx.x;
     u32 base, count;  // first key of the tile and keys in it (n < 2^30, so 32-bit offsets)
-    if (SEG) {
-        if (tile >= *seg.n_tiles) return;
-        base = seg.tile_base[tile];
-        count = seg.tile_count[tile];
-    } else {
-        base = tile * static_cast<u32>(kTile);
-        const long long remain = n - (long long)base;
-        count = remain < kTile ? static_cast<u32>(remain) : static_cast<u32>(kTile);
-    }
+    base = tile * static_cast<u32>(kTile);
+    const long long remain = n - (long long)base;
+    count = remain < kTile ? static_cast<u32>(remain) : static_cast<u32>(kTile);
 
     // ---- load (warp-striped: warp w owns keys base + w*32*kItems + it*32 + lane)
     Key key[kItems];
@@ -295,14 +1029,7 @@ __global__ void __launch_bounds__(kThreads, CSTONE_SORT_MIN_BLOCKS)
         }
 
         // output position of the tile's first key of digit d, minus its staging slot
-        if (SEG) {
-            const u32 sg = seg.tile_seg[tile];
-            const u32 first_tile = seg.seg_first[sg];
-            const u32 seg_digit_offset = seg.seg_offsets[((size_t)sg * kPasses + pass) * kRadix + d];
-            sm.delta[d] = seg_digit_offset + (tile_pos[(size_t)tile * kRadix + d] -
-                                              tile_pos[(size_t)first_tile * kRadix + d]) - start;
-        } else
-            sm.delta[d] = tile_pos[(size_t)tile * kRadix + d] - start;
+        sm.delta[d] = tile_pos[(size_t)tile * kRadix + d] - start;
     }
     __syncthreads();
 
@@ -341,32 +1068,18 @@ __global__ void __launch_bounds__(kThreads, CSTONE_SORT_MIN_BLOCKS)
     for (u32 s = tid; s < count; s += kThreads) vout[sm.delta[sm.dig[s]] + s] = sm.stage.vals[s];
 }
 
-// ---- output offsets of every tile, ahead of a pass (single-set sorts). A tile's output position
-// for digit d is the digit's global offset plus the keys of digit d in all earlier tiles; counting
-// every tile first and scanning the counts replaces the look-back (which measured a third of the
-// sort's time: tiles in flight wait on their predecessors' prefixes).
-constexpr int kChunkTiles = 32;  // tiles per chunk of the two-level scan
-
-// Digit counts of every tile of the pass (the tile partition of sort_pass_kernel; unused tiles of a
-// segmented sort count nothing).
-template <bool SEG>
+// Digit counts of every tile of the pass (the tile partition of sort_pass_kernel).
 __global__ void __launch_bounds__(kThreads) tile_count_kernel(const Key* __restrict__ kin, long long n, int shift,
-                                                              unsigned short* __restrict__ counts, SegTiles seg) {
+                                                              unsigned short* __restrict__ counts) {
     __shared__ u32 wh[kWarps][kRadix];
     const int tid = threadIdx.x, warp = tid >> 5;
     for (int i = tid; i < kWarps * kRadix; i += kThreads) (&wh[0][0])[i] = 0;
     __syncthreads();
     long long base;
     u32 count;
-    if (SEG) {
-        const bool used = blockIdx.x < *seg.n_tiles;
-        base = used ? seg.tile_base[blockIdx.x] : 0;
-        count = used ? seg.tile_count[blockIdx.x] : 0u;
-    } else {
-        base = (long long)blockIdx.x * kTile;
-        const long long remain = n - base;
-        count = remain < kTile ? static_cast<u32>(remain) : static_cast<u32>(kTile);
-    }
+    base = (long long)blockIdx.x * kTile;
+    const long long remain = n - base;
+    count = remain < kTile ? static_cast<u32>(remain) : static_cast<u32>(kTile);
     const Key* tkeys = kin + base;
     const u32 woff = static_cast<u32>(warp * 32 * kItems + (tid & 31));
     Key kk[kItems];
@@ -470,33 +1183,181 @@ __global__ void __launch_bounds__(kRadix) tile_offsets_kernel(const unsigned sho
     }
 }
 
-struct SortLayout {
-    u32* totals;   // keys of each digit in the current pass
-    u32* look[2];  // per-tile digit counts and output offsets
-    u32* chunk;    // per-chunk digit sums, then their scan
+struct Layout {
+    u32 *totals, *chunk, *tile_pos;
+    unsigned short* counts;
     Key* keys_alt;
     u32* vals_alt;
+    long long tiles, chunks;
     size_t bytes;
-    long long tiles;
 };
 
-SortLayout sort_layout(void* ws, long long n) {
-    SortLayout l;
+Layout layout(void* ws, long long n) {
+    Layout l;
     Carver c(ws);
     l.tiles = (n + kTile - 1) / kTile;
+    l.chunks = (l.tiles + kChunkTiles - 1) / kChunkTiles;
     l.totals = c.take<u32>(kRadix);
-    l.look[0] = c.take<u32>((size_t)l.tiles * kRadix);
-    l.look[1] = c.take<u32>((size_t)l.tiles * kRadix);
-    l.chunk = c.take<u32>((size_t)((l.tiles + kChunkTiles - 1) / kChunkTiles) * kRadix);
+    l.counts = c.take<unsigned short>((size_t)l.tiles * kRadix);
+    l.tile_pos = c.take<u32>((size_t)l.tiles * kRadix);
+    l.chunk = c.take<u32>((size_t)l.chunks * kRadix);
     l.keys_alt = c.take<Key>((size_t)n);
     l.vals_alt = c.take<u32>((size_t)n);
     l.bytes = c.size();
     return l;
 }
 
+int run(const Key* keys_in, Key* keys_out, u32* perm, long long n, void* ws, cudaStream_t st) {
+    const Layout l = layout(ws, n);
+    const int smem = static_cast<int>(sizeof(PassSmem));
+    const unsigned tiles = static_cast<unsigned>(l.tiles), chunks = static_cast<unsigned>(l.chunks);
+    CST_CUDA(cudaMemsetAsync(ws, 0, sizeof(WsHeader), st));
+    CST_CUDA(cudaFuncSetAttribute(sort_pass_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CST_CUDA(cudaFuncSetAttribute(sort_pass_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const Key* ksrc = keys_in;
+    const u32* vsrc = nullptr;
+    for (int p = 0; p < kPasses; ++p) {  // odd passes (from 1) write the workspace, even ones the output
+        Key* kdst = (p % 2 == 0) ? l.keys_alt : keys_out;
+        u32* vdst = (p % 2 == 0) ? l.vals_alt : perm;
+        tile_count_kernel<<<tiles, kThreads, 0, st>>>(ksrc, n, p * kRadixBits, l.counts);
+        CST_LAUNCHED("tile_count_kernel");
+        chunk_sum_kernel<<<chunks, kRadix, 0, st>>>(l.counts, l.tiles, l.chunk);
+        CST_LAUNCHED("chunk_sum_kernel");
+        chunk_scan_kernel<<<kRadix, 1024, 0, st>>>(l.chunk, l.chunks, l.totals);
+        CST_LAUNCHED("chunk_scan_kernel");
+        tile_offsets_kernel<<<chunks, kRadix, 0, st>>>(l.counts, l.tiles, l.chunk, l.totals, l.tile_pos);
+        CST_LAUNCHED("tile_offsets_kernel");
+        if (p == 0)
+            sort_pass_kernel<true><<<tiles, kThreads, smem, st>>>(ksrc, kdst, vsrc, vdst, n, p, l.tile_pos);
+        else
+            sort_pass_kernel<false><<<tiles, kThreads, smem, st>>>(ksrc, kdst, vsrc, vdst, n, p, l.tile_pos);
+        CST_LAUNCHED("sort_pass_kernel");
+        ksrc = kdst;
+        vsrc = vdst;
+    }
+    return CSTONE_OK;
+}
+}  // namespace digits
+
+// ---------------------------------------------------------------------------- host
+struct SortLayout {
+    Tables t;
+    Key* keys_a;
+    u32* vals_a;
+    size_t bytes;
+};
+
+struct SortSizes {  // entries of the tables
+    size_t big, parts, small, tiles;
+};
+
+// At most n / kSmall buckets are split in a round, into at most size / kTarget + 1 parts each.
+constexpr SortSizes sort_sizes(long long n, int n_segs) {
+    const size_t big = static_cast<size_t>(n / kSmall) + 1;
+    const size_t parts = static_cast<size_t>(n / kTarget) + 2 * big + 1;
+    return SortSizes{big, parts, static_cast<size_t>(n_segs) + 2 * parts, static_cast<size_t>(n / kTile) + big + 1};
+}
+
+SortLayout sort_layout(void* ws, long long n, int n_segs) {
+    SortLayout l;
+    Carver c(ws);
+    const SortSizes s = sort_sizes(n, n_segs);
+    u32* counters = c.take<u32>(3);
+    l.t.big[0].count = counters;
+    l.t.big[1].count = counters ? counters + 1 : nullptr;
+    l.t.n_small = counters ? counters + 2 : nullptr;
+    for (int k = 0; k < 2; ++k) {
+        l.t.big[k].start = c.take<u32>(s.big);
+        l.t.big[k].size = c.take<u32>(s.big);
+        l.t.big[k].base = c.take<Key>(s.big);
+        l.t.big[k].first_part = c.take<u32>(s.big + 1);
+        l.t.big[k].first_tile = c.take<u32>(s.big + 1);
+    }
+    l.t.part_key = c.take<Key>(s.parts);
+    l.t.part_idx = c.take<u32>(s.parts);
+    l.t.part_pos = c.take<u32>(s.parts * kPosStride);
+    l.t.small = c.take<uint2>(s.small);
+    l.t.small_base = c.take<Key>(s.small);
+    l.t.part_of = c.take<u16>((size_t)n);
+    l.t.tile_bucket = c.take<u32>(s.tiles);
+    l.keys_a = c.take<Key>((size_t)n);
+    l.vals_a = c.take<u32>((size_t)n);
+    l.bytes = c.size();
+    return l;
+}
+
+template <int SRC>
+int run_round(const Pairs& p, const SortLayout& l, const Buckets& cur, const Buckets& next, long long max_big,
+              int idx_bits, cudaStream_t st) {
+    const int sms = sm_count();
+    const int smem = static_cast<int>(sizeof(BigSmem)), ssmem = static_cast<int>(sizeof(ScatterSmem));
+    CST_CUDA(cudaFuncSetAttribute(sort_sample_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    CST_CUDA(cudaFuncSetAttribute(sort_scatter_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssmem));
+    const int bgrid = static_cast<int>(max_big < 2 * sms ? max_big : 2 * sms);
+    sort_sample_kernel<SRC><<<bgrid, kBigThreads, smem, st>>>(p, cur, l.t, idx_bits);
+    CST_LAUNCHED("sort_sample_kernel");
+    sort_count_kernel<SRC><<<sms * kCountBlocks, kThreads, 0, st>>>(p, cur, l.t);
+    CST_LAUNCHED("sort_count_kernel");
+    sort_plan_kernel<<<bgrid, kMaxParts, 0, st>>>(cur, next, l.t, SRC == kBufA ? kBufB : kBufA);
+    CST_LAUNCHED("sort_plan_kernel");
+    sort_scatter_kernel<SRC><<<sms * CSTONE_SORT_MIN_BLOCKS, kThreads, ssmem, st>>>(p, cur, l.t);
+    CST_LAUNCHED("sort_scatter_kernel");
+    return CSTONE_OK;
+}
+
+// Sorts every segment (seg_offsets NULL: one segment of n keys).
+int run_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, const long long* seg_offsets, int n_segs,
+             void* ws, cudaStream_t st) {
+    SortLayout l = sort_layout(ws, n, n_segs);
+    WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
+    if (n == 0) {
+        CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
+        return CSTONE_OK;
+    }
+    if (!seg_offsets && digits::taken(n)) return digits::run(keys_in, keys_out, perm, n, ws, st);
+    const int rounds = rounds_for(n);
+    const Pairs p{keys_in, l.keys_a, l.vals_a, keys_out, perm};
+    int idx_bits = 1;
+    while ((1ll << idx_bits) < n) ++idx_bits;
+    sort_init_kernel<<<1, 1024, 0, st>>>(seg_offsets, n_segs, n, rounds, l.t, hdr);
+    CST_LAUNCHED("sort_init_kernel");
+    // buckets of a round: of round 1, no more than segments
+    const long long cap = static_cast<long long>(sort_sizes(n, n_segs).big);
+    const long long cap1 = cap < n_segs ? cap : n_segs;
+    if (rounds >= 1) {
+        if (int rc = run_round<kInput>(p, l, l.t.big[0], l.t.big[1], cap1, idx_bits, st)) return rc;
+    }
+    if (rounds == 2) {
+        sort_prefix_kernel<<<1, 1024, 0, st>>>(l.t.big[1], l.t.big[0].count, 1);
+        CST_LAUNCHED("sort_prefix_kernel");
+        if (int rc = run_round<kBufA>(p, l, l.t.big[1], l.t.big[0], cap, idx_bits, st)) return rc;
+    }
+    const int sms = sm_count();
+    const int smem = static_cast<int>(sizeof(SmallSmem)), bsmem = static_cast<int>(sizeof(BigSmem));
+    CST_CUDA(cudaFuncSetAttribute(sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    const long long want = static_cast<long long>(sort_sizes(n, n_segs).small);
+    sort_small_kernel<<<(unsigned)(want < kSmallBlocks * sms ? want : kSmallBlocks * sms), kSmallThreads, smem, st>>>(p, l.t, idx_bits);
+    CST_LAUNCHED("sort_small_kernel");
+    if (rounds == 1) {
+        CST_CUDA(cudaFuncSetAttribute(sort_rest_kernel<kBufA>, cudaFuncAttributeMaxDynamicSharedMemorySize, bsmem));
+        sort_rest_kernel<kBufA><<<(unsigned)(cap < 2 * sms ? cap : 2 * sms), kBigThreads, bsmem, st>>>(p, l.t.big[1],
+                                                                                                        idx_bits);
+        CST_LAUNCHED("sort_rest_kernel");
+    } else if (rounds == 2) {
+        CST_CUDA(cudaFuncSetAttribute(sort_rest_kernel<kBufB>, cudaFuncAttributeMaxDynamicSharedMemorySize, bsmem));
+        sort_rest_kernel<kBufB><<<(unsigned)(cap < 2 * sms ? cap : 2 * sms), kBigThreads, bsmem, st>>>(p, l.t.big[0],
+                                                                                                        idx_bits);
+        CST_LAUNCHED("sort_rest_kernel");
+    }
+    return CSTONE_OK;
+}
+
 }  // namespace
 
-size_t sort_ws_bytes(long long n) { return sort_layout(nullptr, n).bytes; }
+size_t sort_ws_bytes(long long n) {
+    return digits::taken(n) ? digits::layout(nullptr, n).bytes : sort_layout(nullptr, n, 1).bytes;
+}
+size_t sort_segmented_ws_bytes(long long n, int n_segs) { return sort_layout(nullptr, n, n_segs).bytes; }
 
 #ifndef CSTONE_KEY32  // the allocation-free sort exists for 63-bit keys only
 // ---------------------------------------------------------------- sort without allocation
@@ -506,11 +1367,12 @@ size_t sort_ws_bytes(long long n) { return sort_layout(nullptr, n).bytes; }
 namespace {
 constexpr size_t round256(size_t b) { return (b + 255) / 256 * 256; }
 constexpr long long kStaticKeys = CSTONE_SORT_STATIC_MAX_KEYS;
-constexpr size_t kStaticTiles = static_cast<size_t>((kStaticKeys + kTile - 1) / kTile);
-constexpr size_t kStaticBytes = sizeof(WsHeader) + round256(kRadix * 4) + 2 * round256(kStaticTiles * kRadix * 4) +
-                                round256((kStaticTiles + kChunkTiles - 1) / kChunkTiles * kRadix * 4) +
-                                round256(static_cast<size_t>(kStaticKeys) * 8) +
-                                round256(static_cast<size_t>(kStaticKeys) * 4);
+constexpr SortSizes kStaticSizes = sort_sizes(kStaticKeys, 1);
+constexpr size_t kStaticBytes =
+    sizeof(WsHeader) + round256(3 * 4) + 2 * (4 * round256((kStaticSizes.big + 1) * 4) + round256(kStaticSizes.big * 8)) +
+    round256(kStaticSizes.parts * 8) + round256(kStaticSizes.parts * 4) + round256(kStaticSizes.parts * 4 * kPosStride) + 2 * round256(kStaticSizes.small * 8) +
+    round256(static_cast<size_t>(kStaticKeys) * 2) + round256(kStaticSizes.tiles * 4) + round256(static_cast<size_t>(kStaticKeys) * 8) +
+    round256(static_cast<size_t>(kStaticKeys) * 4);
 
 __device__ __align__(256) unsigned char g_sort_scratch[kStaticBytes];
 
@@ -546,115 +1408,6 @@ int static_sort_scratch(void** out, cudaStream_t st) {
 }  // namespace
 #endif
 
-// The digit passes (an even number). Ping-pong: odd passes (1-based) write the workspace buffers,
-// even passes the output, so the last pass lands in keys_out / perm. Ahead of each pass: tile
-// counts (counts), chunk sums and their scan (chunk), and the per-tile positions (tile_pos).
-template <bool SEG>
-int run_passes(const Key* keys_in, Key* keys_out, u32* perm, long long n, long long tiles, u32* totals,
-               u32* counts, u32* chunk, u32* tile_pos, Key* keys_alt, u32* vals_alt, SegTiles seg, cudaStream_t st) {
-    const int smem = static_cast<int>(sizeof(PassSmem));
-    CST_CUDA(cudaFuncSetAttribute(sort_pass_kernel<true, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    CST_CUDA(cudaFuncSetAttribute(sort_pass_kernel<false, SEG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    const Key* ksrc = keys_in;
-    const u32* vsrc = nullptr;
-    const long long nchunks = (tiles + kChunkTiles - 1) / kChunkTiles;
-    // tile counts as 16-bit words (a tile holds fewer than 2^16 keys) in the counts buffer
-    unsigned short* counts16 = reinterpret_cast<unsigned short*>(counts);
-    static_assert(kTile < 65536, "16-bit tile counts");
-    static_assert(kPasses % 2 == 0, "the last pass must write the output buffers");
-    for (int p = 0; p < kPasses; ++p) {
-        Key* kdst = (p % 2 == 0) ? keys_alt : keys_out;
-        u32* vdst = (p % 2 == 0) ? vals_alt : perm;
-        tile_count_kernel<SEG><<<(unsigned)tiles, kThreads, 0, st>>>(ksrc, n, p * kRadixBits, counts16, seg);
-        CST_LAUNCHED("tile_count_kernel");
-        chunk_sum_kernel<<<(unsigned)nchunks, kRadix, 0, st>>>(counts16, tiles, chunk);
-        CST_LAUNCHED("chunk_sum_kernel");
-        // a segmented sort scans all tiles from 0 and places the digits per segment; each tile
-        // subtracts its segment's first tile
-        chunk_scan_kernel<<<kRadix, 1024, 0, st>>>(chunk, nchunks, SEG ? nullptr : totals);
-        CST_LAUNCHED("chunk_scan_kernel");
-        tile_offsets_kernel<<<(unsigned)nchunks, kRadix, 0, st>>>(counts16, tiles, chunk, SEG ? nullptr : totals,
-                                                                  tile_pos);
-        CST_LAUNCHED("tile_offsets_kernel");
-        if (p == 0)
-            sort_pass_kernel<true, SEG><<<(unsigned)tiles, kThreads, smem, st>>>(ksrc, kdst, vsrc, vdst, n, p,
-                                                                                 tile_pos, seg);
-        else
-            sort_pass_kernel<false, SEG><<<(unsigned)tiles, kThreads, smem, st>>>(ksrc, kdst, vsrc, vdst, n, p,
-                                                                                  tile_pos, seg);
-        CST_LAUNCHED("sort_pass_kernel");
-        ksrc = kdst;
-        vsrc = vdst;
-    }
-    return CSTONE_OK;
-}
-
-int launch_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, void* ws, cudaStream_t st) {
-    SortLayout l = sort_layout(ws, n);
-    WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-    CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
-    if (n == 0) return CSTONE_OK;
-    return run_passes<false>(keys_in, keys_out, perm, n, l.tiles, l.totals, l.look[0], l.chunk, l.look[1], l.keys_alt,
-                             l.vals_alt, SegTiles{}, st);
-}
-
-// ---------------------------------------------------------------- segmented sort
-namespace {
-struct SegLayout {
-    SegBuild b;
-    u32* look[2];  // per-tile digit counts and positions
-    u32* chunk;
-    Key* keys_alt;
-    u32* vals_alt;
-    size_t bytes;
-    long long max_tiles;
-};
-
-SegLayout seg_layout(void* ws, long long n, int n_segs) {
-    SegLayout l;
-    Carver c(ws);
-    l.max_tiles = (n + kTile - 1) / kTile + n_segs;
-    l.b.n_tiles = c.take<u32>(1);
-    l.b.tile_seg = c.take<u32>((size_t)l.max_tiles);
-    l.b.tile_base = c.take<u32>((size_t)l.max_tiles);
-    l.b.tile_count = c.take<u32>((size_t)l.max_tiles);
-    l.b.seg_first = c.take<u32>((size_t)n_segs + 1);
-    l.b.seg_hist = c.take<u32>((size_t)n_segs * kPasses * kRadix);
-    l.b.seg_offsets = c.take<u32>((size_t)n_segs * kPasses * kRadix);
-    l.look[0] = c.take<u32>((size_t)l.max_tiles * kRadix);
-    l.look[1] = c.take<u32>((size_t)l.max_tiles * kRadix);
-    l.chunk = c.take<u32>((size_t)((l.max_tiles + kChunkTiles - 1) / kChunkTiles) * kRadix);
-    l.keys_alt = c.take<Key>((size_t)n);
-    l.vals_alt = c.take<u32>((size_t)n);
-    l.bytes = c.size();
-    return l;
-}
-
-}  // namespace
-
-size_t sort_segmented_ws_bytes(long long n, int n_segs) { return seg_layout(nullptr, n, n_segs).bytes; }
-
-int launch_sort_segmented(const Key* keys_in, Key* keys_out, u32* perm, long long n, const long long* seg_offsets,
-                          int n_segs, void* ws, cudaStream_t st) {
-    SegLayout l = seg_layout(ws, n, n_segs);
-    WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-    CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
-    if (n == 0) return CSTONE_OK;
-    CST_CUDA(cudaMemsetAsync(l.b.seg_hist, 0, (size_t)n_segs * kPasses * kRadix * sizeof(u32), st));
-    seg_setup_kernel<<<1, 1024, 0, st>>>(seg_offsets, n_segs, l.b);
-    CST_LAUNCHED("seg_setup_kernel");
-    const long long want = (l.max_tiles + kThreads - 1) / kThreads;
-    const int tgrid = static_cast<int>(want < (long long)sm_count() * 4 ? want : (long long)sm_count() * 4);
-    seg_tiles_kernel<<<tgrid, kThreads, 0, st>>>(seg_offsets, n_segs, static_cast<u32>(l.max_tiles), l.b);
-    CST_LAUNCHED("seg_tiles_kernel");
-    const SegTiles view{l.b.n_tiles, l.b.tile_seg, l.b.tile_base, l.b.tile_count, l.b.seg_first, l.b.seg_offsets};
-    seg_hist_kernel<<<(unsigned)l.max_tiles, kThreads, 0, st>>>(keys_in, view, l.b.seg_hist);
-    CST_LAUNCHED("seg_hist_kernel");
-    seg_scan_kernel<<<(unsigned)n_segs, 32 * kPasses, 0, st>>>(seg_offsets, l.b.seg_hist, l.b.seg_offsets);
-    CST_LAUNCHED("seg_scan_kernel");
-    return run_passes<true>(keys_in, keys_out, perm, n, l.max_tiles, nullptr, l.look[0], l.chunk, l.look[1], l.keys_alt,
-                            l.vals_alt, view, st);
-}
 
 }  // namespace CST_NS
 
@@ -673,8 +1426,8 @@ int CSTONE_FN(sort)(const CST_KEY_C* keys_in, CST_KEY_C* keys_out, uint32_t* per
     if (n < 0 || n >= CSTONE_MAX_PARTICLES || (n > 0 && (!keys_in || !keys_out || !perm)))
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(sort)) ": bad argument (n=%lld)", (long long)n);
     if (int rc = cst::check_ws(ws, ws_bytes, CST_NS::sort_ws_bytes(n), CST_STR(CSTONE_FN(sort)))) return rc;
-    return CST_NS::launch_sort(reinterpret_cast<const CST_NS::Key*>(keys_in), reinterpret_cast<CST_NS::Key*>(keys_out),
-                               perm, n, ws, cst::as_stream(stream));
+    return CST_NS::run_sort(reinterpret_cast<const CST_NS::Key*>(keys_in), reinterpret_cast<CST_NS::Key*>(keys_out),
+                            perm, n, nullptr, 1, ws, cst::as_stream(stream));
 }
 
 #ifndef CSTONE_KEY32
@@ -690,8 +1443,8 @@ int cstone_sort_static(const uint64_t* keys_in, uint64_t* keys_out, uint32_t* pe
         return cst::fail(CSTONE_ERR_INVALID_ARG, "cstone_sort_static: static scratch too small");
     void* ws = nullptr;
     if (int rc = cst::static_sort_scratch(&ws, cst::as_stream(stream))) return rc;
-    return cst::launch_sort(reinterpret_cast<const cst::u64*>(keys_in), reinterpret_cast<cst::u64*>(keys_out), perm,
-                            n, ws, cst::as_stream(stream));
+    return cst::run_sort(reinterpret_cast<const cst::u64*>(keys_in), reinterpret_cast<cst::u64*>(keys_out), perm, n,
+                         nullptr, 1, ws, cst::as_stream(stream));
 }
 
 int cstone_sort_segmented_workspace_size(int64_t n, int32_t n_segs, size_t* bytes) {
@@ -711,9 +1464,8 @@ int cstone_sort_segmented(const uint64_t* keys_in, uint64_t* keys_out, uint32_t*
         return cst::fail(CSTONE_ERR_INVALID_ARG, "cstone_sort_segmented: keys_in must not alias keys_out");
     if (int rc = cst::check_ws(ws, ws_bytes, cst::sort_segmented_ws_bytes(n, n_segs), "cstone_sort_segmented"))
         return rc;
-    return cst::launch_sort_segmented(reinterpret_cast<const cst::u64*>(keys_in), reinterpret_cast<cst::u64*>(keys_out),
-                                      perm, n, reinterpret_cast<const long long*>(seg_offsets), n_segs, ws,
-                                      cst::as_stream(stream));
+    return cst::run_sort(reinterpret_cast<const cst::u64*>(keys_in), reinterpret_cast<cst::u64*>(keys_out), perm, n,
+                         reinterpret_cast<const long long*>(seg_offsets), n_segs, ws, cst::as_stream(stream));
 }
 
 #endif

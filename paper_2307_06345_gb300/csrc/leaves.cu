@@ -1,5 +1,6 @@
-// Cornerstone leaf array: the f / g iteration of Sec. 4 (Eqs. histogram, g1, g2, g3) in one
-// persistent cooperative kernel.
+// Cornerstone leaf array. A cold start (from the roots) finds the converged array in one sweep over
+// the keys (leaves_cold.cuh); a warm start, and a cold one with a large N_crit, run the f / g iteration of
+// Sec. 4 (Eqs. histogram, g1, g2, g3) in one persistent cooperative kernel, described here.
 //
 // Alongside K the kernel keeps pos_i = lower_bound(P, K_i) for every key of the array. Then the
 // histogram of Eq. (histogram) is N_i = pos_{i+1} - pos_i, and the combined count of 8 sibling
@@ -47,12 +48,21 @@ struct LoopState {
     u32 changed[kMaxIters];       // pass t changed an array
     u32 nsplit[kMaxIters];        // splits queued in pass t (written by the pass's last tile)
     GridBarrier bar;
-    u32 iters;                    // passes executed (set at convergence)
-    u32 converged;
-    u32 required;                 // elements needed when the capacity was exceeded
-    u32 final_buf;                // buffer holding the converged arrays
     unsigned long long phase_stamp[kMaxIters][2];  // %globaltimer after pass t's first and second sweep
+    int cold_levels[kLevels + 2];  // cold build: internal nodes per level, as differences
+    u32 cold_starts;               // cold build: leaf starts listed so far
 };
+
+// What the host reads of a finished build, in the workspace's header behind the error word: one
+// small copy instead of the whole loop state.
+struct Outcome {
+    u32 iters;
+    u32 converged;
+    u32 required;
+    u32 ne;  // elements of the converged arrays
+};
+static_assert(sizeof(Outcome) <= sizeof(WsHeader::pad), "the outcome fits the header");
+__host__ __device__ inline Outcome* outcome_of(WsHeader* h) { return reinterpret_cast<Outcome*>(h->pad); }
 
 struct LeafBufs {
     uint4* split_q;   // [ecap] queued splits: first particle, particle count, first child's position,
@@ -372,7 +382,8 @@ __global__ void __launch_bounds__(kThreads, CSTONE_LEAVES_MIN_BLOCKS) leaves_loo
                         const u64 ne_next = o_pos + 1;
                         ls->ne[t + 1] = static_cast<u32>(ne_next > 0xffffffffULL ? 0xffffffffULL : ne_next);
                         if (ne_next > ecap) {
-                            ls->required = static_cast<u32>(ne_next > 0xffffffffULL ? 0xffffffffULL : ne_next);
+                            outcome_of(hdr)->required =
+                                static_cast<u32>(ne_next > 0xffffffffULL ? 0xffffffffULL : ne_next);
                             raise_error(hdr, CSTONE_ERR_CAPACITY, 0u);
                         }
                     }
@@ -493,9 +504,7 @@ __global__ void __launch_bounds__(kThreads, CSTONE_LEAVES_MIN_BLOCKS) leaves_loo
         unsigned long long now;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
         ls->stamp[t] = now;
-        ls->iters = static_cast<u32>(t);
-        ls->converged = converged ? 1u : 0u;
-        ls->final_buf = static_cast<u32>(last & 1);
+        *outcome_of(hdr) = Outcome{static_cast<u32>(t), converged ? 1u : 0u, 0u, converged ? ls->ne[last] : 0u};
     }
     if (!converged) {
         if (fallback) write_root_arrays<BATCH>(P, n, sv, gtid, gthreads, out_keys, out_counts, out_offsets);
@@ -519,17 +528,26 @@ __global__ void __launch_bounds__(kThreads, CSTONE_LEAVES_MIN_BLOCKS) leaves_loo
     }
 }
 
+}  // namespace
+}  // namespace CST_NS
+
+#include "leaves_cold.cuh"
+
+namespace CST_NS {
+namespace {
+
 struct LeavesLayout {
     LoopState* ls;
     LeafBufs bufs;
+    cold::Tiles tiles;  // of a cold build: the list lies in the loop's split queue
     size_t bytes;
 };
 
-LeavesLayout leaves_layout(void* ws, long long ecap, int max_iters, bool batch) {
-    (void)max_iters;
+// n: particles (in a batched build the most there can be, the size query does not know them).
+LeavesLayout leaves_layout(void* ws, long long n, long long ecap, bool batch) {
     LeavesLayout l;
     Carver c(ws);
-    l.ls = c.take<LoopState>(1);
+    l.ls = c.take<LoopState>(1);  // directly behind the header: both are cleared together
     l.bufs.split_q = c.take<uint4>((size_t)ecap);
     l.bufs.ops = c.take<unsigned char>((size_t)ecap);
     l.bufs.tile_sum = c.take<u64>((size_t)((ecap + kTile - 1) / kTile));
@@ -538,6 +556,15 @@ LeavesLayout leaves_layout(void* ws, long long ecap, int max_iters, bool batch) 
         l.bufs.pos[k] = c.take<u32>((size_t)ecap);
         l.bufs.set[k] = batch ? c.take<u32>((size_t)ecap) : nullptr;
     }
+    const u32 most = cold::tiles_of(batch ? CSTONE_MAX_PARTICLES : n);
+    l.tiles.list = c.take<u32>(most);
+    l.tiles.count = c.take<u32>(most);
+    l.tiles.elems = c.take<u32>(most);
+    l.tiles.tiles = cold::tiles_of(n);
+    l.tiles.starts = reinterpret_cast<u32*>(l.bufs.split_q);
+    l.tiles.start_cap = static_cast<u32>(ecap);
+    l.tiles.n_starts = l.ls ? &l.ls->cold_starts : nullptr;
+    l.tiles.levels = l.ls ? l.ls->cold_levels : nullptr;
     l.bytes = c.size();
     return l;
 }
@@ -551,12 +578,10 @@ int leaves_grid() {
 // overflow, the count needed). Synchronises the stream.
 int read_leaves_result(void* ws, cudaStream_t st, long long ecap, int max_iters, long long* ne_out, int* iters,
                        const char* who) {
-    LoopState* lsp = reinterpret_cast<LoopState*>(static_cast<char*>(ws) + sizeof(WsHeader));
     WsHeader h;
-    LoopState s;
     CST_CUDA(cudaMemcpyAsync(&h, ws, sizeof(h), cudaMemcpyDeviceToHost, st));
-    CST_CUDA(cudaMemcpyAsync(&s, lsp, sizeof(s), cudaMemcpyDeviceToHost, st));
     CST_CUDA(cudaStreamSynchronize(st));
+    const Outcome s = *outcome_of(&h);
     if (iters) *iters = static_cast<int>(s.iters);
     if (h.err == CSTONE_ERR_CAPACITY) {
         *ne_out = s.required;
@@ -564,11 +589,33 @@ int read_leaves_result(void* ws, cudaStream_t st, long long ecap, int max_iters,
     }
     if (h.err) return fail(static_cast<int>(h.err), "%s: device error %u (info 0x%x)", who, h.err, h.err_info);
     if (!s.converged) return fail(CSTONE_ERR_NOT_CONVERGED, "%s: not converged after %d passes", who, max_iters);
-    *ne_out = s.ne[s.iters - 1];  // the last pass changed nothing: its input is the result
+    *ne_out = s.ne;
     return CSTONE_OK;
 }
 
-// Runs the loop. ne0: element count of the warm-start arrays held in `leaves` (0 = cold start from
+template <bool BATCH>
+int run_cold(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap, u32* counts, u32* offsets,
+             int max_iters, SetView sv, const LeavesLayout& l, WsHeader* hdr, bool fallback, cudaStream_t st) {
+    const cold::View v{BATCH ? sv.particle_offsets : nullptr, sv.n_sets, static_cast<u32>(n)};
+    const u32 tiles = l.tiles.tiles;
+    const u32 sms = static_cast<u32>(sm_count());
+    u32* first = offsets ? offsets : l.bufs.pos[0];
+    auto grid = [&](u32 per_sm) { return tiles < sms * per_sm ? tiles : sms * per_sm; };
+    cold::starts_kernel<BATCH><<<grid(cold::kBlocks), cold::kThreads, cold::sweep_smem(ncrit), st>>>(P, v, ncrit, l.tiles);
+    CST_LAUNCHED("starts_kernel");
+    cold::outcome_kernel<<<1, 1024, 0, st>>>(l.tiles, sv.n_sets, static_cast<u32>(ecap), max_iters, hdr);
+    CST_LAUNCHED("outcome_kernel");
+    cold::emit_kernel<BATCH><<<grid(8), cold::kThreads, 0, st>>>(P, v, l.tiles, static_cast<u32>(ecap), hdr, leaves, first,
+                                                                 sv.element_offsets);
+    CST_LAUNCHED("emit_kernel");
+    const long long want = (ecap + cold::kThreads - 1) / cold::kThreads;
+    cold::counts_kernel<BATCH><<<(unsigned)(want < 8ll * sms ? want : 8ll * sms), cold::kThreads, 0, st>>>(
+        P, v, fallback ? 1 : 0, hdr, leaves, counts, first, offsets, sv.element_offsets);
+    CST_LAUNCHED("counts_kernel");
+    return CSTONE_OK;
+}
+
+// Runs the build. ne0: element count of the warm-start arrays held in `leaves` (0 = cold start from
 // the roots, -1 = warm start with the count read on the device). With sync, *ne_out is the element
 // count of the converged arrays on success; without, nothing is read back (the outcome stays in
 // the workspace for read_leaves_result) and a failure leaves every set's root array as output.
@@ -576,10 +623,17 @@ template <bool BATCH>
 int run_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap, long long ne0, long long* ne_out,
                u32* counts, u32* offsets, int max_iters, int* iters, SetView sv, void* ws, cudaStream_t st,
                const char* who, bool sync = true) {
-    LeavesLayout l = leaves_layout(ws, ecap, max_iters, BATCH);
+    LeavesLayout l = leaves_layout(ws, n, ecap, BATCH);
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
-    CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
-    CST_CUDA(cudaMemsetAsync(l.ls, 0, sizeof(LoopState), st));
+    CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader) + sizeof(LoopState), st));
+    // A cold build takes one sweep over the keys instead of a pass per level (2^27 clumps: 1.47 ms in the
+    // loop); a window of more than kMaxNcrit particles does not fit its shared memory.
+    if (ne0 == 0 && ncrit <= cold::kMaxNcrit) {
+        if (int rc = run_cold<BATCH>(P, n, ncrit, leaves, ecap, counts, offsets, max_iters, sv, l, hdr, !sync, st))
+            return rc;
+        if (!sync) return CSTONE_OK;
+        return read_leaves_result(ws, st, ecap, max_iters, ne_out, iters, who);
+    }
     int warm = ne0 != 0 ? 1 : 0;
     u32 ne_start = ne0 < 0 ? kDeviceCount : static_cast<u32>(ne0);
     int fallback = sync ? 0 : 1;
@@ -602,10 +656,8 @@ int run_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap
 
 }  // namespace
 
-size_t leaves_ws_bytes(long long cap, int max_iters) { return leaves_layout(nullptr, cap + 1, max_iters, false).bytes; }
-size_t leaves_batched_ws_bytes(long long ecap, int max_iters) {
-    return leaves_layout(nullptr, ecap, max_iters, true).bytes;
-}
+size_t leaves_ws_bytes(long long n, long long cap) { return leaves_layout(nullptr, n, cap + 1, false).bytes; }
+size_t leaves_batched_ws_bytes(long long ecap) { return leaves_layout(nullptr, 0, ecap, true).bytes; }
 
 int launch_build_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long cap, long long* n_leaves,
                         u32* counts, u32* offsets, int max_iters, int* iters, void* ws, cudaStream_t st) {
@@ -648,7 +700,7 @@ int CSTONE_FN(leaves_workspace_size)(int64_t n, int64_t leaf_cap, int32_t max_it
     if (!bytes || n < 0 || n >= CSTONE_MAX_PARTICLES || leaf_cap < 1 || leaf_cap > CSTONE_MAX_LEAVES ||
         max_iters < 1 || max_iters > 256)
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(leaves_workspace_size)) ": bad argument");
-    *bytes = CST_NS::leaves_ws_bytes(leaf_cap, max_iters);
+    *bytes = CST_NS::leaves_ws_bytes(n, leaf_cap);
     return CSTONE_OK;
 }
 
@@ -661,7 +713,7 @@ int CSTONE_FN(build_leaves)(const CST_KEY_C* sorted_keys, int64_t n, uint32_t nc
     if (*n_leaves < 0 || *n_leaves > leaf_cap)
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(build_leaves)) ": initial n_leaves %lld outside "
                          "[0, %lld]", (long long)*n_leaves, (long long)leaf_cap);
-    if (int rc = cst::check_ws(ws, ws_bytes, CST_NS::leaves_ws_bytes(leaf_cap, max_iters),
+    if (int rc = cst::check_ws(ws, ws_bytes, CST_NS::leaves_ws_bytes(n, leaf_cap),
                                CST_STR(CSTONE_FN(build_leaves))))
         return rc;
     long long nl = *n_leaves;
@@ -678,7 +730,7 @@ int CSTONE_FN(build_leaves)(const CST_KEY_C* sorted_keys, int64_t n, uint32_t nc
 int cstone_leaves_batched_workspace_size(int64_t elem_cap, int32_t max_iters, size_t* bytes) {
     if (!bytes || elem_cap < 2 || elem_cap > CSTONE_MAX_LEAVES || max_iters < 1 || max_iters > 256)
         return cst::fail(CSTONE_ERR_INVALID_ARG, "cstone_leaves_batched_workspace_size: bad argument");
-    *bytes = cst::leaves_batched_ws_bytes(elem_cap, max_iters);
+    *bytes = cst::leaves_batched_ws_bytes(elem_cap);
     return CSTONE_OK;
 }
 
@@ -693,7 +745,7 @@ int cstone_build_leaves_batched(const uint64_t* sorted_keys, int64_t n, const in
     if (*n_elements < 0 || *n_elements > elem_cap || (*n_elements > 0 && *n_elements < 2 * (int64_t)n_sets))
         return cst::fail(CSTONE_ERR_INVALID_ARG, "cstone_build_leaves_batched: initial n_elements %lld invalid",
                          (long long)*n_elements);
-    if (int rc = cst::check_ws(ws, ws_bytes, cst::leaves_batched_ws_bytes(elem_cap, max_iters),
+    if (int rc = cst::check_ws(ws, ws_bytes, cst::leaves_batched_ws_bytes(elem_cap),
                                "cstone_build_leaves_batched"))
         return rc;
     long long ne = *n_elements;
@@ -716,7 +768,7 @@ int cstone_build_leaves_batched_async(const uint64_t* sorted_keys, int64_t n, co
         !element_offsets || !counts || elem_cap < 2 * (int64_t)n_sets || elem_cap > CSTONE_MAX_LEAVES ||
         max_iters < 1 || max_iters > 256 || (n > 0 && !sorted_keys))
         return cst::fail(CSTONE_ERR_INVALID_ARG, "cstone_build_leaves_batched_async: bad argument");
-    if (int rc = cst::check_ws(ws, ws_bytes, cst::leaves_batched_ws_bytes(elem_cap, max_iters),
+    if (int rc = cst::check_ws(ws, ws_bytes, cst::leaves_batched_ws_bytes(elem_cap),
                                "cstone_build_leaves_batched_async"))
         return rc;
     return cst::launch_build_leaves_batched_async(reinterpret_cast<const cst::u64*>(sorted_keys), n,

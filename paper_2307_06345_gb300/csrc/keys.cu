@@ -178,16 +178,10 @@ __device__ __forceinline__ u32 grid_cell(double x, double lo, double scale) {
 struct FixedGrid {
     long long lo_fixed;   // LO
     u64 scale_fixed;      // S
-    u64 lo_ord, hi_ord;   // order-preserving bits of lo and of lo + 2 side
     double lo, scale;
     int F, R;
     int fast;
 };
-
-__device__ __forceinline__ u64 order_bits(double v) {
-    u64 b = static_cast<u64>(__double_as_longlong(v));
-    return (b >> 63) ? ~b : (b | (1ULL << 63));
-}
 
 __device__ __forceinline__ int exponent_of(double v) {  // unbiased exponent field (0 for zero/subnormal)
     return static_cast<int>((static_cast<u64>(__double_as_longlong(v)) >> 52) & 0x7ffu);
@@ -211,8 +205,6 @@ __device__ FixedGrid make_fixed_grid(double lo, double side, int F_frame = 0) {
     f.lo = lo;
     f.scale = __ddiv_rn(2097152.0, side);
     const double hi = __dadd_rn(lo, __dmul_rn(2.0, side));
-    f.lo_ord = order_bits(lo);
-    f.hi_ord = order_bits(hi);
     // 2^E > max(|lo|, |hi|)
     const int e_max = max(exponent_of(lo), exponent_of(hi)) - 1023 + 1;
     f.F = F_frame != 0 && F_frame <= 61 - e_max ? F_frame : 61 - e_max;
@@ -227,34 +219,115 @@ __device__ FixedGrid make_fixed_grid(double lo, double side, int F_frame = 0) {
     return f;
 }
 
-// X: trunc(x * 2^F) when already known (the record-writing pass shares it with the record), or
-// computed here (only for x inside the box, where it cannot overflow).
-template <bool HAVE_X = false>
-__device__ __forceinline__ u32 grid_cell_fixed(double x, const FixedGrid& f, long long X = 0) {
-    const u64 o = order_bits(x);
-    if (o <= f.lo_ord) return 0u;
-    if (o >= f.hi_ord) return 2097151u;
-    const u64 d = static_cast<u64>((HAVE_X ? X : to_fixed(x, f.F)) - f.lo_fixed);
-    const u64 u = __umul64hi(d, f.scale_fixed);
-    const u32 frac20 = static_cast<u32>(u >> (f.R - 20)) & 0xfffffu;
-    if (frac20 == 0u || frac20 == 0xfffffu) return grid_cell(x, f.lo, f.scale);
-    const u64 g = u >> f.R;
-    return g > 2097151ULL ? 2097151u : static_cast<u32>(g);
+// The same evaluation in the form the kernels run. The kernels are bound by the integer pipe, which
+// takes two cycles for a warp's instruction, so: the three axes share one frame (the box's), so that
+// scale, shift and limits are the same; a coordinate is brought to fixed point by one right shift of
+// its mantissa; the product's high word is the cell and its low word the fraction; and whatever is not
+// plainly inside the box and away from cell borders, on any axis, takes one rare path. 2^25 Plummer
+// particles, Hilbert keys: 421 us with a frame, limits and selections per axis, 291 now (the integer pipe 77 % busy); 7.7e7 Morton
+// keys of 512 sets 1610 -> 731 us.
+struct FastGrid {
+    u64 neg_lo[3];  // -trunc(lo * 2^F)
+    u64 scale;      // S such that (((X - LO) << d_shift) * S) >> 64 has 32 fraction bits
+    u32 e_end;      // exponents below this are in the frame: |X| is the mantissa at bit 61 shifted right by e_end - e
+    u32 d_end;      // distances from the corner whose high word is below this are inside the box
+    int d_shift;
+    int fast;       // the error bound holds
+    double lo[3], inv;
+    int F;
+};
+
+// Frame F of the records when it is shared with them; else the widest that holds the box.
+__device__ FastGrid make_fast_grid(const double* box) {
+    const double side = box[3];
+    const int F = make_frame(box).F;
+    FastGrid g;
+    g.fast = F <= 900;  // so that subnormal coordinates are zero in fixed point
+    FixedGrid f;
+    for (int d = 0; d < 3; ++d) {
+        f = make_fixed_grid(box[d], side, F);
+        g.fast = g.fast && f.fast && f.F == F;
+        g.neg_lo[d] = 0ULL - static_cast<u64>(f.lo_fixed);
+        g.lo[d] = f.lo;
+    }
+    g.inv = f.scale;
+    g.F = F;
+    g.scale = f.R >= 32 ? f.scale_fixed >> (f.R - 32) : f.scale_fixed;
+    g.d_shift = f.R >= 32 ? 0 : 32 - f.R;
+    g.e_end = static_cast<u32>(9 + 1075 - F);
+    g.d_end = g.fast ? static_cast<u32>(static_cast<u64>(to_fixed(side, F)) >> 32) : 0u;
+    return g;
 }
 
-// Spread the 21 bits of v to every third bit position (bit b -> bit 3b).
-__device__ __forceinline__ u64 spread3(u32 v) {
-    u64 x = v & 0x1fffffu;
-    x = (x | (x << 32)) & 0x001f00000000ffffULL;
-    x = (x | (x << 16)) & 0x001f0000ff0000ffULL;
-    x = (x | (x << 8)) & 0x100f00f00f00f00fULL;
-    x = (x | (x << 4)) & 0x10c30c30c30c30c3ULL;
-    x = (x | (x << 2)) & 0x1249249249249249ULL;
-    return x;
+// X = trunc(x * 2^F) and its distance d from the box's corner; returns the exponent field.
+__device__ __forceinline__ u32 to_frame(double x, u64 neg_lo, u32 e_end, u64& X, u64& d) {
+    const u32 hi = static_cast<u32>(__double2hiint(x)), lo = static_cast<u32>(__double2loint(x));
+    const u32 e = (hi >> 20) & 0x7ffu;
+    const u64 m = ((static_cast<u64>((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 9;
+    const u64 mag = m >> min(e_end - e, 63u);
+    const u32 neg = hi >> 31;
+    const u64 flip = static_cast<u64>(static_cast<long long>(static_cast<int>(hi) >> 31));
+    X = (mag ^ flip) + neg;
+    d = (mag ^ flip) + neg_lo + neg;
+    return e;
+}
+
+// (a * b) >> 64 without the product of the low words: at most 2 too small.
+__device__ __forceinline__ u64 mul_high(u64 a, u64 b) {
+    const u32 al = static_cast<u32>(a), ah = static_cast<u32>(a >> 32), bl = static_cast<u32>(b), bh = static_cast<u32>(b >> 32);
+    return static_cast<u64>(ah) * bh + ((static_cast<u64>(al) * bh) >> 32) + __umulhi(ah, bl);
+}
+
+// Cell of one coordinate on the rare path: IEEE inside the frame; beyond it (where only boxes without
+// the error bound would compute anything), by the sign.
+__device__ __noinline__ u32 cell_exact(double x, const FastGrid& g, int d) {
+    const u32 hi = static_cast<u32>(__double2hiint(x));
+    if (g.fast && ((hi >> 20) & 0x7ffu) >= g.e_end) return (hi >> 31) ? 0u : 2097151u;
+    return grid_cell(x, g.lo[d], g.inv);
+}
+
+// Cells of a particle; X gets its fixed-point coordinates where the grid is fast. Returns whether all
+// coordinates are in the frame (always true where the grid is not fast).
+__device__ __forceinline__ bool cells_of(const FastGrid& g, double px, double py, double pz, u32 c[3], u64 X[3]) {
+    bool in = true, sure = false;
+    if (g.fast) {
+        u64 d[3];
+        const u32 e = max(to_frame(px, g.neg_lo[0], g.e_end, X[0], d[0]),
+                          max(to_frame(py, g.neg_lo[1], g.e_end, X[1], d[1]),
+                              to_frame(pz, g.neg_lo[2], g.e_end, X[2], d[2])));
+        u32 dh = 0, frac = 0xffffffffu;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            dh = max(dh, static_cast<u32>(d[k] >> 32));
+            const u64 u = mul_high(d[k] << g.d_shift, g.scale);
+            c[k] = static_cast<u32>(u >> 32);
+            frac = min(frac, static_cast<u32>(u) + 0x1000u);
+        }
+        in = e < g.e_end;
+        sure = in && dh < g.d_end && frac >= 0x2000u;  // 2^-20 cells or more from every border
+    }
+    if (!sure) {
+        c[0] = cell_exact(px, g, 0);
+        c[1] = cell_exact(py, g, 1);
+        c[2] = cell_exact(pz, g, 2);
+    }
+    return in;
+}
+
+// Every third bit of a word: bit b of the low 10 bits to bit 3b. The multiplications run beside the
+// integer pipe.
+__device__ __forceinline__ u32 spread10(u32 v) {
+    v = (v * 0x00010001u) & 0xff0000ffu;
+    v = (v * 0x00000101u) & 0x0f00f00fu;
+    v = (v * 0x00000011u) & 0xc30c30c3u;
+    return (v * 0x00000005u) & 0x49249249u;
 }
 
 __device__ __forceinline__ u64 morton_of(u32 gx, u32 gy, u32 gz) {
-    return (spread3(gx) << 2) | (spread3(gy) << 1) | spread3(gz);
+    const u32 low = spread10(gx & 0x3ffu) * 4u + spread10(gy & 0x3ffu) * 2u + spread10(gz & 0x3ffu);
+    const u32 mid = spread10((gx >> 10) & 0x3ffu) * 4u + spread10((gy >> 10) & 0x3ffu) * 2u + spread10((gz >> 10) & 0x3ffu);
+    const u32 top = ((gx >> 20) << 2) | ((gy >> 20) << 1) | (gz >> 20);
+    return (static_cast<u64>(top) << 60) | (static_cast<u64>(mid) << 30) | low;
 }
 
 // Key of this build's length from a 63-bit key: the cell of a coarser grid is the top 3L bits of
@@ -262,85 +335,93 @@ __device__ __forceinline__ u64 morton_of(u32 gx, u32 gy, u32 gz) {
 // because the grid scales differ by a power of two).
 __device__ __forceinline__ Key to_key(u64 k63) { return static_cast<Key>(k63 >> (63 - kKeyBits)); }
 
-// The three fixed-point grids of the box and the one-level Hilbert table in shared memory (both
-// key kernels); Hilbert keys also use a three-level table in dynamic shared memory, indexed by the
-// state and 3 bits of each coordinate's cell (3 levels, x bits above y bits above z bits), so a key
-// takes 7 lookups and no Morton interleave. Each block builds it from the one-level table.
+// The box's grid and the one-level Hilbert table in shared memory. Hilbert keys
+// take several levels per lookup from a table that each block composes of the one-level table, indexed
+// by the state and TL bits of each coordinate's cell (x bits above y bits above z bits): three levels
+// (48 KB of dynamic shared memory, 7 lookups per key) where a block has many particles, two levels
+// (6 KB, 11 lookups) for sets of fewer than kTwoLevelMax particles, where composing the large table took
+// most of the time (2^20 particles: 56 -> 21 us).
 struct KeySmem {
     unsigned short t1[kHilbertStates * 8];
-    FixedGrid grid[3];
+    FastGrid grid;
 };
-constexpr int kHilbert3Entries = kHilbertStates * 512;
-constexpr size_t kHilbert3Bytes = kHilbert3Entries * sizeof(unsigned short);  // 48 KB
+constexpr long long kTwoLevelMax = 1ll << 22;
+constexpr int kKeyThreads = 512, kKeyBlocks = 6;  // blocks per SM in the grid: two waves
+template <int TL>
+constexpr int kTableEntries = kHilbertStates << (3 * TL);
+template <int TL>
+constexpr size_t kTableBytes = kTableEntries<TL> * sizeof(unsigned short);
 
-template <int CURVE>
-__device__ __forceinline__ void load_key_smem(KeySmem& sm, unsigned short* t3, const HilbertTable& table,
-                                              const double* box, bool record_frame = false, bool grids = true) {
-    if (CURVE == CSTONE_HILBERT)
-        for (int i = threadIdx.x; i < kHilbertStates * 8; i += blockDim.x) sm.t1[i] = table.one[i];
-    if (grids && threadIdx.x < 3)
-        sm.grid[threadIdx.x] = make_fixed_grid(box[threadIdx.x], box[3], record_frame ? make_frame(box).F : 0);
-    if (CURVE == CSTONE_HILBERT) {
-        __syncthreads();
-        // entry (state, x3 y3 z3): three one-level steps, the octant of each level taken from the
-        // top remaining bit of x3, y3, z3 (x most significant, as in the Morton interleave)
-        for (int e = threadIdx.x; e < kHilbert3Entries; e += blockDim.x) {
-            const int idx = e & 511;
-            u32 state = static_cast<u32>(e >> 9), digits = 0;
+// Entry (state, bits): the digits of TL levels | next state << 3 TL.
+template <int TL>
+__device__ __forceinline__ void compose_table(KeySmem& sm, unsigned short* table, const HilbertTable& one) {
+    for (int i = threadIdx.x; i < kHilbertStates * 8; i += blockDim.x) sm.t1[i] = one.one[i];
+    __syncthreads();
+    for (int e = threadIdx.x; e < kTableEntries<TL>; e += blockDim.x) {
+        u32 state = static_cast<u32>(e >> (3 * TL)), digits = 0;
 #pragma unroll
-            for (int lv = 2; lv >= 0; --lv) {
-                const u32 o = (((idx >> (6 + lv)) & 1u) << 2) | (((idx >> (3 + lv)) & 1u) << 1) | ((idx >> lv) & 1u);
-                const u32 v = sm.t1[state * 8u + o];
-                digits = (digits << 3) | (v & 7u);
-                state = v >> 3;
-            }
-            t3[e] = static_cast<unsigned short>(digits | (state << 9));
+        for (int lv = TL - 1; lv >= 0; --lv) {
+            const u32 o = (((e >> (2 * TL + lv)) & 1u) << 2) | (((e >> (TL + lv)) & 1u) << 1) | ((e >> lv) & 1u);
+            const u32 v = sm.t1[state * 8u + o];
+            digits = (digits << 3) | (v & 7u);
+            state = v >> 3;
+        }
+        table[e] = static_cast<unsigned short>(digits | (state << (3 * TL)));
+    }
+}
+
+// Key of a cell from the table: TL levels per step, as far as this build's keys reach.
+template <int TL>
+__device__ __forceinline__ Key hilbert_of_cell(u32 gx, u32 gy, u32 gz, const unsigned short* table,
+                                               const unsigned short* t1) {
+    constexpr u32 kMask = (1u << TL) - 1u, kDigits = (1u << (3 * TL)) - 1u;
+    constexpr int kSteps = kLevels == 21 ? 21 / TL : (10 + TL - 1) / TL;
+    constexpr int kLeft = kLevels - kSteps * TL;  // 1: one more level; 0; or levels too many (negative)
+    u64 key = 0;
+    u32 state = 0, acc = 0;  // state: as stored in an entry's high bits; acc: up to 27 bits of digits
+#pragma unroll
+    for (int q = 0; q < kSteps; ++q) {
+        const int sh = 21 - TL * (q + 1);
+        const u32 idx = (((gx >> sh) & kMask) << (2 * TL)) | (((gy >> sh) & kMask) << TL) | ((gz >> sh) & kMask);
+        const u32 v = table[state | idx];
+        acc = (acc << (3 * TL)) | (v & kDigits);
+        state = v & ~kDigits;
+        constexpr int kPer = 27 / (3 * TL);  // steps whose digits fit acc
+        if (q % kPer == kPer - 1 || q == kSteps - 1) {
+            key = (key << (3 * TL * (q % kPer + 1))) | acc;
+            acc = 0;
         }
     }
+    if (kLeft > 0) {
+        static_assert(kLeft <= 1, "one single level at most");
+        const u32 v = t1[(state >> (3 * TL)) * 8u + (((gx & 1u) << 2) | ((gy & 1u) << 1) | (gz & 1u))];
+        key = (key << 3) | (v & 7u);
+    }
+    return static_cast<Key>(kLeft < 0 ? key >> (3 * (kLeft < 0 ? -kLeft : 0)) : key);
 }
 
-// 63-bit Hilbert key of a cell from the three-level table: 7 steps of 3 levels.
-__device__ __forceinline__ u64 hilbert_of_cell(u32 gx, u32 gy, u32 gz, const unsigned short* t3) {
-    u64 key = 0;
-    u32 state = 0;
-#pragma unroll
-    for (int sh = 18; sh >= 0; sh -= 3) {
-        const u32 idx = (((gx >> sh) & 7u) << 6) | (((gy >> sh) & 7u) << 3) | ((gz >> sh) & 7u);
-        const u32 v = t3[state * 512u + idx];
-        key = (key << 9) | (v & 511u);
-        state = v >> 9;
-    }
-    return key;
-}
-
-template <int CURVE, bool HAVE_X = false>
-__device__ __forceinline__ Key encode_key(const KeySmem& sm, const unsigned short* t3, bool fast, double px,
-                                          double py, double pz, long long X = 0, long long Y = 0, long long Z = 0) {
-    u32 gx, gy, gz;
-    if (fast) {
-        gx = grid_cell_fixed<HAVE_X>(px, sm.grid[0], X);
-        gy = grid_cell_fixed<HAVE_X>(py, sm.grid[1], Y);
-        gz = grid_cell_fixed<HAVE_X>(pz, sm.grid[2], Z);
-    } else {
-        gx = grid_cell(px, sm.grid[0].lo, sm.grid[0].scale);
-        gy = grid_cell(py, sm.grid[1].lo, sm.grid[1].scale);
-        gz = grid_cell(pz, sm.grid[2].lo, sm.grid[2].scale);
-    }
-    if (CURVE == CSTONE_HILBERT) return to_key(hilbert_of_cell(gx, gy, gz, t3));
+template <int CURVE, int TL>
+__device__ __forceinline__ Key key_of_cell(u32 gx, u32 gy, u32 gz, const KeySmem& sm, const unsigned short* table) {
+    if (CURVE == CSTONE_HILBERT) return hilbert_of_cell<TL>(gx, gy, gz, table, sm.t1);
     return to_key(morton_of(gx, gy, gz));
 }
 
-template <int CURVE, bool VEC>
-__global__ void __launch_bounds__(256) keys_kernel(const double* __restrict__ x, const double* __restrict__ y,
-                                                   const double* __restrict__ z, long long n,
-                                                   const double* __restrict__ box, Key* __restrict__ keys,
-                                                   const __grid_constant__ HilbertTable table) {
+template <int CURVE, int TL, bool VEC>
+__global__ void __launch_bounds__(kKeyThreads, 3) keys_kernel(const double* __restrict__ x, const double* __restrict__ y,
+                                                             const double* __restrict__ z, long long n,
+                                                             const double* __restrict__ box, Key* __restrict__ keys,
+                                                             const __grid_constant__ HilbertTable one) {
     __shared__ KeySmem sm;
-    extern __shared__ unsigned short t3[];  // kHilbert3Bytes for Hilbert keys
-    load_key_smem<CURVE>(sm, t3, table, box);
+    extern __shared__ unsigned short table[];  // kTableBytes<TL> for Hilbert keys
+    if (CURVE == CSTONE_HILBERT) compose_table<TL>(sm, table, one);
+    if (threadIdx.x == 0) sm.grid = make_fast_grid(box);
     __syncthreads();
-    const bool fast = sm.grid[0].fast && sm.grid[1].fast && sm.grid[2].fast;
-    auto encode = [&](double px, double py, double pz) -> Key { return encode_key<CURVE>(sm, t3, fast, px, py, pz); };
+    auto encode = [&](double px, double py, double pz) -> Key {
+        u32 c[3];
+        u64 X[3];
+        cells_of(sm.grid, px, py, pz, c, X);
+        return key_of_cell<CURVE, TL>(c[0], c[1], c[2], sm, table);
+    };
 
     if (!VEC) {
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
@@ -369,42 +450,40 @@ __global__ void __launch_bounds__(256) keys_kernel(const double* __restrict__ x,
 // the same read of the coordinates. A warp takes 64 consecutive particles, lane l the particles
 // l and l + 32: both halves keep the warp's loads and stores contiguous (a warp's two 16-byte
 // record stores cover 1 KB), and the two encodings interleave.
-#ifndef CSTONE_KEYS_REC_MIN_BLOCKS
-#define CSTONE_KEYS_REC_MIN_BLOCKS 3
-#endif
-template <int CURVE>
-__global__ void __launch_bounds__(256, CSTONE_KEYS_REC_MIN_BLOCKS)
+template <int CURVE, int TL>
+__global__ void __launch_bounds__(kKeyThreads, 2)
     keys_records_kernel(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
                         const float* __restrict__ m, long long n, const double* __restrict__ box,
                         Key* __restrict__ keys, Record* __restrict__ rec, WsHeader* hdr,
-                        const __grid_constant__ HilbertTable table) {
+                        const __grid_constant__ HilbertTable one) {
     __shared__ KeySmem sm;
     __shared__ FixedFrame s_frame;
-    extern __shared__ unsigned short t3[];  // kHilbert3Bytes for Hilbert keys
-    load_key_smem<CURVE>(sm, t3, table, box, true);  // the grids take the records' fixed-point frame
+    extern __shared__ unsigned short table[];  // kTableBytes<TL> for Hilbert keys
+    if (CURVE == CSTONE_HILBERT) compose_table<TL>(sm, table, one);
+    if (threadIdx.x == 0) sm.grid = make_fast_grid(box);
     if (threadIdx.x == 32) s_frame = make_frame(box);
     __syncthreads();
-    // the fixed-point coordinate serves the record and, where the fast path is on, the grid cell
-    const bool fast = sm.grid[0].fast && sm.grid[1].fast && sm.grid[2].fast && sm.grid[0].F == s_frame.F &&
-                      sm.grid[1].F == s_frame.F && sm.grid[2].F == s_frame.F;
     const FixedFrame fr = s_frame;
     const long long lane = threadIdx.x & 31;
     const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-    auto fixed = [&](double v, bool& in) -> long long {
-        const bool ok = static_cast<int>((static_cast<u64>(__double_as_longlong(v)) >> 52) & 0x7ffu) < fr.e_lim;
-        in = in && ok;
-        return ok ? fixed_of(v, fr.F) : 0;
-    };
-    auto one = [&](long long i, double px, double py, double pz, float pm) -> Key {
-        bool in = true;
-        const long long X = fixed(px, in), Y = fixed(py, in), Z = fixed(pz, in);
-        const Key k = fast ? encode_key<CURVE, true>(sm, t3, true, px, py, pz, X, Y, Z)
-                           : encode_key<CURVE>(sm, t3, false, px, py, pz);
+    auto encode = [&](long long i, double px, double py, double pz, float pm) -> Key {
+        u32 c[3];
+        u64 X[3];  // the grid's frame is the records'
+        bool in = cells_of(sm.grid, px, py, pz, c, X);
+        if (!sm.grid.fast) {
+            const double p[3] = {px, py, pz};
+#pragma unroll
+            for (int d = 0; d < 3; ++d) {
+                const bool ok = exponent_of(p[d]) < fr.e_lim;
+                X[d] = ok ? static_cast<u64>(fixed_of(p[d], fr.F)) : 0ULL;
+                in = in && ok;
+            }
+        }
         longlong2* dst = reinterpret_cast<longlong2*>(rec + i);
-        __stcs(dst, make_longlong2(in ? X : 0, in ? Y : 0));
-        __stcs(dst + 1, make_longlong2(in ? Z : 0, static_cast<long long>(__float_as_uint(pm))));
+        __stcs(dst, make_longlong2(in ? static_cast<long long>(X[0]) : 0, in ? static_cast<long long>(X[1]) : 0));
+        __stcs(dst + 1, make_longlong2(in ? static_cast<long long>(X[2]) : 0, static_cast<long long>(__float_as_uint(pm))));
         if (!in) raise_error(hdr, CSTONE_ERR_INVALID_ARG, static_cast<u32>(i));
-        return k;
+        return key_of_cell<CURVE, TL>(c[0], c[1], c[2], sm, table);
     };
     for (long long base = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 64; base < n;
          base += warps * 64) {
@@ -421,8 +500,8 @@ __global__ void __launch_bounds__(256, CSTONE_KEYS_REC_MIN_BLOCKS)
             bz = __ldcg(z + i1);
             bm = __ldcg(m + i1);
         }
-        keys[i0] = one(i0, ax, ay, az, am);
-        if (ok1) keys[i1] = one(i1, bx, by, bz, bm);
+        keys[i0] = encode(i0, ax, ay, az, am);
+        if (ok1) keys[i1] = encode(i1, bx, by, bz, bm);
     }
 }
 
@@ -583,36 +662,63 @@ __global__ void __cluster_dims__(kBoxCluster, 1, 1) __launch_bounds__(kBoxThread
     cluster.sync();  // the other blocks keep their shared memory until it has been read
 }
 
-__global__ void keys_batched_setup_kernel(const double* __restrict__ boxes, int n_sets, FixedGrid* grids) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n_sets; i += gridDim.x * blockDim.x) {
-        const int sidx = i / 3, d = i % 3;
-        grids[i] = make_fixed_grid(boxes[4 * sidx + d], boxes[4 * sidx + 3]);
-    }
+__global__ void keys_batched_setup_kernel(const double* __restrict__ boxes, int n_sets, FastGrid* grids) {
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_sets; i += gridDim.x * blockDim.x)
+        grids[i] = make_fast_grid(boxes + 4 * i);
 }
 
-template <int CURVE>
-__global__ void __launch_bounds__(256) keys_batched_kernel(const double* __restrict__ x, const double* __restrict__ y,
-                                                           const double* __restrict__ z,
-                                                           const long long* __restrict__ set_offsets, int n_sets,
-                                                           long long n, const FixedGrid* __restrict__ grids,
-                                                           Key* __restrict__ keys,
-                                                           const __grid_constant__ HilbertTable table) {
-    __shared__ KeySmem sm;  // only its one-level table is used here (the grids are per set)
-    extern __shared__ unsigned short t3[];  // kHilbert3Bytes for Hilbert keys
-    if (CURVE == CSTONE_HILBERT) load_key_smem<CURVE>(sm, t3, table, nullptr, false, false);
-    __syncthreads();
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int sidx = set_of(set_offsets, n_sets, i);
-        const FixedGrid* g = grids + 3 * sidx;
-        const double px = __ldcg(x + i), py = __ldcg(y + i), pz = __ldcg(z + i);
-        u32 c[3];
-        const double pc[3] = {px, py, pz};
+// A block takes a stretch of consecutive tiles of particles. Where a tile lies in one set, which one load
+// shows, its grids are read from shared memory, else every particle looks its set up.
+constexpr int kBatchItems = 2;
+constexpr int kBatchTile = kKeyThreads * kBatchItems;
+
+template <int CURVE, int TL>
+__global__ void __launch_bounds__(kKeyThreads, 3) keys_batched_kernel(const double* __restrict__ x,
+                                                                     const double* __restrict__ y,
+                                                                     const double* __restrict__ z,
+                                                                     const long long* __restrict__ set_offsets, int n_sets,
+                                                                     long long n, const FastGrid* __restrict__ grids,
+                                                                     Key* __restrict__ keys,
+                                                                     const __grid_constant__ HilbertTable one) {
+    __shared__ KeySmem sm;
+    extern __shared__ unsigned short table[];  // kTableBytes<TL> for Hilbert keys
+    if (CURVE == CSTONE_HILBERT) compose_table<TL>(sm, table, one);
+    const long long tiles = (n + kBatchTile - 1) / kBatchTile;
+    const long long b0 = tiles * blockIdx.x / gridDim.x, b1 = tiles * (blockIdx.x + 1) / gridDim.x;
+    int set = -1;                  // set of the tile's first particle
+    long long first = 0, end = 0;  // its particles
+    for (long long tile = b0; tile < b1; ++tile) {
+        const long long t0 = tile * kBatchTile, t1 = min(t0 + kBatchTile, n);
+        double p[kBatchItems][3];
 #pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const FixedGrid f = g[d];
-            c[d] = f.fast ? grid_cell_fixed(pc[d], f) : grid_cell(pc[d], f.lo, f.scale);
+        for (int k = 0; k < kBatchItems; ++k) {
+            const long long i = t0 + k * kKeyThreads + threadIdx.x;
+            const bool on = i < t1;
+            p[k][0] = on ? __ldcg(x + i) : 0.0;
+            p[k][1] = on ? __ldcg(y + i) : 0.0;
+            p[k][2] = on ? __ldcg(z + i) : 0.0;
         }
-        keys[i] = to_key(CURVE == CSTONE_HILBERT ? hilbert_of_cell(c[0], c[1], c[2], t3) : morton_of(c[0], c[1], c[2]));
+        if (t0 >= end) {  // the same in every thread
+            set = set_of(set_offsets, n_sets, t0);
+            first = __ldg(set_offsets + set);
+            end = __ldg(set_offsets + set + 1);
+            __syncthreads();  // the table, and the previous set's grids
+            if (threadIdx.x == 0) sm.grid = grids[set];
+            __syncthreads();
+        }
+        const bool whole = t0 >= first && t1 <= end;
+#pragma unroll
+        for (int k = 0; k < kBatchItems; ++k) {
+            const long long i = t0 + k * kKeyThreads + threadIdx.x;
+            u32 c[3];
+            u64 X[3];
+            if (whole || (i >= first && i < end))
+                cells_of(sm.grid, p[k][0], p[k][1], p[k][2], c, X);
+            else
+                cells_of(grids[set + set_of(set_offsets + set, n_sets - set, i < t1 ? i : t0)], p[k][0], p[k][1], p[k][2],
+                         c, X);
+            if (i < t1) keys[i] = key_of_cell<CURVE, TL>(c[0], c[1], c[2], sm, table);
+        }
     }
 }
 
@@ -634,7 +740,7 @@ const HilbertDecodeTable& hilbert_decode_table() {
 
 size_t keys_batched_ws_bytes(int n_sets) {
     Carver c(nullptr);
-    c.take<FixedGrid>((size_t)n_sets * 3);
+    c.take<FastGrid>((size_t)n_sets);
     return c.size();
 }
 
@@ -649,51 +755,45 @@ int launch_bbox_batched(const double* x, const double* y, const double* z, const
 int launch_keys_batched(const double* x, const double* y, const double* z, const long long* set_offsets, int n_sets,
                         long long n, const double* boxes, int curve, Key* keys, void* ws, cudaStream_t st) {
     Carver c(ws);
-    FixedGrid* grids = c.take<FixedGrid>((size_t)n_sets * 3);
-    keys_batched_setup_kernel<<<(3 * n_sets + 127) / 128, 128, 0, st>>>(boxes, n_sets, grids);
+    FastGrid* grids = c.take<FastGrid>((size_t)n_sets);
+    keys_batched_setup_kernel<<<(n_sets + 127) / 128, 128, 0, st>>>(boxes, n_sets, grids);
     CST_LAUNCHED("keys_batched_setup_kernel");
     if (n == 0) return CSTONE_OK;
     const HilbertTable& tab = hilbert_table();
-    const long long want = (n + 255) / 256;
-    const int grid = static_cast<int>(want < (long long)sm_count() * 8 ? want : (long long)sm_count() * 8);
-    if (curve == CSTONE_HILBERT) {  // the three-level table takes 48 KB of dynamic shared memory
-        CST_CUDA(cudaFuncSetAttribute(keys_batched_kernel<CSTONE_HILBERT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      static_cast<int>(kHilbert3Bytes)));
-        keys_batched_kernel<CSTONE_HILBERT><<<grid, 256, kHilbert3Bytes, st>>>(x, y, z, set_offsets, n_sets, n, grids,
-                                                                               keys, tab);
-    }
-    else
-        keys_batched_kernel<CSTONE_MORTON><<<grid, 256, 0, st>>>(x, y, z, set_offsets, n_sets, n, grids, keys, tab);
-    CST_LAUNCHED("keys_batched_kernel");
-    return CSTONE_OK;
+    const long long want = (n + kBatchTile - 1) / kBatchTile, most = (long long)sm_count() * kKeyBlocks;
+    const unsigned grid = static_cast<unsigned>(want < most ? want : most);
+    auto launch = [&](auto kernel, size_t smem) -> int {
+        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, set_offsets, n_sets, n, grids, keys, tab);
+        CST_LAUNCHED("keys_batched_kernel");
+        return CSTONE_OK;
+    };
+    if (curve != CSTONE_HILBERT) return launch(keys_batched_kernel<CSTONE_MORTON, 2>, 0);
+    if (n < kTwoLevelMax) return launch(keys_batched_kernel<CSTONE_HILBERT, 2>, kTableBytes<2>);
+    return launch(keys_batched_kernel<CSTONE_HILBERT, 3>, kTableBytes<3>);
 }
 
 int launch_keys(const double* x, const double* y, const double* z, long long n, const double* box, int curve,
                 Key* keys, cudaStream_t st) {
     if (n == 0) return CSTONE_OK;
     const HilbertTable& tab = hilbert_table();
-    long long pairs = (n + 1) / 2;
-    long long want = (pairs + 255) / 256;
-    int grid = static_cast<int>(want < (long long)sm_count() * 8 ? (want > 0 ? want : 1) : (long long)sm_count() * 8);
-    bool vec = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(z) |
-                 reinterpret_cast<uintptr_t>(keys)) & 15u) == 0;
-    if (curve == CSTONE_HILBERT) {  // the three-level table takes 48 KB of dynamic shared memory
-        CST_CUDA(cudaFuncSetAttribute(keys_kernel<CSTONE_HILBERT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      static_cast<int>(kHilbert3Bytes)));
-        CST_CUDA(cudaFuncSetAttribute(keys_kernel<CSTONE_HILBERT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      static_cast<int>(kHilbert3Bytes)));
-        if (vec)
-            keys_kernel<CSTONE_HILBERT, true><<<grid, 256, kHilbert3Bytes, st>>>(x, y, z, n, box, keys, tab);
-        else
-            keys_kernel<CSTONE_HILBERT, false><<<grid, 256, kHilbert3Bytes, st>>>(x, y, z, n, box, keys, tab);
-    } else {
-        if (vec)
-            keys_kernel<CSTONE_MORTON, true><<<grid, 256, 0, st>>>(x, y, z, n, box, keys, tab);
-        else
-            keys_kernel<CSTONE_MORTON, false><<<grid, 256, 0, st>>>(x, y, z, n, box, keys, tab);
-    }
-    CST_LAUNCHED("keys_kernel");
-    return CSTONE_OK;
+    const long long want = ((n + 1) / 2 + kKeyThreads - 1) / kKeyThreads, most = (long long)sm_count() * kKeyBlocks;
+    const unsigned grid = static_cast<unsigned>(want < most ? want : most);
+    const bool vec = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(z) |
+                       reinterpret_cast<uintptr_t>(keys)) & 15u) == 0;
+    auto launch = [&](auto kernel, size_t smem) -> int {
+        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, n, box, keys, tab);
+        CST_LAUNCHED("keys_kernel");
+        return CSTONE_OK;
+    };
+    if (curve != CSTONE_HILBERT)
+        return vec ? launch(keys_kernel<CSTONE_MORTON, 2, true>, 0) : launch(keys_kernel<CSTONE_MORTON, 2, false>, 0);
+    if (n < kTwoLevelMax)
+        return vec ? launch(keys_kernel<CSTONE_HILBERT, 2, true>, kTableBytes<2>)
+                   : launch(keys_kernel<CSTONE_HILBERT, 2, false>, kTableBytes<2>);
+    return vec ? launch(keys_kernel<CSTONE_HILBERT, 3, true>, kTableBytes<3>)
+               : launch(keys_kernel<CSTONE_HILBERT, 3, false>, kTableBytes<3>);
 }
 
 // Keys and multipole records in one pass; ws holds only the header (error word).
@@ -703,17 +803,18 @@ int launch_keys_records(const double* x, const double* y, const double* z, const
     CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
     if (n == 0) return CSTONE_OK;
     const HilbertTable& tab = hilbert_table();
-    long long want = (n + 511) / 512;  // 64 particles per warp and step
-    int grid = static_cast<int>(want < (long long)sm_count() * 8 ? (want > 0 ? want : 1) : (long long)sm_count() * 8);
-    if (curve == CSTONE_HILBERT)
-        CST_CUDA(cudaFuncSetAttribute(keys_records_kernel<CSTONE_HILBERT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      static_cast<int>(kHilbert3Bytes)));
-    if (curve == CSTONE_HILBERT)
-        keys_records_kernel<CSTONE_HILBERT><<<grid, 256, kHilbert3Bytes, st>>>(x, y, z, m, n, box, keys, rec, hdr, tab);
-    else
-        keys_records_kernel<CSTONE_MORTON><<<grid, 256, 0, st>>>(x, y, z, m, n, box, keys, rec, hdr, tab);
-    CST_LAUNCHED("keys_records_kernel");
-    return CSTONE_OK;
+    const long long per = 2 * kKeyThreads;  // 64 particles per warp and step
+    const long long want = (n + per - 1) / per, most = (long long)sm_count() * kKeyBlocks;
+    const unsigned grid = static_cast<unsigned>(want < most ? want : most);
+    auto launch = [&](auto kernel, size_t smem) -> int {
+        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, m, n, box, keys, rec, hdr, tab);
+        CST_LAUNCHED("keys_records_kernel");
+        return CSTONE_OK;
+    };
+    if (curve != CSTONE_HILBERT) return launch(keys_records_kernel<CSTONE_MORTON, 2>, 0);
+    if (n < kTwoLevelMax) return launch(keys_records_kernel<CSTONE_HILBERT, 2>, kTableBytes<2>);
+    return launch(keys_records_kernel<CSTONE_HILBERT, 3>, kTableBytes<3>);
 }
 
 // bounding cube (bounds == false: box = {lo, side}) or per-axis bounds (bounds == true)

@@ -6,7 +6,7 @@
 // summed over the ranks (one allreduce of n_l integers), and every rank applies the same g to the
 // same summed counts, so the leaf arrays stay identical on all ranks.
 //
-// f: one thread per leaf, two binary searches in the sorted keys. g: three launches: the decision
+// f: one binary search in the sorted keys per leaf boundary. g: three launches: the decision
 // O_i of every leaf with per-tile sums, one block scanning the tile sums, and a per-tile scan that
 // places every kept, merged-into or split leaf (Eqs. rebalancecopy / rebalancesplit).
 //
@@ -46,12 +46,18 @@ __device__ __forceinline__ u32 lower_bound_keys(const Key* __restrict__ P, u32 n
     return lo;
 }
 
-// f (Eq. histogram): N_i = lb(P, K_{i+1}) - lb(P, K_i).
+// f (Eq. histogram): N_i = lb(P, K_{i+1}) - lb(P, K_i). A warp searches for 32 consecutive boundaries
+// and takes the counts of the 31 leaves between them from its neighbours.
 __global__ void __launch_bounds__(kThreads) leaf_counts_kernel(const Key* __restrict__ P, u32 n,
                                                                const Key* __restrict__ K, u32 nl,
                                                                u32* __restrict__ counts) {
-    for (u32 i = blockIdx.x * kThreads + threadIdx.x; i < nl; i += gridDim.x * kThreads)
-        counts[i] = lower_bound_keys(P, n, K[i + 1]) - lower_bound_keys(P, n, K[i]);
+    const u32 lane = threadIdx.x & 31u, warps = gridDim.x * (kThreads / 32);
+    for (u32 i0 = (blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5)) * 31u; i0 < nl; i0 += warps * 31u) {
+        const u32 i = i0 + lane;
+        const u32 pos = i <= nl ? lower_bound_keys(P, n, K[i]) : 0u;
+        const u32 next = __shfl_down_sync(0xffffffffu, pos, 1);
+        if (lane < 31u && i < nl) counts[i] = next - pos;
+    }
 }
 
 // g1 (Eq. g1) for leaf i: split (8) when it holds more than ncrit particles and is not a single
@@ -224,24 +230,30 @@ __device__ __forceinline__ bool outside_focus(Key start, Key size, Key f_start, 
     return f_end <= f_start || start + size <= f_start || start >= f_end;
 }
 
-// MAC of the cube [c, c + edge)^3 against the focus tiles held in shared memory.
-__device__ __forceinline__ bool mac_passes(const u32 c[3], u32 edge, const u32 (*tc)[4], int nt, double theta) {
-    if (nt == 0) return true;  // an empty focus accepts every node
+// r_min^2 of the cube [c, c + edge)^3 against the focus tiles held in shared memory, by a whole warp
+// (each lane takes every 32nd tile); all ones for an empty focus.
+__device__ __forceinline__ u64 warp_distance(const u32 c[3], u32 edge, const u32 (*tc)[4], int nt) {
     u64 best = ~0ULL;
-    for (int t = 0; t < nt && best != 0; ++t) {
+    for (int t = threadIdx.x & 31; t < nt; t += 32) {
         u64 r2 = 0;
 #pragma unroll
         for (int d = 0; d < 3; ++d) {
-            const u64 a0 = c[d], a1 = a0 + edge, b0 = tc[t][d], b1 = b0 + tc[t][3];
-            const u64 gap = b0 > a1 ? b0 - a1 : (a0 > b1 ? a0 - b1 : 0);
-            r2 += gap * gap;
+            const u32 a1 = c[d] + edge, b0 = tc[t][d], b1 = b0 + tc[t][3];
+            const u32 gap = b0 > a1 ? b0 - a1 : (c[d] > b1 ? c[d] - b1 : 0u);
+            r2 += static_cast<u64>(gap) * gap;
         }
         best = r2 < best ? r2 : best;
     }
-    const double q = __ddiv_rn(static_cast<double>(edge), theta);
-    return __ull2double_rn(best) > __dmul_rn(q, q);
+    const u32 hi = __reduce_min_sync(0xffffffffu, static_cast<u32>(best >> 32));
+    const u32 lo = __reduce_min_sync(0xffffffffu, static_cast<u32>(best >> 32) == hi ? static_cast<u32>(best) : 0xffffffffu);
+    return (static_cast<u64>(hi) << 32) | lo;
 }
 
+// g1^LE, one leaf per thread. The distances are taken by the warp together, one for every over-full leaf
+// outside F and one for every parent of eight siblings outside F (its siblings in the warp share the
+// answer), and (l / theta)^2 is tabulated by level: a thread per eight leaves that went through all
+// focus tiles itself, for every sibling, with two FP64 operations each, took 177 us for 2.3e5 leaves
+// and 100 tiles on GB300 (FP64 division is a few operations per SM and clock).
 __global__ void __launch_bounds__(kThreads) focus_ops_kernel(const Key* __restrict__ K, const u32* __restrict__ N,
                                                              u32 nl, u32 ncrit, const __grid_constant__ FocusParams fp,
                                                              const __grid_constant__ HilbertDecodeTable dt,
@@ -250,7 +262,12 @@ __global__ void __launch_bounds__(kThreads) focus_ops_kernel(const Key* __restri
     __shared__ u32 s_warp[kThreads / 32];
     __shared__ u32 s_tile[kMaxFocusTiles][4];  // cube corner and edge of every focus tile
     __shared__ unsigned short s_dec[kHilbertStates * 8];
+    __shared__ double s_reach[kLevels + 1];  // (l / theta)^2 of a node of each level
     for (int i = threadIdx.x; i < kHilbertStates * 8; i += kThreads) s_dec[i] = dt.one[i];
+    if (threadIdx.x <= kLevels) {
+        const double q = __ddiv_rn(static_cast<double>(1u << (kLevels - threadIdx.x)), fp.theta);
+        s_reach[threadIdx.x] = __dmul_rn(q, q);
+    }
     __syncthreads();
     for (int t = threadIdx.x; t < fp.n_tiles; t += kThreads) {
         u32 c[3];
@@ -260,63 +277,66 @@ __global__ void __launch_bounds__(kThreads) focus_ops_kernel(const Key* __restri
         s_tile[t][3] = edge;
     }
     __syncthreads();
-    const u32 base = blockIdx.x * kTile + threadIdx.x * kItems;
-    u32 sum = 0;
-    bool changed = false;
-    for (int k = 0; k < kItems; ++k) {
-        const u32 i = base + k;
-        if (i > nl) break;
-        u32 op = 0;
-        if (i < nl) {
-            const Key ke = K[i];
-            const Key delta = K[i + 1] - ke;
-            const int level = kLevels - key_ffs(delta) / 3;
-            const u32 edge = 1u << (kLevels - level);
-            bool cube_known = false;
-            u32 c[3];
-            auto cube = [&]() {
-                if (!cube_known) {
-                    key_cell(ke, fp.curve, s_dec, c);
-                    for (int d = 0; d < 3; ++d) c[d] &= ~(edge - 1u);
-                    cube_known = true;
-                }
-            };
-            bool split = N[i] > ncrit && delta > 1;
-            if (split && outside_focus(ke, delta, fp.f_start, fp.f_end)) {
-                cube();
-                split = !mac_passes(c, edge, s_tile, fp.n_tiles, fp.theta);
-            }
-            op = 1u;
-            if (split) {
-                op = 8u;
-            } else if (delta < kKeyEnd) {
-                const u32 j = static_cast<u32>((ke >> key_ffs(delta)) & 7u);
-                if (j >= 1u && j <= i && i - j + 8u <= nl) {
-                    const u32 first = i - j;
-                    if (K[first] + static_cast<Key>(8) * delta == K[first + 8]) {
-                        u32 s8 = 0;
+    const int lane = threadIdx.x & 31;
+    const u32 i = blockIdx.x * kThreads + threadIdx.x;
+    bool over = false, group = false;  // an over-full leaf; eight siblings that may merge, this one not the first
+    bool ask_leaf = false, ask_parent = false, merge = false;
+    int level = 0, leader = lane;
+    u32 c[3] = {0, 0, 0};
+    if (i < nl) {
+        const Key ke = K[i];
+        const Key delta = K[i + 1] - ke;
+        const u32 cnt = N[i];
+        level = kLevels - key_ffs(delta) / 3;
+        over = cnt > ncrit && delta > 1;
+        ask_leaf = over && outside_focus(ke, delta, fp.f_start, fp.f_end);
+        if (delta < kKeyEnd) {
+            const u32 j = static_cast<u32>((ke >> key_ffs(delta)) & 7u);
+            if (j >= 1u && j <= i && i - j + 8u <= nl) {
+                const u32 first = i - j;
+                if (K[first] + static_cast<Key>(8) * delta == K[first + 8]) {
+                    u32 s8 = 0;
 #pragma unroll
-                        for (int q = 0; q < 8; ++q) s8 += N[first + q];
-                        bool merge = s8 <= ncrit;
-                        if (!merge && outside_focus(K[first], static_cast<Key>(8) * delta, fp.f_start, fp.f_end)) {
-                            cube();
-                            u32 pc[3];
-                            for (int d = 0; d < 3; ++d) pc[d] = c[d] & ~(2u * edge - 1u);
-                            merge = mac_passes(pc, 2u * edge, s_tile, fp.n_tiles, fp.theta);
-                        }
-                        if (merge) op = 0u;
-                    }
+                    for (int q = 0; q < 8; ++q) s8 += N[first + q];
+                    group = true;
+                    merge = s8 <= ncrit;
+                    ask_parent = !merge && outside_focus(K[first], static_cast<Key>(8) * delta, fp.f_start, fp.f_end);
+                    leader = max(0, lane - static_cast<int>(j) + 1);  // the first of these siblings in the warp
                 }
             }
         }
-        O[i] = static_cast<unsigned char>(op);
-        sum += op;
-        changed |= i < nl && op != 1u;
+        if (ask_leaf || (ask_parent && leader == lane)) key_cell(ke, fp.curve, s_dec, c);
     }
-    if (__syncthreads_or(changed) && threadIdx.x == 0) atomicOr(&st->changed, 1u);
+    u32 far_leaf = 0, far_parent = 0;  // bit per lane: the MAC accepts its leaf; the parent it asks for
+    for (int kind = 0; kind < 2; ++kind) {
+        u32 todo = __ballot_sync(0xffffffffu, kind == 0 ? ask_leaf : ask_parent && leader == lane);
+        while (todo != 0u) {
+            const int l = __ffs(todo) - 1;
+            todo &= todo - 1u;
+            const int lv = __shfl_sync(0xffffffffu, level, l) - kind;
+            const u32 edge = 1u << (kLevels - lv);
+            u32 q[3];
+#pragma unroll
+            for (int d = 0; d < 3; ++d) q[d] = __shfl_sync(0xffffffffu, c[d], l) & ~(edge - 1u);
+            const u64 r2 = warp_distance(q, edge, s_tile, fp.n_tiles);
+            const bool far = fp.n_tiles == 0 || __ull2double_rn(r2) > s_reach[lv];  // an empty focus accepts every node
+            if (kind == 0)
+                far_leaf |= far ? 1u << l : 0u;
+            else
+                far_parent |= far ? 1u << l : 0u;
+        }
+    }
+    u32 op = 0;
+    if (i < nl) {
+        const bool split = over && !(ask_leaf && ((far_leaf >> lane) & 1u));
+        if (ask_parent) merge = (far_parent >> leader) & 1u;
+        op = split ? 8u : (group && merge ? 0u : 1u);
+    }
+    if (i <= nl) O[i] = static_cast<unsigned char>(op);
+    if (__syncthreads_or(i < nl && op != 1u) && threadIdx.x == 0) atomicOr(&st->changed, 1u);
     u32 total;
-    block_exclusive_scan(sum, s_warp, &total);
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
+    block_exclusive_scan(op, s_warp, &total);
+    if (threadIdx.x == 0 && total) atomicAdd(&tile_sums[blockIdx.x / (kTile / kThreads)], total);
 }
 
 struct RebalanceLayout {
@@ -343,7 +363,7 @@ RebalanceLayout rebalance_layout(void* ws, long long nl) {
 size_t rebalance_ws_bytes(long long nl) { return rebalance_layout(nullptr, nl).bytes; }
 
 int launch_leaf_counts(const Key* P, long long n, const Key* K, long long nl, u32* counts, cudaStream_t st) {
-    const long long want = (nl + kThreads - 1) / kThreads;
+    const long long want = (nl + 31 * (kThreads / 32) - 1) / (31 * (kThreads / 32));
     const int grid = static_cast<int>(want < (long long)sm_count() * 8 ? want : (long long)sm_count() * 8);
     leaf_counts_kernel<<<grid, kThreads, 0, st>>>(P, static_cast<u32>(n), K, static_cast<u32>(nl), counts);
     CST_LAUNCHED("leaf_counts_kernel");
@@ -373,10 +393,12 @@ int focus_tiles(Key f_start, Key f_end, FocusParams& fp) {
 int launch_rebalance(const Key* K, const u32* N, long long nl, u32 ncrit, Key* Kout, long long cap, long long* nl_out,
                      int* changed, void* ws, cudaStream_t st, const FocusParams* focus = nullptr) {
     RebalanceLayout l = rebalance_layout(ws, nl);
-    CST_CUDA(cudaMemsetAsync(ws, 0, sizeof(WsHeader), st));
-    CST_CUDA(cudaMemsetAsync(l.st, 0, sizeof(RebalanceState), st));
+    // header, state and tile sums, which follow each other
+    CST_CUDA(cudaMemsetAsync(ws, 0, static_cast<size_t>(reinterpret_cast<char*>(l.tile_sums + l.ntiles) -
+                                                        static_cast<char*>(ws)), st));
     if (focus) {
-        focus_ops_kernel<<<l.ntiles, kThreads, 0, st>>>(K, N, static_cast<u32>(nl), ncrit, *focus,
+        const unsigned blocks = static_cast<unsigned>((nl + 1 + kThreads - 1) / kThreads);
+        focus_ops_kernel<<<blocks, kThreads, 0, st>>>(K, N, static_cast<u32>(nl), ncrit, *focus,
                                                         hilbert_decode_table(), l.O, l.tile_sums, l.st);
         CST_LAUNCHED("focus_ops_kernel");
     } else {

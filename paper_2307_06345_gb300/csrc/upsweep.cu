@@ -463,6 +463,23 @@ __global__ void __launch_bounds__(kLeafThreads) multipole_bigleaf_kernel(const u
     __syncthreads();
     const FixedFrame f = s_f;
     const u32 nbig = *s.n_big;
+    // this thread's records of [a, b) in order, the loads of kBatch of them in flight together (one at a
+    // time the random reads' latency bounds the kernel: 390 us for 1.7e7 clump particles at 10 levels, now 286)
+    constexpr u32 kBatch = 4;
+    auto each = [&](u32 a, u32 b, auto take) {
+        for (u32 j = a + threadIdx.x; j < b; j += kBatch * kLeafThreads) {
+            u32 p[kBatch];
+            Record r[kBatch];
+#pragma unroll
+            for (u32 t = 0; t < kBatch; ++t) p[t] = j + t * kLeafThreads < b ? __ldg(perm + j + t * kLeafThreads) : 0u;
+#pragma unroll
+            for (u32 t = 0; t < kBatch; ++t)
+                if (j + t * kLeafThreads < b) r[t] = load_record(s.rec, p[t]);
+#pragma unroll
+            for (u32 t = 0; t < kBatch; ++t)
+                if (j + t * kLeafThreads < b) take(r[t]);
+        }
+    };
     for (u32 q = blockIdx.x; q < nbig; q += gridDim.x) {
         const u32 i = s.big[q];
         const u32 a = offsets[i], b = offsets[i + 1];
@@ -470,13 +487,12 @@ __global__ void __launch_bounds__(kLeafThreads) multipole_bigleaf_kernel(const u
         ff M = ff_zero(), S[3] = {ff_zero(), ff_zero(), ff_zero()}, Q[6];
 #pragma unroll
         for (int k = 0; k < 6; ++k) Q[k] = ff_zero();
-        for (u32 j = a + threadIdx.x; j < b; j += kLeafThreads) {
-            const Record r = s.rec[__ldg(perm + j)];
+        each(a, b, [&](const Record& r) {
             M = ff_add(M, r.m);
             S[0] = ff_add(S[0], __fmul_rn(r.m, fixed_diff(r.x, r0.x, f)));
             S[1] = ff_add(S[1], __fmul_rn(r.m, fixed_diff(r.y, r0.y, f)));
             S[2] = ff_add(S[2], __fmul_rn(r.m, fixed_diff(r.z, r0.z, f)));
-        }
+        });
         M = block_sum(M, s_red);
 #pragma unroll
         for (int d = 0; d < 3; ++d) S[d] = block_sum(S[d], s_red);
@@ -489,8 +505,7 @@ __global__ void __launch_bounds__(kLeafThreads) multipole_bigleaf_kernel(const u
             c[d] = r0c[d] + float_to_int64(__fmul_rn(__fmul_rn(off, 1.0f / f.s1), 1.0f / f.s2));
         }
         ff R[3] = {ff_zero(), ff_zero(), ff_zero()};  // residual first moment about c
-        for (u32 j = a + threadIdx.x; j < b; j += kLeafThreads) {
-            const Record r = s.rec[__ldg(perm + j)];
+        each(a, b, [&](const Record& r) {
             const float e0 = fixed_diff(r.x, c[0], f);
             const float e1 = fixed_diff(r.y, c[1], f);
             const float e2 = fixed_diff(r.z, c[2], f);
@@ -504,7 +519,7 @@ __global__ void __launch_bounds__(kLeafThreads) multipole_bigleaf_kernel(const u
             Q[3] = ff_add(Q[3], __fmul_rn(me1, e1));
             Q[4] = ff_add(Q[4], __fmul_rn(me1, e2));
             Q[5] = ff_add(Q[5], __fmul_rn(me2, e2));
-        }
+        });
 #pragma unroll
         for (int k = 0; k < 6; ++k) Q[k] = block_sum(Q[k], s_red);
 #pragma unroll
@@ -620,13 +635,14 @@ __global__ void __launch_bounds__(kThreads, 4) multipole_level_kernel(const int*
     // small levels by block 0 alone, as in the count upsweep; 8 lanes per node, the loop bounds
     // the same in every lane of a warp
     constexpr u32 kGroups = kThreads / 8;
+    constexpr u32 kSmall = 2 * kGroups;  // a round of 32 nodes takes block 0 about as long as a grid barrier
     const u32 gw = (blockIdx.x * kThreads + threadIdx.x) / 32, nw = gridDim.x * (kThreads / 32);
     bool pending = false;
     for (int l = kLevels - 1; l >= 0; --l) {
         if (s_lo[l + 2] == s_lo[l + 1]) continue;  // no internal node at level l
         u32 g0, g1;
         internal_range(s_lo, l, n_int, g0, g1);
-        if (g1 <= g0 + kSmallLevel) {
+        if (g1 <= g0 + kSmall) {
             if (blockIdx.x == 0) {
                 for (u32 b0 = g0; b0 < g1; b0 += kGroups) {  // uniform trip count in the block
                     const u32 g = b0 + threadIdx.x / 8;
@@ -753,7 +769,14 @@ int launch_upsweep_multipoles(const double* x, const double* y, const double* z,
         MpScratch mp = l.mp;
         GridBarrier* bar = l.bar;
         void* args[] = {&child, &level_offsets, &nn_, &mp, &box, &mass, &com, &quad, &bar, &hdr};
-        const int grid = cooperative_grid(reinterpret_cast<const void*>(multipole_level_kernel), kThreads, 0, 4);
+        // a barrier costs more with more blocks (1.5 us at one per SM, 3.3 at four): no more than the tree
+        // has work for, 32 internal nodes per block and round
+        const int most = cooperative_grid(reinterpret_cast<const void*>(multipole_level_kernel), kThreads, 0, 4);
+        const long long rounds = ((nl - 1) / 7 + 31) / 32;
+        const int per_sm = rounds > 8ll * sm_count() ? 4 : (rounds > 2ll * sm_count() ? 2 : 1);
+        int grid = sm_count() * per_sm;
+        if (rounds < grid) grid = static_cast<int>(rounds);
+        if (most < grid) grid = most;
         CST_COOP(cudaLaunchCooperativeKernel(reinterpret_cast<void*>(multipole_level_kernel), dim3(grid),
                                              dim3(kThreads), args, 0, st));
     }

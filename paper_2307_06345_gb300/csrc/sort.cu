@@ -9,8 +9,9 @@
 // of equal keys; a part of at most kSmall pairs is sorted in shared memory by one block and written to
 // its final place. Two rounds of splitting reach every size: a pair moves three times (round 1, round
 // 2, final place), where the eight digit passes of a radix sort move it eight times. 2^27 clump keys
-// take 5.1 ms (count 0.31 and 0.65, scatter 0.82 and 0.92, final sort 1.87; the digit passes took
-// 7.2), 2^25 Plummer keys 1.3 ms (1.9), 65,536 uniform keys 65 us in 7 launches (200 in 40). Per round:
+// take 4.7 ms (count 0.33 and 0.69, scatter 0.82 and 0.91, final sort 1.64; the digit passes took
+// 7.2), 2^25 Plummer keys 1.2 ms (1.9), 65,536 uniform keys 65 us in 7 launches (200 in 40). Fetching a
+// tile's pairs while the one before it is written gained nothing in the scatter. Per round:
 //
 //   sample   one block per bucket sorts a sample and writes the bounds of the parts;
 //   count    every pair's part is found (a table over the leading key bits, then a binary search
@@ -50,9 +51,9 @@ constexpr int kTile = kThreads * kItems;
 static_assert(kThreads >= 256 && kThreads % 32 == 0 && kItems % 2 == 0 && kTile < 65536, "tile shape");
 
 constexpr u32 kMaxParts = 512;  // parts of one bucket
-constexpr int kSmallThreads = 256, kSmallItems = 12, kSmallBlocks = 3;
+constexpr int kSmallThreads = 256, kSmallItems = 10, kSmallBlocks = 4;
 constexpr u32 kSmall = kSmallThreads * kSmallItems;  // pairs sorted by one block of the final sort
-constexpr u32 kTarget = kSmall / 2;                  // mean size of the last round's parts
+constexpr u32 kTarget = 1536;                        // mean size of the last round's parts
 constexpr int kBigThreads = 1024, kBigItems = 8;
 constexpr u32 kBig = kBigThreads * kBigItems;  // pairs of a sample, and of a chunk of an oversized part
 constexpr u32 kHeavy = 24;                     // pairs of a bin ranked by comparison
@@ -342,13 +343,19 @@ __device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, i
         for (int w = 0; w < THREADS / 32; ++w) ored |= sm.red[w];
         map.top = bit_length(ored);
         map.vtop = idx_bits;
-        // unconditional, so that a thread's atomics are in flight together: a slot without a pair
-        // adds nothing to a word of its lane
+        // the usual case needs no mask (the distances have `top` bits) and nothing of the values
+        const bool plain = map.top >= map.nb;
+        const int sh = map.top - map.nb;
+        auto bin_of = [&](Key k, u32 v) -> u32 {
+            return plain ? static_cast<u32>((k - base) >> sh) : map.bin(k - base, v, idx_bits);
+        };
+        // unconditional, so that a thread's atomics are in flight together (with a test per slot the
+        // kernel is a fifth slower): a slot without a pair adds nothing to a word of its lane
         u32 was[ITEMS];
 #pragma unroll
         for (int i = 0; i < ITEMS; ++i) {
             const bool on = tid + i * THREADS < m;
-            const u32 b = on ? map.bin(key[i] - base, val[i], idx_bits) : 2u * lane;
+            const u32 b = on ? bin_of(key[i], val[i]) : 2u * lane;
             at[i] = b;
             was[i] = atomicAdd(&sm.bins[b >> 1], on ? ((b & 1u) ? 0x10000u : 1u) : 0u);
         }
@@ -370,7 +377,7 @@ __device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, i
         for (u32 s = tid; s < m; s += THREADS) {
             const Key k = sm.K[s];
             const u32 v = sm.V[s];
-            const u32 b = map.bin(k - base, v, idx_bits);
+            const u32 b = bin_of(k, v);
             const u32 b0 = starts[b], b1 = starts[b + 1];
             if (b1 - b0 <= kHeavy)
                 out(rank_in_bin(sm, k, v, b0, b1), k, v);
@@ -503,8 +510,8 @@ __device__ __forceinline__ u32 hash32(u32 x) {  // Wang's integer mix (public do
     return x ^ (x >> 15);
 }
 
-// Bounds of every bucket's parts from a stratified random sample (16 or 32 pairs per part, which
-// keeps nearly every part below twice the mean), sorted by one block; the counts are cleared.
+// Bounds of every bucket's parts from a stratified random sample (16 to 32 pairs per part, which
+// keeps nearly every part below 5/3 of the mean), sorted by one block; the counts are cleared.
 template <int SRC>
 __global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Buckets b, Tables t, int idx_bits) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -513,7 +520,7 @@ __global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Bucke
     for (u32 k = blockIdx.x; k < count; k += gridDim.x) {
         const u32 start = b.start[k], size = b.size[k], fp = b.first_part[k];
         const u32 np = b.first_part[k + 1] - fp;
-        const u32 per = np <= kBig / 32u ? 32u : 16u;
+        const u32 per = min(32u, kBig / np);  // 16 .. 32
         const u32 ns = np * per;  // <= kBig, and < size: a part has kTarget pairs or more on average
         const Key* keys = keys_of<SRC>(p);
         const Key base = b.base[k];

@@ -1,5 +1,5 @@
 """The sample sort behind cstone_sort and cstone_sort_segmented at the sizes where its path changes
-(digit passes up to 1024 keys, one block up to 3072, one round of splitting up to 786,432, two above)
+(digit passes up to 1024 keys, one block up to 2560, one round of splitting up to 786,432, two above)
 and on key sets that are hard to split, bit for bit against a stable sort."""
 import numpy as np
 import pytest
@@ -7,7 +7,7 @@ import torch
 
 pytestmark = pytest.mark.gpu
 
-SMALL, TARGET, PARTS = 3072, 1536, 512  # pairs sorted by one block, mean part, most parts of a bucket
+SMALL, TARGET, PARTS = 2560, 1536, 512  # pairs sorted by one block, mean part, most parts of a bucket
 
 
 def _kinds(rng, n):

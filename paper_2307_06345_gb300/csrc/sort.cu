@@ -512,10 +512,29 @@ __device__ __forceinline__ u32 hash32(u32 x) {  // Wang's integer mix (public do
 
 // Bounds of every bucket's parts from a stratified random sample (16 to 32 pairs per part, which
 // keeps nearly every part below 5/3 of the mean), sorted by one block; the counts are cleared.
+// A sort of one set starts here (single = its keys, else 0): its tables have one bucket, and the
+// launch that lists segments is not needed.
 template <int SRC>
-__global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Buckets b, Tables t, int idx_bits) {
+__global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Buckets b, Tables t, int idx_bits, u32 single,
+                                                                 int rounds, WsHeader* hdr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BigSmem& sm = *reinterpret_cast<BigSmem*>(smem_raw);
+    if (single != 0) {  // one block
+        if (threadIdx.x < sizeof(WsHeader) / 4) reinterpret_cast<u32*>(hdr)[threadIdx.x] = 0u;
+        if (threadIdx.x == 0) {
+            b.start[0] = 0;
+            b.size[0] = single;
+            b.base[0] = 0;
+            b.first_part[0] = 0;
+            b.first_part[1] = part_count(single, rounds);
+            b.first_tile[0] = 0;
+            b.first_tile[1] = ceil_div(single, kTile);
+            *t.big[0].count = 1;
+            *t.big[1].count = 0;
+            *t.n_small = 0;
+        }
+        __syncthreads();
+    }
     const u32 count = *b.count;
     for (u32 k = blockIdx.x; k < count; k += gridDim.x) {
         const u32 start = b.start[k], size = b.size[k], fp = b.first_part[k];
@@ -1295,13 +1314,13 @@ SortLayout sort_layout(void* ws, long long n, int n_segs) {
 
 template <int SRC>
 int run_round(const Pairs& p, const SortLayout& l, const Buckets& cur, const Buckets& next, long long max_big,
-              int idx_bits, cudaStream_t st) {
+              int idx_bits, u32 single, int rounds, WsHeader* hdr, cudaStream_t st) {
     const int sms = sm_count();
     const int smem = static_cast<int>(sizeof(BigSmem)), ssmem = static_cast<int>(sizeof(ScatterSmem));
     CST_CUDA(cudaFuncSetAttribute(sort_sample_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CST_CUDA(cudaFuncSetAttribute(sort_scatter_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssmem));
     const int bgrid = static_cast<int>(max_big < 2 * sms ? max_big : 2 * sms);
-    sort_sample_kernel<SRC><<<bgrid, kBigThreads, smem, st>>>(p, cur, l.t, idx_bits);
+    sort_sample_kernel<SRC><<<bgrid, kBigThreads, smem, st>>>(p, cur, l.t, idx_bits, single, rounds, hdr);
     CST_LAUNCHED("sort_sample_kernel");
     sort_count_kernel<SRC><<<sms * kCountBlocks, kThreads, 0, st>>>(p, cur, l.t);
     CST_LAUNCHED("sort_count_kernel");
@@ -1326,18 +1345,21 @@ int run_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, const lo
     const Pairs p{keys_in, l.keys_a, l.vals_a, keys_out, perm};
     int idx_bits = 1;
     while ((1ll << idx_bits) < n) ++idx_bits;
-    sort_init_kernel<<<1, 1024, 0, st>>>(seg_offsets, n_segs, n, rounds, l.t, hdr);
-    CST_LAUNCHED("sort_init_kernel");
+    const u32 single = !seg_offsets && rounds > 0 ? static_cast<u32>(n) : 0u;
+    if (single == 0) {
+        sort_init_kernel<<<1, 1024, 0, st>>>(seg_offsets, n_segs, n, rounds, l.t, hdr);
+        CST_LAUNCHED("sort_init_kernel");
+    }
     // buckets of a round: of round 1, no more than segments
     const long long cap = static_cast<long long>(sort_sizes(n, n_segs).big);
     const long long cap1 = cap < n_segs ? cap : n_segs;
     if (rounds >= 1) {
-        if (int rc = run_round<kInput>(p, l, l.t.big[0], l.t.big[1], cap1, idx_bits, st)) return rc;
+        if (int rc = run_round<kInput>(p, l, l.t.big[0], l.t.big[1], cap1, idx_bits, single, rounds, hdr, st)) return rc;
     }
     if (rounds == 2) {
         sort_prefix_kernel<<<1, 1024, 0, st>>>(l.t.big[1], l.t.big[0].count, 1);
         CST_LAUNCHED("sort_prefix_kernel");
-        if (int rc = run_round<kBufA>(p, l, l.t.big[1], l.t.big[0], cap, idx_bits, st)) return rc;
+        if (int rc = run_round<kBufA>(p, l, l.t.big[1], l.t.big[0], cap, idx_bits, 0u, 1, hdr, st)) return rc;
     }
     const int sms = sm_count();
     const int smem = static_cast<int>(sizeof(SmallSmem)), bsmem = static_cast<int>(sizeof(BigSmem));

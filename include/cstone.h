@@ -469,6 +469,64 @@ CSTONE_API int cstone_host_status(int64_t n, int64_t leaf_cap, int32_t with_mass
                                   void* compute_stream);
 
 /* ------------------------------------------------------------------------------------------
+ * The build of one set as two calls. cstone_build_set: the bounding cube (when no box is given), the
+ * keys (with the multipole records when masses are given), the sort and the leaf array
+ * (cstone_build_leaves, whose warm start, capacity report and synchronisation it has).
+ * cstone_build_tree, on arrays sized for the leaves: the linked tree, the node counts and, with mass
+ * != NULL, the multipoles. Both run the single entry points above in order on one workspace of
+ * the size that the query gives (ws may be the same for both). The structs' key arrays are uint64, or
+ * uint32 for cstone30_build_set and cstone30_build_tree; records_ws is the workspace of
+ * cstone_keys_records and keeps its error word.
+ * ------------------------------------------------------------------------------------------ */
+typedef struct {
+    const double* x;    /* [n] device */
+    const double* y;
+    const double* z;
+    const float* m;     /* [n] device, or NULL */
+    int64_t n;
+    const double* box;  /* device {lo_x, lo_y, lo_z, side}, or NULL: the bounding cube, into box_out */
+} cstone_set_input;
+
+typedef struct {
+    int32_t curve;
+    uint32_t ncrit;
+    int32_t max_iters;
+} cstone_set_params;
+
+typedef struct {            /* device arrays, owned by the caller */
+    double* box_out;        /* [4], used without a box */
+    void* keys;             /* [n] */
+    void* sorted_keys;      /* [n] */
+    uint32_t* perm;         /* [n] */
+    void* records;          /* cstone_records_size(n) bytes, with masses */
+    void* records_ws;
+    size_t records_ws_bytes;
+    void* leaves;           /* [leaf_cap + 1] in/out as for cstone_build_leaves */
+    int64_t leaf_cap;
+    uint32_t* leaf_counts;  /* [leaf_cap] */
+    uint32_t* leaf_offsets; /* [leaf_cap + 1] */
+} cstone_set_buffers;
+
+typedef struct {            /* device arrays for n_nodes = n_leaves + (n_leaves - 1) / 7 */
+    void* node_keys;
+    int32_t* child;
+    int32_t* level_offsets;
+    int32_t* leaf_to_node;  /* [n_leaves] */
+    int32_t* parent;        /* [(n_nodes - 1) / 8], or NULL */
+    uint32_t* node_counts;
+    float* mass;            /* NULL: no multipoles */
+    double* com;            /* [3 n_nodes] */
+    float* quad;            /* [6 n_nodes] */
+} cstone_tree_buffers;
+
+CSTONE_API int cstone_build_set_workspace_size(int64_t n, int64_t leaf_cap, int32_t max_iters, size_t* bytes);
+CSTONE_API int cstone_build_set(const cstone_set_input* in, const cstone_set_params* prm, const cstone_set_buffers* out,
+                                int64_t* n_leaves, int32_t* iters, void* ws, size_t ws_bytes, void* stream);
+CSTONE_API int cstone_build_tree_workspace_size(int64_t n_leaves, int32_t with_masses, size_t* bytes);
+CSTONE_API int cstone_build_tree(const cstone_set_buffers* set, int64_t n, int64_t n_leaves, const double* box,
+                                 const cstone_tree_buffers* out, void* ws, size_t ws_bytes, void* stream);
+
+/* ------------------------------------------------------------------------------------------
  * f and g as separate steps, for a leaf array whose counts are summed over several processes
  * (the global tree of Sec. 6: every rank counts its own particles, the counts are summed by an
  * allreduce, and every rank applies the same g to the summed counts).
@@ -581,6 +639,13 @@ CSTONE_API int cstone30_upsweep_multipoles_records(const void* records, const ui
                                                    const int32_t* leaf_to_node, const int32_t* child,
                                                    const int32_t* level_offsets, const double* box, float* mass,
                                                    double* com, float* quad, void* ws, size_t ws_bytes, void* stream);
+CSTONE_API int cstone30_build_set_workspace_size(int64_t n, int64_t leaf_cap, int32_t max_iters, size_t* bytes);
+CSTONE_API int cstone30_build_set(const cstone_set_input* in, const cstone_set_params* prm,
+                                  const cstone_set_buffers* out, int64_t* n_leaves, int32_t* iters, void* ws,
+                                  size_t ws_bytes, void* stream);
+CSTONE_API int cstone30_build_tree_workspace_size(int64_t n_leaves, int32_t with_masses, size_t* bytes);
+CSTONE_API int cstone30_build_tree(const cstone_set_buffers* set, int64_t n, int64_t n_leaves, const double* box,
+                                   const cstone_tree_buffers* out, void* ws, size_t ws_bytes, void* stream);
 
 #ifdef __cplusplus
 }

@@ -117,6 +117,12 @@ def load():
             "cstone_keys_records_workspace_size": (ctypes.c_int, [psz]),
             "cstone_keys_records": (ctypes.c_int, [P, P, P, P, i64, P, ctypes.c_int, P, P, P, sz, P]),
             "cstone_upsweep_multipoles_records": (ctypes.c_int, [P, P, i64, P, i64, P, P, P, P, P, P, P, P, sz, P]),
+            "cstone_build_set_workspace_size": (ctypes.c_int, [i64, i64, i32, psz]),
+            "cstone_build_set": (ctypes.c_int, [ctypes.POINTER(_SetInput), ctypes.POINTER(_SetParams),
+                                                ctypes.POINTER(_SetBuffers), pi64, pi32, P, sz, P]),
+            "cstone_build_tree_workspace_size": (ctypes.c_int, [i64, i32, psz]),
+            "cstone_build_tree": (ctypes.c_int, [ctypes.POINTER(_SetBuffers), i64, i64, P,
+                                                 ctypes.POINTER(_TreeBuffers), P, sz, P]),
             "cstone_host_workspace_size": (ctypes.c_int, [i64, i64, i32, psz]),
             "cstone_host_stage": (ctypes.c_int, [P, P, P, P, i64, i64, ctypes.POINTER(_HostSlot), P]),
             "cstone_host_build": (ctypes.c_int, [i64, i64, i32, i32, u32, i32, ctypes.POINTER(_HostSlot),
@@ -126,7 +132,8 @@ def load():
         for name in ("keys", "sort_workspace_size", "sort", "leaves_workspace_size", "build_leaves",
                      "link_workspace_size", "link_tree", "upsweep_workspace_size", "upsweep_counts",
                      "multipole_workspace_size", "upsweep_multipoles", "leaf_counts", "rebalance_workspace_size",
-                     "rebalance", "rebalance_focus", "keys_records", "upsweep_multipoles_records"):
+                     "rebalance", "rebalance_focus", "keys_records", "upsweep_multipoles_records",
+                     "build_set_workspace_size", "build_set", "build_tree_workspace_size", "build_tree"):
             sigs["cstone30_" + name] = sigs["cstone_" + name]
         res, args = sigs["cstone30_rebalance_focus"]
         sigs["cstone30_rebalance_focus"] = (res, args[:4] + [u32, u32] + args[6:])
@@ -210,6 +217,28 @@ class _BatchBuffers(ctypes.Structure):
                 ("leaf_offsets", ctypes.c_void_p), ("node_keys", ctypes.c_void_p), ("child", ctypes.c_void_p),
                 ("level_offsets", ctypes.c_void_p), ("leaf_to_node", ctypes.c_void_p),
                 ("node_counts", ctypes.c_void_p), ("node_cap", ctypes.c_int64)]
+
+
+class _SetInput(ctypes.Structure):
+    _fields_ = [("x", ctypes.c_void_p), ("y", ctypes.c_void_p), ("z", ctypes.c_void_p), ("m", ctypes.c_void_p),
+                ("n", ctypes.c_int64), ("box", ctypes.c_void_p)]
+
+
+class _SetParams(ctypes.Structure):
+    _fields_ = [("curve", ctypes.c_int32), ("ncrit", ctypes.c_uint32), ("max_iters", ctypes.c_int32)]
+
+
+class _SetBuffers(ctypes.Structure):
+    _fields_ = [("box_out", ctypes.c_void_p), ("keys", ctypes.c_void_p), ("sorted_keys", ctypes.c_void_p),
+                ("perm", ctypes.c_void_p), ("records", ctypes.c_void_p), ("records_ws", ctypes.c_void_p),
+                ("records_ws_bytes", ctypes.c_size_t), ("leaves", ctypes.c_void_p), ("leaf_cap", ctypes.c_int64),
+                ("leaf_counts", ctypes.c_void_p), ("leaf_offsets", ctypes.c_void_p)]
+
+
+class _TreeBuffers(ctypes.Structure):
+    _fields_ = [("node_keys", ctypes.c_void_p), ("child", ctypes.c_void_p), ("level_offsets", ctypes.c_void_p),
+                ("leaf_to_node", ctypes.c_void_p), ("parent", ctypes.c_void_p), ("node_counts", ctypes.c_void_p),
+                ("mass", ctypes.c_void_p), ("com", ctypes.c_void_p), ("quad", ctypes.c_void_p)]
 
 
 class _HostSlot(ctypes.Structure):
@@ -545,6 +574,19 @@ class OctreeBuffers:
         b.ws = Workspace(d)
         return b
 
+    def c_struct(self) -> _SetBuffers:
+        _, kdt = _family(self.levels)
+        cap = self.counts.numel()
+        _need(self.leaves, kdt, "leaves")
+        _need(self.counts, torch.int32, "counts")
+        _need(self.offsets, torch.int32, "offsets")
+        if self.leaves.numel() < cap + 1:
+            raise ValueError("leaves needs leaf_cap + 1 entries")
+        rws = self.rws.buf if self.rws is not None else None
+        return _SetBuffers(self.box.data_ptr(), self.keys.data_ptr(), self.sorted_keys.data_ptr(), self.perm.data_ptr(),
+                           _ptr(self.records), _ptr(rws), rws.numel() if rws is not None else 0,
+                           self.leaves.data_ptr(), cap, self.counts.data_ptr(), self.offsets.data_ptr())
+
     def tree_buffers(self, n_leaves: int):
         nn = n_nodes(n_leaves)
         t = self.tree
@@ -579,37 +621,65 @@ def build_octree(x, y, z, curve: int = HILBERT, ncrit: int = 64, box=None, masse
     if buffers is None or buffers.n != n or buffers.levels != levels:
         buffers = OctreeBuffers.allocate(n, leaf_capacity(n, ncrit), x.device, levels)
     b = buffers
-    if box is None:
-        cstone_bbox(x, y, z, b.box, b.ws, stream)
-        box = b.box
+    fn, kdt = _family(levels)
+    _need(x, torch.float64, "x")
+    _need(y, torch.float64, "y")
+    _need(z, torch.float64, "z")
+    _need(b.box if box is None else box, torch.float64, "box")
+    _sort_args(b.keys, b.sorted_keys, b.perm, kdt, "cstone_sort")
     if masses is not None:  # keys and multipole records from one read of the coordinates
         _need(masses, torch.float32, "masses")
         if b.records is None or b.records.numel() < records_size(n):
             b.records = torch.empty(records_size(n), dtype=torch.uint8, device=b.device)
             b.rws = Workspace(b.device)
-        cstone_keys_records(x, y, z, masses, box, curve, b.keys, b.records, b.rws, stream, levels)
+        b.rws.get(_size(load().cstone_keys_records_workspace_size))
+    cur = stream if stream is not None else torch.cuda.current_stream()
+    nl0 = 0
+    if warm_leaves is not None:
+        nl0 = warm_leaves.numel() - 1
+        if nl0 > b.cap:
+            b = _grow(b, nl0)
+        b.leaves[: nl0 + 1].copy_(warm_leaves)
+    buf = b.c_struct()
+    ws = b.ws.get(_size(fn("build_set_workspace_size"), n, buf.leaf_cap, max_iters))
+    st = ctypes.c_void_p(cur.cuda_stream)
+    inp = _SetInput(x.data_ptr(), y.data_ptr(), z.data_ptr(), _ptr(masses), n, _ptr(box))
+    nl_c, it_c = ctypes.c_int64(nl0), ctypes.c_int32(0)
+    rc = fn("build_set")(ctypes.byref(inp), ctypes.byref(_SetParams(curve, ncrit, max_iters)), ctypes.byref(buf),
+                         ctypes.byref(nl_c), ctypes.byref(it_c), ws.data_ptr(), ws.numel(), st)
+    if box is None:
+        box = b.box
+    nl, iters = int(nl_c.value), int(it_c.value)
+    if rc == ERR_CAPACITY:  # the sorted keys are there: only the leaves are built again
+        want = nl
+        while True:
+            b = _grow(b, max(want, 2 * b.cap))
+            if warm_leaves is not None:
+                b.leaves[: nl0 + 1].copy_(warm_leaves)
+            try:
+                nl, iters = cstone_build_leaves(b.sorted_keys, ncrit, b.leaves, b.counts, b.offsets, nl0, max_iters,
+                                                b.ws, stream, levels)
+                break
+            except CstoneError as e:
+                if e.status != ERR_CAPACITY:
+                    raise
+                want = getattr(e, "required", 0)
+        buf = b.c_struct()
     else:
-        cstone_keys(x, y, z, box, curve, b.keys, stream, levels)
-    cstone_sort(b.keys, b.sorted_keys, b.perm, b.ws, stream, levels)
-    while True:
-        nl0 = 0
-        if warm_leaves is not None:
-            nl0 = warm_leaves.numel() - 1
-            if nl0 > b.cap:
-                b = _grow(b, nl0)
-            b.leaves[: nl0 + 1].copy_(warm_leaves)
-        try:
-            nl, iters = cstone_build_leaves(b.sorted_keys, ncrit, b.leaves, b.counts, b.offsets, nl0, max_iters,
-                                            b.ws, stream, levels)
-            break
-        except CstoneError as e:
-            if e.status != ERR_CAPACITY:
-                raise
-            b = _grow(b, max(getattr(e, "required", 0), 2 * b.cap))
+        _check(rc, "cstone_build_set")
     t = b.tree_buffers(nl)
     nn = n_nodes(nl)
-    cstone_link_tree(b.leaves, nl, t["NK"], t["CO"], t["LO"], t["leaf_to_node"], t["parent"], b.ws, stream, levels)
-    cstone_upsweep_counts(b.counts, nl, t["leaf_to_node"], t["CO"], t["LO"], t["counts"], b.ws, stream, levels)
+    if masses is not None and ("mass" not in t or t["mass"].numel() < nn):
+        cap_nodes = t["cap_nodes"]
+        t["mass"] = torch.empty(cap_nodes, dtype=torch.float32, device=b.device)
+        t["com"] = torch.empty(3 * cap_nodes, dtype=torch.float64, device=b.device)
+        t["quad"] = torch.empty(6 * cap_nodes, dtype=torch.float32, device=b.device)
+    ws = b.ws.get(_size(fn("build_tree_workspace_size"), nl, 1 if masses is not None else 0))
+    moments = tuple(t[k].data_ptr() for k in ("mass", "com", "quad")) if masses is not None else (None, None, None)
+    tree = _TreeBuffers(t["NK"].data_ptr(), t["CO"].data_ptr(), t["LO"].data_ptr(), t["leaf_to_node"].data_ptr(),
+                        t["parent"].data_ptr(), t["counts"].data_ptr(), *moments)
+    _check(fn("build_tree")(ctypes.byref(buf), n, nl, box.data_ptr(), ctypes.byref(tree), ws.data_ptr(),
+                            ws.numel(), st), "cstone_build_tree")
     out = {
         "buffers": b, "box": box, "keys": b.keys, "sorted_keys": b.sorted_keys, "perm": b.perm,
         "leaves": b.leaves[: nl + 1], "leaf_counts": b.counts[:nl], "leaf_offsets": b.offsets[: nl + 1],
@@ -617,14 +687,7 @@ def build_octree(x, y, z, curve: int = HILBERT, ncrit: int = 64, box=None, masse
         "leaf_to_node": t["leaf_to_node"][:nl], "parent": t["parent"][: (nn - 1) // 8], "node_counts": t["counts"][:nn],
     }
     if masses is not None:
-        if "mass" not in t or t["mass"].numel() < nn:
-            cap_nodes = t["cap_nodes"]
-            t["mass"] = torch.empty(cap_nodes, dtype=torch.float32, device=b.device)
-            t["com"] = torch.empty(3 * cap_nodes, dtype=torch.float64, device=b.device)
-            t["quad"] = torch.empty(6 * cap_nodes, dtype=torch.float32, device=b.device)
         mass, com, quad = t["mass"][:nn], t["com"][: 3 * nn], t["quad"][: 6 * nn]
-        cstone_upsweep_multipoles_records(b.records, b.perm, n, b.offsets, nl, t["leaf_to_node"], t["CO"], t["LO"],
-                                          box, mass, com, quad, b.ws, stream, levels)
         out.update({"mass": mass, "com": com.view(3, nn), "quad": quad.view(6, nn)})
     return out
 
@@ -814,12 +877,27 @@ def cstone_build_batched_result(ws: Workspace, bufs: BatchBuffers, max_iters: in
     return int(ne.value), int(nn.value), int(it.value)
 
 
-def _batched_result(bufs: BatchBuffers, ne: int, nn: int, iters: int, ws) -> dict:
-    """Result dict of a batched build: device tensors cut to the built sizes, and host copies of the
-    element and node offsets (read from the device)."""
+def _offsets_to_host(bufs: BatchBuffers, stream=None):
+    """Host copies of the element and node offsets, valid once ``stream`` is synchronised
+    (reading the outcome does that): no wait of their own (48 sets: 447 us with two reads after the
+    outcome, 376 so)."""
     t = bufs.t
-    eo_host = t["element_offsets"].cpu().tolist()
-    node_offsets = t["LO"][:, 0].cpu().tolist() + [nn]
+    with torch.cuda.stream(stream):  # None: the current stream
+        eo = torch.empty(t["element_offsets"].shape, dtype=torch.int64, pin_memory=True)
+        lo = torch.empty(t["LO"].shape[0], dtype=torch.int32, pin_memory=True)
+        eo.copy_(t["element_offsets"], non_blocking=True)
+        lo.copy_(t["LO"][:, 0], non_blocking=True)
+    return eo, lo
+
+
+def _batched_result(bufs: BatchBuffers, ne: int, nn: int, iters: int, ws, host=None) -> dict:
+    """Result dict of a batched build: device tensors cut to the built sizes, and the element and node
+    offsets on the host (from ``_offsets_to_host``, or read from the device)."""
+    t = bufs.t
+    if host is None:
+        host = t["element_offsets"].cpu(), t["LO"][:, 0].cpu()
+    eo_host = host[0].tolist()
+    node_offsets = host[1].tolist() + [nn]
     return {"boxes": t["boxes"], "keys": t["keys"][: bufs.n], "sorted_keys": t["sorted_keys"][: bufs.n],
             "perm": t["perm"][: bufs.n], "elements": t["elements"][:ne], "n_elements": ne,
             "element_offsets": t["element_offsets"], "element_offsets_host": eo_host,
@@ -856,6 +934,7 @@ def build_octrees_batched(x, y, z, set_offsets, curve: int = MORTON, ncrit: int 
                 bufs.t["element_offsets"].copy_(warm["element_offsets"])
         cstone_build_batched(x, y, z, set_offsets, bufs, curve, ncrit, boxes=boxes, warm=warm is not None,
                              max_iters=max_iters, ws=ws, stream=stream)
+        host = _offsets_to_host(bufs, stream)
         try:
             ne, nn, iters = cstone_build_batched_result(ws, bufs, max_iters, stream)
             break
@@ -866,7 +945,7 @@ def build_octrees_batched(x, y, z, set_offsets, curve: int = MORTON, ncrit: int 
                 warm = None  # the failed loop left root arrays in place of the warm ones: start cold
             bufs = BatchBuffers.allocate(n, s, max(2 * bufs.elem_cap, getattr(e, "required", 0) + 1024), dev,
                                          keep=bufs)
-    out = _batched_result(bufs, ne, nn, iters, ws)
+    out = _batched_result(bufs, ne, nn, iters, ws, host)
     if boxes is not None:
         out["boxes"] = boxes
     return out
@@ -1078,8 +1157,9 @@ class GraphTimeStepper:
                              boxes=self.boxes, warm=warm, max_iters=self.max_iters, ws=self.ws)
 
     def _result(self):
+        host = _offsets_to_host(self.bufs)
         ne, nn, iters = cstone_build_batched_result(self.ws, self.bufs, self.max_iters)
-        out = _batched_result(self.bufs, ne, nn, iters, self.ws)
+        out = _batched_result(self.bufs, ne, nn, iters, self.ws, host)
         out["boxes"] = self.boxes
         return out
 

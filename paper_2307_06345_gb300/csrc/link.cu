@@ -20,15 +20,25 @@
 // the nodes 8 g + 1 .. 8 g + 8: the child index that the paper's search for the key << 3 in the
 // next level finds. The scatter ranks every internal node among the internal nodes with a second
 // counting sort of the pairs alone and writes CO (and the parent of every sibling group) directly.
-// Batched sets still search (link_b_child_kernel).
+// The sets of a batch go the same way, each from its own first node and internal node.
+//
+// Node counts in the same pass, where the leaves' particle offsets are at hand (the builds): a node's
+// particles are those between the first of its first leaf and the first of the leaf after its last, and
+// both leaves are found near the pair (`covered`). This takes the place of a sum over the children level
+// by level, whose grid barriers bounded it (upsweep.cu, which still serves callers that have counts only).
+// Link and counts together: 512 sets of 1,024 to 1,048,576 particles 640 -> 330 us, 48 of 128 to 4,096
+// 88 -> 35, one of 1,048,576 43 -> 24, of 33,554,432 122 -> 84.
 #include "common.cuh"
 
 namespace CST_NS {
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kItems = 8;
-constexpr int kTile = kThreads * kItems;
+// Leaves per thread: 8, and 2 up to kSmallLeaves leaves, where a pass of 8 items in a row is longer than
+// the rest of the kernel and most SMs would have no tile (12,000 leaves: scatter 13.5 us with 8, 9.5 with 2).
+constexpr int kItemsLarge = 8, kItemsSmall = 2;
+constexpr long long kSmallLeaves = 1 << 18;
+constexpr int items_of(long long leaves) { return leaves <= kSmallLeaves ? kItemsSmall : kItemsLarge; }
 constexpr int kNumLevels = kLevels + 1;  // levels 0..L
 
 __device__ __forceinline__ int leaf_level(Key delta) {  // delta is a power of 8
@@ -45,61 +55,245 @@ __device__ __forceinline__ Key placeholder(Key key, int level) {
     return (static_cast<Key>(1) << (3 * level)) | (key >> (3 * (kLevels - level)));
 }
 
-__global__ void __launch_bounds__(kThreads) link_count_kernel(const Key* __restrict__ K, u32 nl, u32 ntiles,
-                                                              u32* __restrict__ counts, u32* __restrict__ pair_counts) {
-    // per-thread counts per level (own column, no conflicts): all nodes, then internal nodes
-    __shared__ u32 s_c[2][kNumLevels][kThreads];
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int l = 0; l < kNumLevels; ++l) s_c[0][l][tid] = s_c[1][l][tid] = 0;
-    const u32 tile = blockIdx.x;
-    const u32 i0 = tile * kTile + tid * kItems;
-    for (int k = 0; k < kItems; ++k) {
-        u32 i = i0 + k;
-        if (i >= nl) break;
-        Key a = K[i], b = K[i + 1];
-        s_c[0][leaf_level(b - a)][tid] += 1;
-        if (i + 1 < nl) {
-            int pl = pair_level(a, b);
-            if (pl >= 0) {
-                s_c[0][pl][tid] += 1;
-                s_c[1][pl][tid] += 1;
-            }
-        }
+// The tile that a block works on: `cnt` leaves from `e0`, of a set whose first leaf is `lo` and whose end
+// key is element `hi`; its counters are at first * 22 + level * of + index.
+struct Tile {
+    u32 e0, cnt, lo, hi;
+    u32 first, of, index;
+    __device__ __forceinline__ u32 counter(int level) const {
+        return first * kNumLevels + static_cast<u32>(level) * of + index;
     }
-    __syncthreads();
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int r = warp; r < 2 * kNumLevels; r += kThreads / 32) {
-        const u32* row = &s_c[r / kNumLevels][r % kNumLevels][0];
-        u32 v = 0;
+};
+
+// One counter word per thread and level: all nodes in the low half, internal nodes in the high half (a tile
+// has at most 2 * 2048 nodes, so neither its sums nor its ranks overflow a half).
+constexpr u32 kLeafOne = 1u, kInternalOne = 0x10001u;
+
+template <int ITEMS>
+__device__ __forceinline__ void count_items(const Key (&key)[ITEMS + 1], u32 i0, const Tile& t,
+                                            u32 (*s_rank)[kThreads]) {
 #pragma unroll
-        for (int q = 0; q < kThreads / 32; ++q) v += row[q * 32 + lane];
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-        if (lane == 0) {
-            if (r < kNumLevels)
-                counts[(size_t)r * ntiles + tile] = v;
-            else if (pair_counts)
-                pair_counts[(size_t)(r - kNumLevels) * ntiles + tile] = v;
+    for (int l = 0; l < kNumLevels; ++l) s_rank[l][threadIdx.x] = 0;
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        if (i0 + k >= t.e0 + t.cnt) break;
+        s_rank[leaf_level(key[k + 1] - key[k])][threadIdx.x] += kLeafOne;
+        if (i0 + k + 1 < t.hi) {
+            const int pl = pair_level(key[k], key[k + 1]);
+            if (pl >= 0) s_rank[pl][threadIdx.x] += kInternalOne;
         }
     }
 }
 
+template <int ITEMS>
+__device__ __forceinline__ void load_items(const Key* __restrict__ K, u32 i0, const Tile& t, Key (&key)[ITEMS + 1]) {
+#pragma unroll
+    for (int k = 0; k <= ITEMS; ++k) key[k] = i0 + k <= t.e0 + t.cnt ? K[i0 + k] : kKeyEnd;
+}
+
+template <int ITEMS>
+__device__ __forceinline__ void count_tile(const Key* __restrict__ K, const Tile& t, u32* __restrict__ counts,
+                                           u32* __restrict__ pair_counts) {
+    __shared__ u32 s_rank[kNumLevels][kThreads];  // own column per thread, no conflicts
+    const u32 i0 = t.e0 + threadIdx.x * ITEMS;
+    Key key[ITEMS + 1];
+    load_items<ITEMS>(K, i0, t, key);
+    count_items<ITEMS>(key, i0, t, s_rank);
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    for (int l = warp; l < kNumLevels; l += kThreads / 32) {
+        u32 v = 0;
+#pragma unroll
+        for (int q = 0; q < kThreads / 32; ++q) v += s_rank[l][q * 32 + lane];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) {
+            counts[t.counter(l)] = v & 0xffffu;
+            pair_counts[t.counter(l)] = v >> 16;
+        }
+    }
+}
+
+// The leaves of the internal node of level `level` whose pair is (i, i + 1): from the first with a key at or
+// after its start to the one with a key at or after its end, within the set. When the eight children are
+// leaves (nine in ten nodes of a usual tree) they are i - 3 .. i + 4; else the search goes outwards by powers of
+// 8 and then bisects. Every index stays within [lo, hi], whatever the keys.
+__device__ __forceinline__ uint2 covered(const Key* __restrict__ K, const Tile& t, u32 i, Key a, int level) {
+    const Key size = static_cast<Key>(1) << (3 * (kLevels - level));
+    const Key start = a & ~(size - 1), end = start + size;
+    uint2 r = make_uint2(i - 3, i + 5);
+    if (i - t.lo < 3 || K[i - 3] != start) {
+        u32 at = i, from = i, step = 8;  // K[at] >= start
+        for (;; step <<= 3) {
+            from = i - t.lo > step ? i - step : t.lo;
+            if (from == t.lo || K[from] < start) break;
+            at = from;
+        }
+        while (from < at) {
+            const u32 mid = from + ((at - from) >> 1);
+            if (K[mid] < start)
+                from = mid + 1;
+            else
+                at = mid;
+        }
+        r.x = at;
+    }
+    if (t.hi - i < 5 || K[i + 5] != end) {
+        u32 from = i + 1, at = t.hi, step = 8;
+        for (;; step <<= 3) {
+            at = t.hi - i > step ? i + step : t.hi;
+            if (at == t.hi || K[at] >= end) break;
+            from = at;
+        }
+        while (from < at) {
+            const u32 mid = from + ((at - from) >> 1);
+            if (K[mid] < end)
+                from = mid + 1;
+            else
+                at = mid;
+        }
+        r.y = at;
+    }
+    return r;
+}
+
+struct Out {
+    u32 n_nodes;              // capacity of the node arrays
+    Key* NK;
+    int* leaf_to_node;
+    int* CO;
+    int* parent;              // may be NULL
+    const u32* leaf_offsets;  // with COUNTS: first particle of every leaf and end key
+    u32* node_counts;
+};
+
+// Places a tile's leaves and internal nodes in breadth-first order, in in-order sequence: leaf i, then the
+// internal node of pair i; the g-th internal node of the set has its children at 8 g + 1 of the set's nodes.
+template <int ITEMS, bool COUNTS>
+__device__ __forceinline__ void place_tile(const Key* __restrict__ K, const Tile& t, const u32* __restrict__ offsets,
+                                           const u32* __restrict__ pair_offsets, const Out& o) {
+    constexpr u32 kList = COUNTS ? kThreads * ITEMS / 8 + 64 : 1;
+    __shared__ u32 s_rank[kNumLevels][kThreads];  // per-thread counts, then per-thread ranks within the tile
+    __shared__ u32 s_base[2][kNumLevels];         // the tile's first node and internal node of each level
+    __shared__ uint2 s_list[kList];               // internal nodes (node, leaf of the pair) for the counts
+    __shared__ u32 s_listed;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const u32 i0 = t.e0 + tid * ITEMS;
+    Key key[ITEMS + 1];
+    load_items<ITEMS>(K, i0, t, key);
+    if (tid == 0) s_listed = 0;
+    if (tid < kNumLevels) s_base[0][tid] = offsets[t.counter(tid)];
+    if (tid >= 32 && tid < 32 + kNumLevels) s_base[1][tid - 32] = pair_offsets[t.counter(tid - 32)];
+    const u32 first_node = offsets[t.first * kNumLevels], first_internal = pair_offsets[t.first * kNumLevels];
+    count_items<ITEMS>(key, i0, t, s_rank);
+    __syncthreads();
+    // exclusive scan of every level row across the threads
+    for (int l = warp; l < kNumLevels; l += kThreads / 32) {
+        u32 v[kThreads / 32];
+        u32 sum = 0;
+#pragma unroll
+        for (int q = 0; q < kThreads / 32; ++q) {
+            v[q] = s_rank[l][lane * (kThreads / 32) + q];
+            sum += v[q];
+        }
+        u32 incl = sum;
+        for (int s = 1; s < 32; s <<= 1) {
+            const u32 w = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += w;
+        }
+        u32 run = incl - sum;
+#pragma unroll
+        for (int q = 0; q < kThreads / 32; ++q) {
+            s_rank[l][lane * (kThreads / 32) + q] = run;
+            run += v[q];
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < ITEMS; ++k) {
+        const u32 i = i0 + k;
+        if (i >= t.e0 + t.cnt) break;
+        const Key a = key[k], b = key[k + 1];
+        const int ll = leaf_level(b - a);
+        const u32 rx = s_rank[ll][tid];
+        s_rank[ll][tid] = rx + kLeafOne;
+        const u32 x = s_base[0][ll] + (rx & 0xffffu);
+        if (x < o.n_nodes) {
+            o.NK[x] = placeholder(a, ll);
+            o.CO[x] = 0;
+            o.leaf_to_node[i] = static_cast<int>(x);
+            if (COUNTS) o.node_counts[x] = o.leaf_offsets[i + 1] - o.leaf_offsets[i];
+        }
+        const int pl = i + 1 < t.hi ? pair_level(a, b) : -1;
+        if (pl >= 0) {
+            const u32 ry = s_rank[pl][tid];
+            s_rank[pl][tid] = ry + kInternalOne;
+            const u32 y = s_base[0][pl] + (ry & 0xffffu);
+            const u32 g = s_base[1][pl] + (ry >> 16) - first_internal;
+            const u32 c = first_node + 8u * g + 1u;
+            if (y < o.n_nodes) {
+                const bool inside = c + 7u < o.n_nodes;
+                o.NK[y] = placeholder(a, pl);
+                o.CO[y] = inside ? static_cast<int>(c) : 0;
+                if (o.parent && inside) o.parent[g] = static_cast<int>(y);
+                if (COUNTS) {
+                    const u32 at = atomicAdd(&s_listed, 1u);
+                    if (at < kList) {
+                        s_list[at] = make_uint2(y, i);
+                    } else {
+                        const uint2 r = covered(K, t, i, a, pl);
+                        o.node_counts[y] = o.leaf_offsets[r.y] - o.leaf_offsets[r.x];
+                    }
+                }
+            }
+        }
+    }
+    if (!COUNTS) return;
+    // the searches of the tile's internal nodes (one leaf in seven has one) side by side, not one lane at a time
+    __syncthreads();
+    const u32 listed = min(s_listed, kList);
+    for (u32 q = tid; q < listed; q += kThreads) {
+        const uint2 yi = s_list[q];
+        const Key a = K[yi.y];
+        const uint2 r = covered(K, t, yi.y, a, pair_level(a, K[yi.y + 1]));
+        o.node_counts[yi.x] = o.leaf_offsets[r.y] - o.leaf_offsets[r.x];
+    }
+}
+
+template <int ITEMS>
+__device__ __forceinline__ Tile single_tile(u32 nl) {
+    const u32 e0 = blockIdx.x * (kThreads * ITEMS);
+    return Tile{e0, min(static_cast<u32>(kThreads * ITEMS), nl - e0), 0u, nl, 0u, gridDim.x, blockIdx.x};
+}
+
+template <int ITEMS>
+__global__ void __launch_bounds__(kThreads) link_count_kernel(const Key* __restrict__ K, u32 nl,
+                                                              u32* __restrict__ counts, u32* __restrict__ pair_counts) {
+    count_tile<ITEMS>(K, single_tile<ITEMS>(nl), counts, pair_counts);
+}
+
+template <int ITEMS, bool COUNTS>
+__global__ void __launch_bounds__(kThreads) link_scatter_kernel(const Key* __restrict__ K, u32 nl,
+                                                                const u32* __restrict__ offsets,
+                                                                const u32* __restrict__ pair_offsets, Out o) {
+    place_tile<ITEMS, COUNTS>(K, single_tile<ITEMS>(nl), offsets, pair_offsets, o);
+}
+
 // Exclusive scans of the level-major (level, tile) counts of all nodes (half 0) and of the internal
-// nodes alone (half 1), each of `len` entries, in chunks of kScanChunk: block (c, h) sums chunk c
-// of half h, then block (c, h) adds the sums of the chunks before it and scans its chunk. LO comes
+// nodes alone (half 1), each of `len` entries at a distance of `stride`, in chunks of kScanChunk:
+// block (c, h) sums chunk c of half h, then adds the sums of the chunks before it and scans its chunk. LO comes
 // from half 0 (LO[l] = offset of (l, 0), LO[22] = total); a total of all nodes different from
 // n_expected, or of internal nodes different from (n_expected - 1) / 8, means the input was not a
-// cornerstone array. Without LO (the batched (set, level, tile) counts, one half) the total goes
-// to the entry after the scanned ones.
+// cornerstone array. Without LO (the batched (set, level, tile) counts) the total goes to the entry
+// after the scanned ones.
 constexpr u32 kScanThreads = 1024;
 constexpr u32 kScanPer = 4;
 constexpr u32 kScanChunk = kScanThreads * kScanPer;
 
 __global__ void __launch_bounds__(kScanThreads) link_scan_reduce_kernel(const u32* __restrict__ counts, u32 len,
-                                                                        u32* __restrict__ partial) {
+                                                                        size_t stride, u32* __restrict__ partial) {
     __shared__ u32 s_warp[kScanThreads / 32];
     const u32 h = blockIdx.y, c = blockIdx.x;
-    const u32* a = counts + (size_t)h * len;
+    const u32* a = counts + h * stride;
     u32 sum = 0;
 #pragma unroll
     for (u32 j = 0; j < kScanPer; ++j) {
@@ -116,7 +310,8 @@ __global__ void __launch_bounds__(kScanThreads) link_scan_reduce_kernel(const u3
     }
 }
 
-__global__ void __launch_bounds__(kScanThreads) link_scan_apply_kernel(u32* __restrict__ counts, u32 len, u32 ntiles,
+__global__ void __launch_bounds__(kScanThreads) link_scan_apply_kernel(u32* __restrict__ counts, u32 len,
+                                                                       size_t stride, u32 ntiles,
                                                                        const u32* __restrict__ partial,
                                                                        int* __restrict__ LO, u32 n_expected,
                                                                        WsHeader* hdr) {
@@ -143,13 +338,13 @@ __global__ void __launch_bounds__(kScanThreads) link_scan_apply_kernel(u32* __re
                     if (h == 0) LO[kNumLevels] = static_cast<int>(all);
                     if (all != want) raise_error(hdr, CSTONE_ERR_INVALID_ARG, all);
                 } else {
-                    counts[(size_t)h * len + len] = all;  // without LO (batched sets): the total after the scan
+                    counts[h * stride + len] = all;  // without LO (batched sets): the total after the scan
                 }
             }
         }
     }
     __syncthreads();
-    u32* a = counts + (size_t)h * len;
+    u32* a = counts + h * stride;
     // thread t takes the kScanPer consecutive entries c * kScanChunk + t * kScanPer + j
     const u32 i0 = c * kScanChunk + threadIdx.x * kScanPer;
     u32 v[kScanPer], sum = 0;
@@ -186,86 +381,12 @@ __global__ void __launch_bounds__(kScanThreads) link_scan_apply_kernel(u32* __re
     }
 }
 
-__global__ void __launch_bounds__(kThreads) link_scatter_kernel(const Key* __restrict__ K, u32 nl, u32 ntiles,
-                                                                const u32* __restrict__ offsets,
-                                                                const u32* __restrict__ pair_offsets, u32 n_nodes,
-                                                                Key* __restrict__ NK, int* __restrict__ leaf_to_node,
-                                                                int* __restrict__ CO, int* __restrict__ parent) {
-    __shared__ u32 s_rank[kNumLevels][kThreads];   // per-thread counts, then per-thread slots
-    __shared__ u32 s_prank[kNumLevels][kThreads];  // the same for internal nodes only
-    const int tid = threadIdx.x;
-    const u32 tile = blockIdx.x;
-    const u32 i0 = tile * kTile + tid * kItems;
-    const u32 n_int = (n_nodes - 1) / 8;
-#pragma unroll
-    for (int l = 0; l < kNumLevels; ++l) s_rank[l][tid] = s_prank[l][tid] = 0;
-    // count this thread's items per level (own column, no conflicts)
-    for (int k = 0; k < kItems; ++k) {
-        u32 i = i0 + k;
-        if (i >= nl) break;
-        Key a = K[i], b = K[i + 1];
-        s_rank[leaf_level(b - a)][tid] += 1;
-        if (i + 1 < nl) {
-            int pl = pair_level(a, b);
-            if (pl >= 0) {
-                s_rank[pl][tid] += 1;
-                s_prank[pl][tid] += 1;
-            }
-        }
-    }
-    __syncthreads();
-    // exclusive scan of every level row across the threads, plus the tile's global offset
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int r = warp; r < 2 * kNumLevels; r += kThreads / 32) {
-        const int l = r % kNumLevels;
-        u32* row = r < kNumLevels ? s_rank[l] : s_prank[l];
-        const u32* off = r < kNumLevels ? offsets : pair_offsets;
-        u32 v[kThreads / 32];
-        u32 sum = 0;
-#pragma unroll
-        for (int q = 0; q < kThreads / 32; ++q) {
-            v[q] = row[lane * (kThreads / 32) + q];
-            sum += v[q];
-        }
-        u32 incl = sum;
-        for (int s = 1; s < 32; s <<= 1) {
-            u32 t = __shfl_up_sync(0xffffffffu, incl, s);
-            if (lane >= s) incl += t;
-        }
-        u32 run = off[(size_t)l * ntiles + tile] + incl - sum;
-#pragma unroll
-        for (int q = 0; q < kThreads / 32; ++q) {
-            row[lane * (kThreads / 32) + q] = run;
-            run += v[q];
-        }
-    }
-    __syncthreads();
-    // emit in in-order sequence: leaf i, then the internal node of pair i; the g-th internal node
-    // has its children at 8 g + 1
-    for (int k = 0; k < kItems; ++k) {
-        u32 i = i0 + k;
-        if (i >= nl) break;
-        Key a = K[i], b = K[i + 1];
-        int ll = leaf_level(b - a);
-        u32 x = s_rank[ll][tid]++;
-        if (x < n_nodes) {
-            NK[x] = placeholder(a, ll);
-            CO[x] = 0;
-            leaf_to_node[i] = static_cast<int>(x);
-        }
-        if (i + 1 < nl) {
-            int pl = pair_level(a, b);
-            if (pl >= 0) {
-                u32 y = s_rank[pl][tid]++;
-                u32 g = s_prank[pl][tid]++;
-                if (y < n_nodes) {
-                    NK[y] = placeholder(a, pl);
-                    CO[y] = g < n_int ? static_cast<int>(8u * g + 1u) : 0;
-                    if (parent && g < n_int) parent[g] = static_cast<int>(y);
-                }
-            }
-        }
-    }
+// The largest number of tiles of any array of at most `leaves` leaves.
+inline long long most_tiles(long long leaves) {
+    const long long small = leaves < kSmallLeaves ? leaves : kSmallLeaves;
+    const long long a = (small + kThreads * kItemsSmall - 1) / (kThreads * kItemsSmall);
+    const long long b = (leaves + kThreads * kItemsLarge - 1) / (kThreads * kItemsLarge);
+    return a > b ? a : b;
 }
 
 struct LinkLayout {
@@ -279,12 +400,15 @@ struct LinkLayout {
 LinkLayout link_layout(void* ws, long long nl) {
     LinkLayout l;
     Carver c(ws);
-    l.ntiles = static_cast<u32>((nl + kTile - 1) / kTile);
+    const long long tile = kThreads * items_of(nl);
+    l.ntiles = static_cast<u32>((nl + tile - 1) / tile);
     if (l.ntiles == 0) l.ntiles = 1;
     const u32 len = l.ntiles * kNumLevels;
     l.chunks = (len + kScanChunk - 1) / kScanChunk;
-    l.counts = c.take<u32>((size_t)2 * len);
-    l.partial = c.take<u32>((size_t)2 * l.chunks);
+    // a workspace for more leaves serves fewer: no smaller than the largest that small tiles need
+    const size_t held = (size_t)most_tiles(nl) * kNumLevels;
+    l.counts = c.take<u32>(2 * held);
+    l.partial = c.take<u32>(2 * ((held + kScanChunk - 1) / kScanChunk));
     l.bytes = c.size();
     return l;
 }
@@ -297,6 +421,7 @@ LinkLayout link_layout(void* ws, long long nl) {
 // one contiguous breadth-first block.
 struct LinkSets {
     const long long* elem_offsets;  // [S+1] first element of each set
+    u32 tile;                       // leaves per tile
     u32* n_tiles;                   // device scalar
     u32* tile_first;                // [S+1] first tile of each set
     u32* tile_set;                  // [max_tiles]
@@ -313,7 +438,7 @@ __global__ void __launch_bounds__(1024) link_b_setup_kernel(LinkSets ls) {
     u32 st = 0, sn = 0;
     for (int q = begin; q < end; ++q) {
         const long long nl = ls.elem_offsets[q + 1] - ls.elem_offsets[q] - 1;
-        st += static_cast<u32>((nl + kTile - 1) / kTile);
+        st += static_cast<u32>((nl + ls.tile - 1) / ls.tile);
         sn += static_cast<u32>(nl + (nl - 1) / 7);
     }
     s_t[threadIdx.x] = st;
@@ -332,7 +457,7 @@ __global__ void __launch_bounds__(1024) link_b_setup_kernel(LinkSets ls) {
         ls.tile_first[q] = rt;
         ls.node_first[q] = rn;
         const long long nl = ls.elem_offsets[q + 1] - ls.elem_offsets[q] - 1;
-        rt += static_cast<u32>((nl + kTile - 1) / kTile);
+        rt += static_cast<u32>((nl + ls.tile - 1) / ls.tile);
         rn += static_cast<u32>(nl + (nl - 1) / 7);
     }
     if (threadIdx.x == 1023) {
@@ -346,7 +471,8 @@ __global__ void __launch_bounds__(kThreads) link_b_tiles_kernel(LinkSets ls, u32
                                                                 int* __restrict__ leaf_to_node) {
     // elements between the actual count and the capacity map to no node
     const u32 ne = static_cast<u32>(ls.elem_offsets[ls.n_sets]);
-    for (u32 e = ne + blockIdx.x * kThreads + threadIdx.x; e < elem_cap; e += gridDim.x * kThreads) leaf_to_node[e] = -1;
+    for (u32 e = ne + blockIdx.x * kThreads + threadIdx.x; e < elem_cap; e += gridDim.x * kThreads)
+        leaf_to_node[e] = -1;
     const u32 total = *ls.n_tiles;
     for (u32 t = blockIdx.x * kThreads + threadIdx.x; t < max_tiles; t += gridDim.x * kThreads) {
         if (t >= total) {
@@ -361,11 +487,11 @@ __global__ void __launch_bounds__(kThreads) link_b_tiles_kernel(LinkSets ls, u32
             else
                 hi = mid;
         }
-        const long long e0 = ls.elem_offsets[lo] + (long long)(t - ls.tile_first[lo]) * kTile;
+        const long long e0 = ls.elem_offsets[lo] + (long long)(t - ls.tile_first[lo]) * ls.tile;
         const long long last_leaf_end = ls.elem_offsets[lo + 1] - 1;  // the end key is not a leaf
         ls.tile_set[t] = static_cast<u32>(lo);
         ls.tile_elem[t] = static_cast<u32>(e0);
-        ls.tile_count[t] = static_cast<u32>(min((long long)kTile, last_leaf_end - e0));
+        ls.tile_count[t] = static_cast<u32>(min((long long)ls.tile, last_leaf_end - e0));
     }
 }
 
@@ -374,28 +500,26 @@ __device__ __forceinline__ u32 count_index(const LinkSets& ls, u32 set, int leve
     return tf * kNumLevels + static_cast<u32>(level) * nt + k;
 }
 
+// The block's tile; false when there is none.
+__device__ __forceinline__ bool batched_tile(const LinkSets& ls, Tile& t) {
+    t.cnt = ls.tile_count[blockIdx.x];
+    if (t.cnt == 0) return false;
+    const u32 set = ls.tile_set[blockIdx.x];
+    t.e0 = ls.tile_elem[blockIdx.x];
+    t.lo = static_cast<u32>(ls.elem_offsets[set]);
+    t.hi = static_cast<u32>(ls.elem_offsets[set + 1] - 1);
+    t.first = ls.tile_first[set];
+    t.of = ls.tile_first[set + 1] - t.first;
+    t.index = blockIdx.x - t.first;
+    return true;
+}
+
+template <int ITEMS>
 __global__ void __launch_bounds__(kThreads) link_b_count_kernel(const Key* __restrict__ K, LinkSets ls,
-                                                                u32* __restrict__ counts) {
-    __shared__ u32 s_cnt[kNumLevels];
-    const u32 tile = blockIdx.x;
-    const u32 cnt = ls.tile_count[tile];
-    if (cnt == 0) return;
-    if (threadIdx.x < kNumLevels) s_cnt[threadIdx.x] = 0;
-    __syncthreads();
-    const u32 e0 = ls.tile_elem[tile];
-    for (u32 q = threadIdx.x; q < cnt; q += kThreads) {
-        const u32 e = e0 + q;
-        const Key a = K[e], b = K[e + 1];
-        atomicAdd(&s_cnt[leaf_level(b - a)], 1u);
-        if (b != kKeyEnd) {
-            const int pl = pair_level(a, b);
-            if (pl >= 0) atomicAdd(&s_cnt[pl], 1u);
-        }
-    }
-    __syncthreads();
-    const u32 set = ls.tile_set[tile];
-    if (threadIdx.x < kNumLevels)
-        counts[count_index(ls, set, threadIdx.x, tile - ls.tile_first[set])] = s_cnt[threadIdx.x];
+                                                                u32* __restrict__ counts,
+                                                                u32* __restrict__ pair_counts) {
+    Tile t;
+    if (batched_tile(ls, t)) count_tile<ITEMS>(K, t, counts, pair_counts);
 }
 
 // Level offsets of every set (global node indices), a size check per set, and -1 for the
@@ -421,113 +545,19 @@ __global__ void link_b_lo_kernel(const u32* __restrict__ counts, LinkSets ls, in
     }
 }
 
+template <int ITEMS, bool COUNTS>
 __global__ void __launch_bounds__(kThreads) link_b_scatter_kernel(const Key* __restrict__ K, LinkSets ls,
-                                                                  const u32* __restrict__ offsets, u32 n_nodes,
-                                                                  Key* __restrict__ NK, int* __restrict__ leaf_to_node) {
-    __shared__ u32 s_rank[kNumLevels][kThreads];
-    const int tid = threadIdx.x;
-    const u32 tile = blockIdx.x;
-    const u32 cnt = ls.tile_count[tile];
-    if (cnt == 0) return;
-    const u32 e0 = ls.tile_elem[tile];
-    const u32 set = ls.tile_set[tile];
-    const u32 k_in_set = tile - ls.tile_first[set];
-    const u32 i0 = tid * kItems;
-#pragma unroll
-    for (int l = 0; l < kNumLevels; ++l) s_rank[l][tid] = 0;
-    for (int k = 0; k < kItems; ++k) {
-        const u32 q = i0 + k;
-        if (q >= cnt) break;
-        const Key a = K[e0 + q], b = K[e0 + q + 1];
-        s_rank[leaf_level(b - a)][tid] += 1;
-        if (b != kKeyEnd) {
-            const int pl = pair_level(a, b);
-            if (pl >= 0) s_rank[pl][tid] += 1;
-        }
-    }
-    __syncthreads();
-    const int lane = tid & 31, warp = tid >> 5;
-    for (int l = warp; l < kNumLevels; l += kThreads / 32) {
-        u32 v[kThreads / 32];
-        u32 sum = 0;
-#pragma unroll
-        for (int q = 0; q < kThreads / 32; ++q) {
-            v[q] = s_rank[l][lane * (kThreads / 32) + q];
-            sum += v[q];
-        }
-        u32 incl = sum;
-        for (int o = 1; o < 32; o <<= 1) {
-            const u32 t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        u32 run = offsets[count_index(ls, set, l, k_in_set)] + incl - sum;
-#pragma unroll
-        for (int q = 0; q < kThreads / 32; ++q) {
-            s_rank[l][lane * (kThreads / 32) + q] = run;
-            run += v[q];
-        }
-    }
-    __syncthreads();
-    for (int k = 0; k < kItems; ++k) {
-        const u32 q = i0 + k;
-        if (q >= cnt) break;
-        const u32 e = e0 + q;
-        const Key a = K[e], b = K[e + 1];
-        const int ll = leaf_level(b - a);
-        const u32 x = s_rank[ll][tid]++;
-        if (x < n_nodes) {
-            NK[x] = placeholder(a, ll);
-            leaf_to_node[e] = static_cast<int>(x);
-        }
-        if (b != kKeyEnd) {
-            const int pl = pair_level(a, b);
-            if (pl >= 0) {
-                const u32 y = s_rank[pl][tid]++;
-                if (y < n_nodes) NK[y] = placeholder(a, pl);
-            }
-        }
-    }
-}
-
-__global__ void __launch_bounds__(kThreads) link_b_child_kernel(const Key* __restrict__ NK, u32 node_cap, int n_sets,
-                                                                const int* __restrict__ LO, int* __restrict__ CO) {
-    const u32 last = static_cast<u32>(LO[n_sets * (kNumLevels + 1) - 1]);  // nodes of all sets
-    const u32 n_nodes = last < node_cap ? last : node_cap;
-    for (u32 x = blockIdx.x * kThreads + threadIdx.x; x < n_nodes; x += gridDim.x * kThreads) {
-        int lo_s = 0, hi_s = n_sets;  // set whose node block contains x
-        while (hi_s - lo_s > 1) {
-            const int mid = (lo_s + hi_s) >> 1;
-            if (static_cast<u32>(LO[mid * (kNumLevels + 1)]) <= x)
-                lo_s = mid;
-            else
-                hi_s = mid;
-        }
-        const int* row = LO + lo_s * (kNumLevels + 1);
-        const Key k = NK[x];
-        const int level = (kWordBits - 1 - key_clz(k)) / 3;
-        int c = 0;
-        if (level < kLevels) {
-            const Key want = k << 3;
-            u32 lo = min(static_cast<u32>(row[level + 1]), n_nodes);
-            u32 hi = min(static_cast<u32>(row[level + 2]), n_nodes);
-            const u32 end = hi;
-            while (lo < hi) {
-                const u32 mid = lo + ((hi - lo) >> 1);
-                if (NK[mid] < want)
-                    lo = mid + 1;
-                else
-                    hi = mid;
-            }
-            if (lo < end && NK[lo] == want) c = static_cast<int>(lo);
-        }
-        CO[x] = c;
-    }
+                                                                  const u32* __restrict__ offsets,
+                                                                  const u32* __restrict__ pair_offsets, Out o) {
+    Tile t;
+    if (batched_tile(ls, t)) place_tile<ITEMS, COUNTS>(K, t, offsets, pair_offsets, o);
 }
 
 struct LinkBLayout {
     LinkSets ls;
-    u32* counts;   // [max_tiles * 22 + 1]: (set, level, tile) counts, their exclusive scan, the total
-    u32* partial;  // [chunks] chunk sums of the scan
+    u32* counts;   // 2 x [max_tiles * 22 + 1]: (set, level, tile) counts of all nodes and of internal nodes,
+                   // their exclusive scans, the totals
+    u32* partial;  // [2][chunks] chunk sums of the scans
     u32 max_tiles;
     u32 chunks;
     size_t bytes;
@@ -536,7 +566,8 @@ struct LinkBLayout {
 LinkBLayout link_b_layout(void* ws, long long n_elements, int n_sets) {
     LinkBLayout l;
     Carver c(ws);
-    l.max_tiles = static_cast<u32>((n_elements + kTile - 1) / kTile + n_sets);
+    l.ls.tile = static_cast<u32>(kThreads * items_of(n_elements));
+    l.max_tiles = static_cast<u32>((n_elements + l.ls.tile - 1) / l.ls.tile + n_sets);
     l.ls.n_tiles = c.take<u32>(1);
     l.ls.tile_first = c.take<u32>((size_t)n_sets + 1);
     l.ls.tile_set = c.take<u32>(l.max_tiles);
@@ -545,76 +576,119 @@ LinkBLayout link_b_layout(void* ws, long long n_elements, int n_sets) {
     l.ls.node_first = c.take<u32>((size_t)n_sets + 1);
     l.ls.n_sets = n_sets;
     l.ls.elem_offsets = nullptr;
-    l.counts = c.take<u32>((size_t)l.max_tiles * kNumLevels + 1);
+    l.counts = c.take<u32>(2 * ((size_t)l.max_tiles * kNumLevels + 1));
     l.chunks = static_cast<u32>(((size_t)l.max_tiles * kNumLevels + kScanChunk - 1) / kScanChunk);
-    l.partial = c.take<u32>(l.chunks);
+    l.partial = c.take<u32>((size_t)2 * l.chunks);
     l.bytes = c.size();
     return l;
 }
 
 }  // namespace
 
-size_t link_batched_ws_bytes(long long n_elements, int n_sets) { return link_b_layout(nullptr, n_elements, n_sets).bytes; }
+size_t link_batched_ws_bytes(long long n_elements, int n_sets) {
+    return link_b_layout(nullptr, n_elements, n_sets).bytes;
+}
 
 int launch_link_batched(const Key* K, long long n_elements, const long long* elem_offsets, int n_sets, Key* NK,
-                        int* CO, int* LO, int* leaf_to_node, long long n_nodes, void* ws, cudaStream_t st) {
+                        int* CO, int* LO, int* leaf_to_node, long long n_nodes, const u32* leaf_offsets,
+                        u32* node_counts, void* ws, cudaStream_t st) {
     LinkBLayout l = link_b_layout(ws, n_elements, n_sets);
     l.ls.elem_offsets = elem_offsets;
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
+    const u32 len = l.max_tiles * kNumLevels;  // unused tail entries are zero
+    const size_t stride = (size_t)len + 1;
     CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
-    CST_CUDA(cudaMemsetAsync(l.counts, 0, ((size_t)l.max_tiles * kNumLevels + 1) * sizeof(u32), st));
+    CST_CUDA(cudaMemsetAsync(l.counts, 0, 2 * stride * sizeof(u32), st));
     link_b_setup_kernel<<<1, 1024, 0, st>>>(l.ls);
     CST_LAUNCHED("link_b_setup_kernel");
-    const long long want = (l.max_tiles + kThreads - 1) / kThreads;
+    // a thread per tile, and enough threads for the -1 entries of the capacity beyond the elements
+    const long long fill = n_elements / 8 > l.max_tiles ? n_elements / 8 : l.max_tiles;
+    const long long want = (fill + kThreads - 1) / kThreads;
     const int tgrid = static_cast<int>(want < (long long)sm_count() * 4 ? want : (long long)sm_count() * 4);
     link_b_tiles_kernel<<<tgrid, kThreads, 0, st>>>(l.ls, l.max_tiles, static_cast<u32>(n_elements), leaf_to_node);
     CST_LAUNCHED("link_b_tiles_kernel");
-    link_b_count_kernel<<<l.max_tiles, kThreads, 0, st>>>(K, l.ls, l.counts);
+    u32* pairs = l.counts + stride;
+    const bool small = l.ls.tile == static_cast<u32>(kThreads * kItemsSmall);
+    if (small)
+        link_b_count_kernel<kItemsSmall><<<l.max_tiles, kThreads, 0, st>>>(K, l.ls, l.counts, pairs);
+    else
+        link_b_count_kernel<kItemsLarge><<<l.max_tiles, kThreads, 0, st>>>(K, l.ls, l.counts, pairs);
     CST_LAUNCHED("link_b_count_kernel");
-    // one exclusive scan over all (set, level, tile) counts; unused tail entries are zero
-    const u32 len = l.max_tiles * kNumLevels;
-    link_scan_reduce_kernel<<<dim3(l.chunks, 1), kScanThreads, 0, st>>>(l.counts, len, l.partial);
+    link_scan_reduce_kernel<<<dim3(l.chunks, 2), kScanThreads, 0, st>>>(l.counts, len, stride, l.partial);
     CST_LAUNCHED("link_scan_reduce_kernel");
-    link_scan_apply_kernel<<<dim3(l.chunks, 1), kScanThreads, 0, st>>>(l.counts, len, 1u, l.partial, nullptr, 0u, hdr);
+    link_scan_apply_kernel<<<dim3(l.chunks, 2), kScanThreads, 0, st>>>(l.counts, len, stride, 1u, l.partial, nullptr,
+                                                                        0u, hdr);
     CST_LAUNCHED("link_scan_apply_kernel");
     const int lo_threads = n_sets * (kNumLevels + 1);
     link_b_lo_kernel<<<(lo_threads + 255) / 256, 256, 0, st>>>(l.counts, l.ls, LO, leaf_to_node, hdr);
     CST_LAUNCHED("link_b_lo_kernel");
-    link_b_scatter_kernel<<<l.max_tiles, kThreads, 0, st>>>(K, l.ls, l.counts, static_cast<u32>(n_nodes), NK,
-                                                            leaf_to_node);
+    const Out o{static_cast<u32>(n_nodes), NK, leaf_to_node, CO, nullptr, leaf_offsets, node_counts};
+    auto* scatter = small ? (node_counts ? link_b_scatter_kernel<kItemsSmall, true>
+                                         : link_b_scatter_kernel<kItemsSmall, false>)
+                          : (node_counts ? link_b_scatter_kernel<kItemsLarge, true>
+                                         : link_b_scatter_kernel<kItemsLarge, false>);
+    scatter<<<l.max_tiles, kThreads, 0, st>>>(K, l.ls, l.counts, pairs, o);
     CST_LAUNCHED("link_b_scatter_kernel");
-    const long long wantc = (n_nodes + kThreads - 1) / kThreads;
-    const int cgrid = static_cast<int>(wantc < (long long)sm_count() * 8 ? (wantc > 0 ? wantc : 1) : (long long)sm_count() * 8);
-    link_b_child_kernel<<<cgrid, kThreads, 0, st>>>(NK, static_cast<u32>(n_nodes), n_sets, LO, CO);
-    CST_LAUNCHED("link_b_child_kernel");
     return CSTONE_OK;
 }
-
-namespace {
-}  // namespace
 
 size_t link_ws_bytes(long long nl) { return link_layout(nullptr, nl).bytes; }
 
-int launch_link(const Key* K, long long nl, Key* NK, int* CO, int* LO, int* leaf_to_node, int* parent, void* ws,
-                cudaStream_t st) {
+int launch_link(const Key* K, long long nl, Key* NK, int* CO, int* LO, int* leaf_to_node, int* parent,
+                const u32* leaf_offsets, u32* node_counts, void* ws, cudaStream_t st) {
     LinkLayout l = link_layout(ws, nl);
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader), st));
-    const u32 n_nodes = static_cast<u32>(nl + (nl - 1) / 7);
+    const u32 n_nodes = static_cast<u32>(nl + (nl - 1) / 7), n = static_cast<u32>(nl);
     const u32 len = l.ntiles * kNumLevels;
-    u32* pair_counts = l.counts + len;
-    link_count_kernel<<<l.ntiles, kThreads, 0, st>>>(K, static_cast<u32>(nl), l.ntiles, l.counts, pair_counts);
+    u32* pairs = l.counts + len;
+    const bool small = items_of(nl) == kItemsSmall;
+    if (small)
+        link_count_kernel<kItemsSmall><<<l.ntiles, kThreads, 0, st>>>(K, n, l.counts, pairs);
+    else
+        link_count_kernel<kItemsLarge><<<l.ntiles, kThreads, 0, st>>>(K, n, l.counts, pairs);
     CST_LAUNCHED("link_count_kernel");
-    link_scan_reduce_kernel<<<dim3(l.chunks, 2), kScanThreads, 0, st>>>(l.counts, len, l.partial);
+    link_scan_reduce_kernel<<<dim3(l.chunks, 2), kScanThreads, 0, st>>>(l.counts, len, len, l.partial);
     CST_LAUNCHED("link_scan_reduce_kernel");
-    link_scan_apply_kernel<<<dim3(l.chunks, 2), kScanThreads, 0, st>>>(l.counts, len, l.ntiles, l.partial, LO, n_nodes,
-                                                                        hdr);
+    link_scan_apply_kernel<<<dim3(l.chunks, 2), kScanThreads, 0, st>>>(l.counts, len, len, l.ntiles, l.partial, LO,
+                                                                        n_nodes, hdr);
     CST_LAUNCHED("link_scan_apply_kernel");
-    link_scatter_kernel<<<l.ntiles, kThreads, 0, st>>>(K, static_cast<u32>(nl), l.ntiles, l.counts, pair_counts,
-                                                       n_nodes, NK, leaf_to_node, CO, parent);
+    const Out o{n_nodes, NK, leaf_to_node, CO, parent, leaf_offsets, node_counts};
+    auto* scatter = small ? (node_counts ? link_scatter_kernel<kItemsSmall, true>
+                                         : link_scatter_kernel<kItemsSmall, false>)
+                          : (node_counts ? link_scatter_kernel<kItemsLarge, true>
+                                         : link_scatter_kernel<kItemsLarge, false>);
+    scatter<<<l.ntiles, kThreads, 0, st>>>(K, n, l.counts, pairs, o);
     CST_LAUNCHED("link_scatter_kernel");
     return CSTONE_OK;
 }
+
+// The linked tree, with its node counts when node_counts is given (then leaf_offsets [n_leaves + 1] too).
+int link_tree(const char* who, const void* leaves, long long n_leaves, void* node_keys, int* child, int* level_offsets,
+              int* leaf_to_node, int* parent, const u32* leaf_offsets, u32* node_counts, void* ws, size_t ws_bytes,
+              cudaStream_t st) {
+    if (n_leaves < 1 || n_leaves > CSTONE_MAX_LEAVES || (n_leaves - 1) % 7 != 0 || !leaves || !node_keys || !child ||
+        !level_offsets || !leaf_to_node || (node_counts && !leaf_offsets))
+        return cst::fail(CSTONE_ERR_INVALID_ARG, "%s: bad argument (n_leaves=%lld must be 1 + 7k, arrays non-NULL)",
+                         who, n_leaves);
+    if (int rc = cst::check_ws(ws, ws_bytes, link_ws_bytes(n_leaves), who)) return rc;
+    return launch_link(static_cast<const Key*>(leaves), n_leaves, static_cast<Key*>(node_keys), child, level_offsets,
+                       leaf_to_node, parent, leaf_offsets, node_counts, ws, st);
+}
+
+#ifndef CSTONE_KEY32  // batched builds exist for 63-bit keys only
+int link_tree_batched(const char* who, const u64* elements, long long n_elements, const long long* element_offsets,
+                      int n_sets, long long n_nodes, u64* node_keys, int* child, int* level_offsets, int* leaf_to_node,
+                      const u32* leaf_offsets, u32* node_counts, void* ws, size_t ws_bytes, cudaStream_t st) {
+    if (n_sets < 1 || n_sets > (1 << 20) || n_elements < 2 * (long long)n_sets || n_elements > CSTONE_MAX_LEAVES ||
+        n_nodes < n_sets || n_nodes > 2 * (long long)CSTONE_MAX_LEAVES || !elements || !element_offsets ||
+        !node_keys || !child || !level_offsets || !leaf_to_node || (node_counts && !leaf_offsets))
+        return cst::fail(CSTONE_ERR_INVALID_ARG, "%s: bad argument", who);
+    if (int rc = cst::check_ws(ws, ws_bytes, link_batched_ws_bytes(n_elements, n_sets), who)) return rc;
+    return launch_link_batched(elements, n_elements, element_offsets, n_sets, node_keys, child, level_offsets,
+                               leaf_to_node, n_nodes, leaf_offsets, node_counts, ws, st);
+}
+#endif
 
 }  // namespace CST_NS
 
@@ -630,16 +704,8 @@ int CSTONE_FN(link_workspace_size)(int64_t n_leaves, size_t* bytes) {
 int CSTONE_FN(link_tree)(const CST_KEY_C* leaves, int64_t n_leaves, CST_KEY_C* node_keys, int32_t* child,
                          int32_t* level_offsets, int32_t* leaf_to_node, int32_t* parent, void* ws, size_t ws_bytes,
                          void* stream) {
-    if (n_leaves < 1 || n_leaves > CSTONE_MAX_LEAVES || (n_leaves - 1) % 7 != 0 || !leaves || !node_keys || !child ||
-        !level_offsets || !leaf_to_node)
-        return cst::fail(CSTONE_ERR_INVALID_ARG,
-                         CST_STR(CSTONE_FN(link_tree)) ": bad argument (n_leaves=%lld must be 1 + 7k, arrays non-NULL)",
-                         (long long)n_leaves);
-    if (int rc = cst::check_ws(ws, ws_bytes, CST_NS::link_ws_bytes(n_leaves), CST_STR(CSTONE_FN(link_tree))))
-        return rc;
-    return CST_NS::launch_link(reinterpret_cast<const CST_NS::Key*>(leaves), n_leaves,
-                               reinterpret_cast<CST_NS::Key*>(node_keys), child, level_offsets, leaf_to_node, parent,
-                               ws, cst::as_stream(stream));
+    return CST_NS::link_tree(CST_STR(CSTONE_FN(link_tree)), leaves, n_leaves, node_keys, child, level_offsets,
+                             leaf_to_node, parent, nullptr, nullptr, ws, ws_bytes, cst::as_stream(stream));
 }
 
 #ifndef CSTONE_KEY32  // batched builds exist for 63-bit keys only
@@ -654,17 +720,10 @@ int cstone_link_batched_workspace_size(int64_t n_elements, int32_t n_sets, size_
 int cstone_link_tree_batched(const uint64_t* elements, int64_t n_elements, const int64_t* element_offsets,
                              int32_t n_sets, int64_t n_nodes, uint64_t* node_keys, int32_t* child,
                              int32_t* level_offsets, int32_t* leaf_to_node, void* ws, size_t ws_bytes, void* stream) {
-    if (n_sets < 1 || n_sets > (1 << 20) || n_elements < 2 * (int64_t)n_sets || n_elements > CSTONE_MAX_LEAVES ||
-        n_nodes < n_sets || n_nodes > 2 * (int64_t)CSTONE_MAX_LEAVES || !elements || !element_offsets ||
-        !node_keys || !child || !level_offsets || !leaf_to_node)
-        return cst::fail(CSTONE_ERR_INVALID_ARG, "cstone_link_tree_batched: bad argument");
-    if (int rc = cst::check_ws(ws, ws_bytes, cst::link_batched_ws_bytes(n_elements, n_sets),
-                               "cstone_link_tree_batched"))
-        return rc;
-    return cst::launch_link_batched(reinterpret_cast<const cst::u64*>(elements), n_elements,
-                                    reinterpret_cast<const long long*>(element_offsets), n_sets,
-                                    reinterpret_cast<cst::u64*>(node_keys), child, level_offsets, leaf_to_node,
-                                    n_nodes, ws, cst::as_stream(stream));
+    return cst::link_tree_batched("cstone_link_tree_batched", reinterpret_cast<const cst::u64*>(elements), n_elements,
+                                  reinterpret_cast<const long long*>(element_offsets), n_sets, n_nodes,
+                                  reinterpret_cast<cst::u64*>(node_keys), child, level_offsets, leaf_to_node, nullptr,
+                                  nullptr, ws, ws_bytes, cst::as_stream(stream));
 }
 
 #endif

@@ -8,6 +8,11 @@
 #include "common.cuh"
 
 namespace CST_NS {
+
+int link_tree(const char* who, const void* leaves, long long n_leaves, void* node_keys, int* child, int* level_offsets,
+              int* leaf_to_node, int* parent, const u32* leaf_offsets, u32* node_counts, void* ws, size_t ws_bytes,
+              cudaStream_t st);
+
 namespace {
 
 inline size_t larger(size_t a, size_t b) { return a > b ? a : b; }
@@ -30,7 +35,8 @@ int CSTONE_FN(build_set_workspace_size)(int64_t n, int64_t leaf_cap, int32_t max
 
 int CSTONE_FN(build_set)(const cstone_set_input* in, const cstone_set_params* prm, const cstone_set_buffers* out,
                          int64_t* n_leaves, int32_t* iters, void* ws, size_t ws_bytes, void* stream) {
-    if (!in || !prm || !out || !n_leaves || (in->m && (!out->records || !out->records_ws)) || (!in->box && !out->box_out))
+    if (!in || !prm || !out || !n_leaves || (in->m && (!out->records || !out->records_ws)) ||
+        (!in->box && !out->box_out))
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(build_set)) ": bad argument");
     const double* box = in->box;
     CST_KEY_C* keys = static_cast<CST_KEY_C*>(out->keys);
@@ -47,32 +53,29 @@ int CSTONE_FN(build_set)(const cstone_set_input* in, const cstone_set_params* pr
         return rc;
     }
     if (int rc = CSTONE_FN(sort)(keys, sorted, out->perm, in->n, ws, ws_bytes, stream)) return rc;
-    return CSTONE_FN(build_leaves)(sorted, in->n, prm->ncrit, static_cast<CST_KEY_C*>(out->leaves), out->leaf_cap, n_leaves,
-                                   out->leaf_counts, out->leaf_offsets, prm->max_iters, iters, ws, ws_bytes, stream);
+    return CSTONE_FN(build_leaves)(sorted, in->n, prm->ncrit, static_cast<CST_KEY_C*>(out->leaves), out->leaf_cap,
+                                   n_leaves, out->leaf_counts, out->leaf_offsets, prm->max_iters, iters, ws, ws_bytes,
+                                   stream);
 }
 
 int CSTONE_FN(build_tree_workspace_size)(int64_t n_leaves, int32_t with_masses, size_t* bytes) {
     if (!bytes)
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(build_tree_workspace_size)) ": bad argument");
-    size_t link = 0, counts = 0, moments = 0;
+    size_t link = 0, moments = 0;
     if (int rc = CSTONE_FN(link_workspace_size)(n_leaves, &link)) return rc;
-    if (int rc = CSTONE_FN(upsweep_workspace_size)(n_leaves, &counts)) return rc;
     if (with_masses)
         if (int rc = CSTONE_FN(multipole_workspace_size)(0, n_leaves, &moments)) return rc;
-    *bytes = CST_NS::larger(link, CST_NS::larger(counts, moments));
+    *bytes = CST_NS::larger(link, moments);
     return CSTONE_OK;
 }
 
 int CSTONE_FN(build_tree)(const cstone_set_buffers* set, int64_t n, int64_t n_leaves, const double* box,
                           const cstone_tree_buffers* out, void* ws, size_t ws_bytes, void* stream) {
-    if (!set || !out || (out->mass && (!box || !set->records)))
+    if (!set || !out || !set->leaf_offsets || !out->node_counts || (out->mass && (!box || !set->records)))
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(build_tree)) ": bad argument");
-    if (int rc = CSTONE_FN(link_tree)(static_cast<const CST_KEY_C*>(set->leaves), n_leaves,
-                                      static_cast<CST_KEY_C*>(out->node_keys), out->child, out->level_offsets,
-                                      out->leaf_to_node, out->parent, ws, ws_bytes, stream))
-        return rc;
-    if (int rc = CSTONE_FN(upsweep_counts)(set->leaf_counts, n_leaves, out->leaf_to_node, out->child, out->level_offsets,
-                                           out->node_counts, ws, ws_bytes, stream))
+    if (int rc = CST_NS::link_tree(CST_STR(CSTONE_FN(build_tree)), set->leaves, n_leaves, out->node_keys, out->child,
+                                   out->level_offsets, out->leaf_to_node, out->parent, set->leaf_offsets,
+                                   out->node_counts, ws, ws_bytes, cst::as_stream(stream)))
         return rc;
     if (!out->mass) return CSTONE_OK;
     return CSTONE_FN(upsweep_multipoles_records)(set->records, set->perm, n, set->leaf_offsets, n_leaves,

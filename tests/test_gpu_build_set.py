@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("levels", [21, 10])
-@pytest.mark.parametrize("n,ncrit", [(1, 1), (1000, 16), (4096, 5000), (70001, 8)])
+@pytest.mark.parametrize("n,ncrit", [(1, 1), (1000, 16), (4096, 5000), (70001, 8), (3_000_000, 8)])
 @pytest.mark.parametrize("boxed,masses,cap", [(False, True, 0), (True, False, 0), (True, True, 1)])
 def test_build_octree_equals_single_calls(lib, levels, n, ncrit, boxed, masses, cap):
     rng = np.random.default_rng(n + levels)

@@ -68,20 +68,27 @@ struct Tile {
 // One counter word per thread and level: all nodes in the low half, internal nodes in the high half (a tile
 // has at most 2 * 2048 nodes, so neither its sums nor its ranks overflow a half).
 constexpr u32 kLeafOne = 1u, kInternalOne = 0x10001u;
+// A row of them has a gap after every 8 threads, so that neither a thread per column nor a lane per 8
+// columns meets bank conflicts.
+constexpr int kRow = kThreads + kThreads / 8;
+__device__ __forceinline__ int column(int thread) { return thread + (thread >> 3); }
 
+// Counts a thread's items by level; `levels` keeps each leaf's level and its pair's (kNoPair: none) << 8.
+constexpr u32 kNoPair = 255u;
 template <int ITEMS>
 __device__ __forceinline__ void count_items(const Key (&key)[ITEMS + 1], u32 i0, const Tile& t,
-                                            u32 (*s_rank)[kThreads]) {
+                                            u32 (*s_rank)[kRow], u32 (&levels)[ITEMS]) {
+    const int me = column(threadIdx.x);
 #pragma unroll
-    for (int l = 0; l < kNumLevels; ++l) s_rank[l][threadIdx.x] = 0;
+    for (int l = 0; l < kNumLevels; ++l) s_rank[l][me] = 0;
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
         if (i0 + k >= t.e0 + t.cnt) break;
-        s_rank[leaf_level(key[k + 1] - key[k])][threadIdx.x] += kLeafOne;
-        if (i0 + k + 1 < t.hi) {
-            const int pl = pair_level(key[k], key[k + 1]);
-            if (pl >= 0) s_rank[pl][threadIdx.x] += kInternalOne;
-        }
+        const int ll = leaf_level(key[k + 1] - key[k]);
+        const int pl = i0 + k + 1 < t.hi ? pair_level(key[k], key[k + 1]) : -1;
+        s_rank[ll][me] += kLeafOne;
+        if (pl >= 0) s_rank[pl][me] += kInternalOne;
+        levels[k] = static_cast<u32>(ll) | (pl >= 0 ? static_cast<u32>(pl) : kNoPair) << 8;
     }
 }
 
@@ -94,17 +101,18 @@ __device__ __forceinline__ void load_items(const Key* __restrict__ K, u32 i0, co
 template <int ITEMS>
 __device__ __forceinline__ void count_tile(const Key* __restrict__ K, const Tile& t, u32* __restrict__ counts,
                                            u32* __restrict__ pair_counts) {
-    __shared__ u32 s_rank[kNumLevels][kThreads];  // own column per thread, no conflicts
+    __shared__ u32 s_rank[kNumLevels][kRow];
     const u32 i0 = t.e0 + threadIdx.x * ITEMS;
     Key key[ITEMS + 1];
+    u32 levels[ITEMS];
     load_items<ITEMS>(K, i0, t, key);
-    count_items<ITEMS>(key, i0, t, s_rank);
+    count_items<ITEMS>(key, i0, t, s_rank, levels);
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int l = warp; l < kNumLevels; l += kThreads / 32) {
         u32 v = 0;
 #pragma unroll
-        for (int q = 0; q < kThreads / 32; ++q) v += s_rank[l][q * 32 + lane];
+        for (int q = 0; q < kThreads / 32; ++q) v += s_rank[l][column(q * 32 + lane)];
         for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         if (lane == 0) {
             counts[t.counter(l)] = v & 0xffffu;
@@ -166,25 +174,35 @@ struct Out {
     u32* node_counts;
 };
 
-// Places a tile's leaves and internal nodes in breadth-first order, in in-order sequence: leaf i, then the
-// internal node of pair i; the g-th internal node of the set has its children at 8 g + 1 of the set's nodes.
+// Places a tile's leaves and internal nodes in breadth-first order. Each thread ranks its leaves and pairs
+// in in-order sequence (leaf i, then the internal node of pair i). With 8 leaves per thread it lists them by
+// level in shared memory, and the nodes are then written from that list, a thread each, so that the lanes of a
+// warp write neighbouring nodes: written from the ranking loop, the eight stores of a warp to one sector were
+// eight transactions (7.6 million leaves: 204 us, listed 150; 1.7 million 64 and 43). With 2 it writes them as it
+// ranks them (the list costs 2 us where the whole takes 10). Six blocks per SM hide the searches' chains of
+// loads better than five (43 us against 51). The g-th internal node of the set has its children at 8 g + 1 of the
+// set's nodes.
 template <int ITEMS, bool COUNTS>
 __device__ __forceinline__ void place_tile(const Key* __restrict__ K, const Tile& t, const u32* __restrict__ offsets,
                                            const u32* __restrict__ pair_offsets, const Out& o) {
-    constexpr u32 kList = COUNTS ? kThreads * ITEMS / 8 + 64 : 1;
-    __shared__ u32 s_rank[kNumLevels][kThreads];  // per-thread counts, then per-thread ranks within the tile
+    constexpr bool kListed = ITEMS > kItemsSmall;
+    constexpr u32 kList = kThreads * ITEMS / 8 + 64;
+    __shared__ u32 s_rank[kNumLevels][kRow];      // per-thread counts, then per-thread ranks within the tile
     __shared__ u32 s_base[2][kNumLevels];         // the tile's first node and internal node of each level
-    __shared__ uint2 s_list[kList];               // internal nodes (node, leaf of the pair) for the counts
+    __shared__ u32 s_start[kNumLevels];           // nodes of the tile at the levels before
+    __shared__ unsigned short s_slot[kListed ? 2 * kThreads * ITEMS : 1];  // by level: 2 x leaf in the tile, + 1: pair
+    __shared__ uint2 s_list[kList];               // internal nodes: node, leaf | rank among the level's << 16
     __shared__ u32 s_listed;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, me = column(tid);
     const u32 i0 = t.e0 + tid * ITEMS;
     Key key[ITEMS + 1];
+    u32 levels[ITEMS];
     load_items<ITEMS>(K, i0, t, key);
     if (tid == 0) s_listed = 0;
     if (tid < kNumLevels) s_base[0][tid] = offsets[t.counter(tid)];
     if (tid >= 32 && tid < 32 + kNumLevels) s_base[1][tid - 32] = pair_offsets[t.counter(tid - 32)];
     const u32 first_node = offsets[t.first * kNumLevels], first_internal = pair_offsets[t.first * kNumLevels];
-    count_items<ITEMS>(key, i0, t, s_rank);
+    count_items<ITEMS>(key, i0, t, s_rank, levels);
     __syncthreads();
     // exclusive scan of every level row across the threads
     for (int l = warp; l < kNumLevels; l += kThreads / 32) {
@@ -192,7 +210,7 @@ __device__ __forceinline__ void place_tile(const Key* __restrict__ K, const Tile
         u32 sum = 0;
 #pragma unroll
         for (int q = 0; q < kThreads / 32; ++q) {
-            v[q] = s_rank[l][lane * (kThreads / 32) + q];
+            v[q] = s_rank[l][column(lane * (kThreads / 32) + q)];
             sum += v[q];
         }
         u32 incl = sum;
@@ -200,62 +218,91 @@ __device__ __forceinline__ void place_tile(const Key* __restrict__ K, const Tile
             const u32 w = __shfl_up_sync(0xffffffffu, incl, s);
             if (lane >= s) incl += w;
         }
+        if (kListed && lane == 31) s_start[l] = incl & 0xffffu;
         u32 run = incl - sum;
 #pragma unroll
         for (int q = 0; q < kThreads / 32; ++q) {
-            s_rank[l][lane * (kThreads / 32) + q] = run;
+            s_rank[l][column(lane * (kThreads / 32) + q)] = run;
             run += v[q];
         }
     }
     __syncthreads();
+    if (kListed && warp == 0) {  // the levels' totals to their starts
+        const u32 own = lane < kNumLevels ? s_start[lane] : 0u;
+        u32 incl = own;
+        for (int s = 1; s < 32; s <<= 1) {
+            const u32 w = __shfl_up_sync(0xffffffffu, incl, s);
+            if (lane >= s) incl += w;
+        }
+        if (lane < kNumLevels) s_start[lane] = incl - own;
+    }
+    if (kListed) __syncthreads();
+    auto leaf = [&](u32 x, u32 i, Key a, int level) {
+        if (x >= o.n_nodes) return;
+        o.NK[x] = placeholder(a, level);
+        o.CO[x] = 0;
+        o.leaf_to_node[i] = static_cast<int>(x);
+        if (COUNTS) o.node_counts[x] = o.leaf_offsets[i + 1] - o.leaf_offsets[i];
+    };
+    // CO, parent and count of internal node y of pair i, the r-th internal node of the tile at its level
+    auto internal = [&](u32 y, u32 i, Key a, int level, u32 r) {
+        if (y >= o.n_nodes) return;
+        const u32 g = s_base[1][level] + r - first_internal;
+        const u32 c = first_node + 8u * g + 1u;
+        const bool inside = c + 7u < o.n_nodes;
+        if (!kListed) o.NK[y] = placeholder(a, level);
+        o.CO[y] = inside ? static_cast<int>(c) : 0;
+        if (o.parent && inside) o.parent[g] = static_cast<int>(y);
+        if (COUNTS) {
+            const uint2 range = covered(K, t, i, a, level);
+            o.node_counts[y] = o.leaf_offsets[range.y] - o.leaf_offsets[range.x];
+        }
+    };
 #pragma unroll
     for (int k = 0; k < ITEMS; ++k) {
         const u32 i = i0 + k;
         if (i >= t.e0 + t.cnt) break;
-        const Key a = key[k], b = key[k + 1];
-        const int ll = leaf_level(b - a);
-        const u32 rx = s_rank[ll][tid];
-        s_rank[ll][tid] = rx + kLeafOne;
-        const u32 x = s_base[0][ll] + (rx & 0xffffu);
-        if (x < o.n_nodes) {
-            o.NK[x] = placeholder(a, ll);
-            o.CO[x] = 0;
-            o.leaf_to_node[i] = static_cast<int>(x);
-            if (COUNTS) o.node_counts[x] = o.leaf_offsets[i + 1] - o.leaf_offsets[i];
-        }
-        const int pl = i + 1 < t.hi ? pair_level(a, b) : -1;
-        if (pl >= 0) {
-            const u32 ry = s_rank[pl][tid];
-            s_rank[pl][tid] = ry + kInternalOne;
+        const u32 item = 2u * (tid * ITEMS + k);
+        const u32 ll = levels[k] & 255u, pl = levels[k] >> 8;
+        const u32 rx = s_rank[ll][me];
+        s_rank[ll][me] = rx + kLeafOne;
+        if (kListed)
+            s_slot[s_start[ll] + (rx & 0xffffu)] = static_cast<unsigned short>(item);
+        else
+            leaf(s_base[0][ll] + (rx & 0xffffu), i, key[k], static_cast<int>(ll));
+        if (pl != kNoPair) {
+            const u32 ry = s_rank[pl][me];
+            s_rank[pl][me] = ry + kInternalOne;
+            if (kListed) s_slot[s_start[pl] + (ry & 0xffffu)] = static_cast<unsigned short>(item + 1u);
             const u32 y = s_base[0][pl] + (ry & 0xffffu);
-            const u32 g = s_base[1][pl] + (ry >> 16) - first_internal;
-            const u32 c = first_node + 8u * g + 1u;
-            if (y < o.n_nodes) {
-                const bool inside = c + 7u < o.n_nodes;
-                o.NK[y] = placeholder(a, pl);
-                o.CO[y] = inside ? static_cast<int>(c) : 0;
-                if (o.parent && inside) o.parent[g] = static_cast<int>(y);
-                if (COUNTS) {
-                    const u32 at = atomicAdd(&s_listed, 1u);
-                    if (at < kList) {
-                        s_list[at] = make_uint2(y, i);
-                    } else {
-                        const uint2 r = covered(K, t, i, a, pl);
-                        o.node_counts[y] = o.leaf_offsets[r.y] - o.leaf_offsets[r.x];
-                    }
-                }
-            }
+            const u32 at = atomicAdd(&s_listed, 1u);
+            if (at < kList)
+                s_list[at] = make_uint2(y, (item >> 1) | (ry & 0xffff0000u));
+            else
+                internal(y, i, key[k], static_cast<int>(pl), ry >> 16);
         }
     }
-    if (!COUNTS) return;
-    // the searches of the tile's internal nodes (one leaf in seven has one) side by side, not one lane at a time
     __syncthreads();
+    if (kListed) {
+        const u32 nodes = s_start[kNumLevels - 1] + (s_rank[kNumLevels - 1][column(kThreads - 1)] & 0xffffu);
+        for (u32 p = tid; p < nodes; p += kThreads) {
+            const u32 item = s_slot[p], i = t.e0 + (item >> 1);
+            const Key a = K[i], b = K[i + 1];
+            const int level = (item & 1u) ? pair_level(a, b) : leaf_level(b - a);
+            const u32 x = s_base[0][level] + (p - s_start[level]);
+            if ((item & 1u) == 0u)
+                leaf(x, i, a, level);
+            else if (x < o.n_nodes)
+                o.NK[x] = placeholder(a, level);
+        }
+    }
+    // the internal nodes (one leaf in seven has one) side by side, not one lane of a warp at a time
     const u32 listed = min(s_listed, kList);
     for (u32 q = tid; q < listed; q += kThreads) {
-        const uint2 yi = s_list[q];
-        const Key a = K[yi.y];
-        const uint2 r = covered(K, t, yi.y, a, pair_level(a, K[yi.y + 1]));
-        o.node_counts[yi.x] = o.leaf_offsets[r.y] - o.leaf_offsets[r.x];
+        const uint2 e = s_list[q];
+        const u32 i = t.e0 + (e.y & 0xffffu);
+        const Key a = K[i];
+        internal(e.x, i, a, pair_level(a, K[i + 1]), e.y >> 16);
     }
 }
 
@@ -272,7 +319,7 @@ __global__ void __launch_bounds__(kThreads) link_count_kernel(const Key* __restr
 }
 
 template <int ITEMS, bool COUNTS>
-__global__ void __launch_bounds__(kThreads) link_scatter_kernel(const Key* __restrict__ K, u32 nl,
+__global__ void __launch_bounds__(kThreads, 6) link_scatter_kernel(const Key* __restrict__ K, u32 nl,
                                                                 const u32* __restrict__ offsets,
                                                                 const u32* __restrict__ pair_offsets, Out o) {
     place_tile<ITEMS, COUNTS>(K, single_tile<ITEMS>(nl), offsets, pair_offsets, o);
@@ -500,26 +547,24 @@ __device__ __forceinline__ u32 count_index(const LinkSets& ls, u32 set, int leve
     return tf * kNumLevels + static_cast<u32>(level) * nt + k;
 }
 
-// The block's tile; false when there is none.
-__device__ __forceinline__ bool batched_tile(const LinkSets& ls, Tile& t) {
-    t.cnt = ls.tile_count[blockIdx.x];
-    if (t.cnt == 0) return false;
-    const u32 set = ls.tile_set[blockIdx.x];
-    t.e0 = ls.tile_elem[blockIdx.x];
+__device__ __forceinline__ Tile batched_tile(const LinkSets& ls, u32 tile) {
+    const u32 set = ls.tile_set[tile];
+    Tile t;
+    t.cnt = ls.tile_count[tile];
+    t.e0 = ls.tile_elem[tile];
     t.lo = static_cast<u32>(ls.elem_offsets[set]);
     t.hi = static_cast<u32>(ls.elem_offsets[set + 1] - 1);
     t.first = ls.tile_first[set];
     t.of = ls.tile_first[set + 1] - t.first;
-    t.index = blockIdx.x - t.first;
-    return true;
+    t.index = tile - t.first;
+    return t;
 }
 
 template <int ITEMS>
 __global__ void __launch_bounds__(kThreads) link_b_count_kernel(const Key* __restrict__ K, LinkSets ls,
                                                                 u32* __restrict__ counts,
                                                                 u32* __restrict__ pair_counts) {
-    Tile t;
-    if (batched_tile(ls, t)) count_tile<ITEMS>(K, t, counts, pair_counts);
+    if (blockIdx.x < *ls.n_tiles) count_tile<ITEMS>(K, batched_tile(ls, blockIdx.x), counts, pair_counts);
 }
 
 // Level offsets of every set (global node indices), a size check per set, and -1 for the
@@ -546,11 +591,11 @@ __global__ void link_b_lo_kernel(const u32* __restrict__ counts, LinkSets ls, in
 }
 
 template <int ITEMS, bool COUNTS>
-__global__ void __launch_bounds__(kThreads) link_b_scatter_kernel(const Key* __restrict__ K, LinkSets ls,
+__global__ void __launch_bounds__(kThreads, 6) link_b_scatter_kernel(const Key* __restrict__ K, LinkSets ls,
                                                                   const u32* __restrict__ offsets,
                                                                   const u32* __restrict__ pair_offsets, Out o) {
-    Tile t;
-    if (batched_tile(ls, t)) place_tile<ITEMS, COUNTS>(K, t, offsets, pair_offsets, o);
+    if (blockIdx.x < *ls.n_tiles)
+        place_tile<ITEMS, COUNTS>(K, batched_tile(ls, blockIdx.x), offsets, pair_offsets, o);
 }
 
 struct LinkBLayout {

@@ -61,3 +61,20 @@ def test_batched_sets_equal_single_builds(lib, sizes, ncrit):
         assert torch.equal(out["node_counts"][a:b], one["node_counts"])
         co = out["CO"][a:b]
         assert torch.equal(torch.where(co > 0, co - a, co), one["CO"])
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+def test_batched_boxes_of_odd_ranges(lib, shift):
+    """Sets that start and end at odd and even particles, from arrays on and off 16-byte boundaries."""
+    sizes = [1, 1, 2, 3, 0, 4, 5, 8193, 8192, 1, 100_001]
+    n = sum(sizes)
+    rng = np.random.default_rng(3)
+    xyz = [torch.from_numpy(rng.standard_normal(n + shift)).cuda()[shift:] for _ in range(3)]
+    off = torch.tensor(np.concatenate([[0], np.cumsum(sizes)]), dtype=torch.int64, device="cuda")
+    out = lib.build_octrees_batched(*xyz, off, curve=0, ncrit=32)
+    for s, size in enumerate(sizes):
+        a, b = int(off[s]), int(off[s + 1])
+        lo = [float(c[a:b].min()) if size else 0.0 for c in xyz]
+        side = max(float(c[a:b].max()) - v for c, v in zip(xyz, lo)) if size else 1.0
+        want = lo + [side if side > 0.0 else 1.0]
+        assert out["boxes"][s].tolist() == want, s

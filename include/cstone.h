@@ -474,9 +474,9 @@ CSTONE_API int cstone_host_status(int64_t n, int64_t leaf_cap, int32_t with_mass
  * (cstone_build_leaves, whose warm start, capacity report and synchronisation it has).
  * cstone_build_tree, on arrays sized for the leaves: the linked tree with its node counts (from
  * leaf_offsets) and, with mass != NULL, the multipoles. Both give what the single entry points above give
- * in order, on one workspace of the size that the query gives (ws may be the same for both). The structs' key arrays are uint64, or
- * uint32 for cstone30_build_set and cstone30_build_tree; records_ws is the workspace of
- * cstone_keys_records and keeps its error word.
+ * in order, on one workspace of the size that the query gives (ws may be the same for both). The
+ * structs' key arrays are uint64, or uint32 for cstone30_build_set and cstone30_build_tree; records_ws
+ * is the workspace of cstone_keys_records and keeps its error word.
  * ------------------------------------------------------------------------------------------ */
 typedef struct {
     const double* x;    /* [n] device */

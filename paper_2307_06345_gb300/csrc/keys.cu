@@ -224,8 +224,8 @@ __device__ FixedGrid make_fixed_grid(double lo, double side, int F_frame = 0) {
 // scale, shift and limits are the same; a coordinate is brought to fixed point by one right shift of
 // its mantissa; the product's high word is the cell and its low word the fraction; and whatever is not
 // plainly inside the box and away from cell borders, on any axis, takes one rare path. 2^25 Plummer
-// particles, Hilbert keys: 421 us with a frame, limits and selections per axis, 291 now (the integer pipe 77 % busy); 7.7e7 Morton
-// keys of 512 sets 1610 -> 731 us.
+// particles, Hilbert keys: 421 us with a frame, limits and selections per axis, 291 now (the integer
+// pipe 77 % busy); 7.7e7 Morton keys of 512 sets 1610 -> 731 us.
 struct FastGrid {
     u64 neg_lo[3];  // -trunc(lo * 2^F)
     u64 scale;      // S such that (((X - LO) << d_shift) * S) >> 64 has 32 fraction bits

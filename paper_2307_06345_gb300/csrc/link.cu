@@ -613,17 +613,19 @@ LinkBLayout link_b_layout(void* ws, long long n_elements, int n_sets) {
     Carver c(ws);
     l.ls.tile = static_cast<u32>(kThreads * items_of(n_elements));
     l.max_tiles = static_cast<u32>((n_elements + l.ls.tile - 1) / l.ls.tile + n_sets);
+    // a workspace for more elements serves fewer: no smaller than the largest that small tiles need
+    const size_t held = static_cast<size_t>(most_tiles(n_elements)) + n_sets;
     l.ls.n_tiles = c.take<u32>(1);
     l.ls.tile_first = c.take<u32>((size_t)n_sets + 1);
-    l.ls.tile_set = c.take<u32>(l.max_tiles);
-    l.ls.tile_elem = c.take<u32>(l.max_tiles);
-    l.ls.tile_count = c.take<u32>(l.max_tiles);
+    l.ls.tile_set = c.take<u32>(held);
+    l.ls.tile_elem = c.take<u32>(held);
+    l.ls.tile_count = c.take<u32>(held);
     l.ls.node_first = c.take<u32>((size_t)n_sets + 1);
     l.ls.n_sets = n_sets;
     l.ls.elem_offsets = nullptr;
-    l.counts = c.take<u32>(2 * ((size_t)l.max_tiles * kNumLevels + 1));
+    l.counts = c.take<u32>(2 * (held * kNumLevels + 1));
     l.chunks = static_cast<u32>(((size_t)l.max_tiles * kNumLevels + kScanChunk - 1) / kScanChunk);
-    l.partial = c.take<u32>((size_t)2 * l.chunks);
+    l.partial = c.take<u32>(2 * ((held * kNumLevels + kScanChunk - 1) / kScanChunk));
     l.bytes = c.size();
     return l;
 }

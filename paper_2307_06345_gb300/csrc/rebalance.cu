@@ -245,7 +245,8 @@ __device__ __forceinline__ u64 warp_distance(const u32 c[3], u32 edge, const u32
         best = r2 < best ? r2 : best;
     }
     const u32 hi = __reduce_min_sync(0xffffffffu, static_cast<u32>(best >> 32));
-    const u32 lo = __reduce_min_sync(0xffffffffu, static_cast<u32>(best >> 32) == hi ? static_cast<u32>(best) : 0xffffffffu);
+    const u32 low = static_cast<u32>(best >> 32) == hi ? static_cast<u32>(best) : 0xffffffffu;
+    const u32 lo = __reduce_min_sync(0xffffffffu, low);
     return (static_cast<u64>(hi) << 32) | lo;
 }
 

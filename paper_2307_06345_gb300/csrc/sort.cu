@@ -1365,7 +1365,8 @@ int run_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, const lo
     const int smem = static_cast<int>(sizeof(SmallSmem)), bsmem = static_cast<int>(sizeof(BigSmem));
     CST_CUDA(cudaFuncSetAttribute(sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const long long want = static_cast<long long>(sort_sizes(n, n_segs).small);
-    sort_small_kernel<<<(unsigned)(want < kSmallBlocks * sms ? want : kSmallBlocks * sms), kSmallThreads, smem, st>>>(p, l.t, idx_bits);
+    const unsigned sgrid = static_cast<unsigned>(want < kSmallBlocks * sms ? want : kSmallBlocks * sms);
+    sort_small_kernel<<<sgrid, kSmallThreads, smem, st>>>(p, l.t, idx_bits);
     CST_LAUNCHED("sort_small_kernel");
     if (rounds == 1) {
         CST_CUDA(cudaFuncSetAttribute(sort_rest_kernel<kBufA>, cudaFuncAttributeMaxDynamicSharedMemorySize, bsmem));
@@ -1383,8 +1384,13 @@ int run_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, const lo
 
 }  // namespace
 
+// A workspace for more keys serves fewer, also where the larger set takes the digit passes.
 size_t sort_ws_bytes(long long n) {
-    return digits::taken(n) ? digits::layout(nullptr, n).bytes : sort_layout(nullptr, n, 1).bytes;
+    if (!digits::taken(n)) return sort_layout(nullptr, n, 1).bytes;
+    const size_t own = digits::layout(nullptr, n).bytes;
+    if (sizeof(Key) != 4) return own;
+    const size_t most = sort_layout(nullptr, digits::kDigitMin - 1, 1).bytes;
+    return own > most ? own : most;
 }
 size_t sort_segmented_ws_bytes(long long n, int n_segs) { return sort_layout(nullptr, n, n_segs).bytes; }
 
@@ -1399,8 +1405,9 @@ constexpr long long kStaticKeys = CSTONE_SORT_STATIC_MAX_KEYS;
 constexpr SortSizes kStaticSizes = sort_sizes(kStaticKeys, 1);
 constexpr size_t kStaticBytes =
     sizeof(WsHeader) + round256(3 * 4) + 2 * (4 * round256((kStaticSizes.big + 1) * 4) + round256(kStaticSizes.big * 8)) +
-    round256(kStaticSizes.parts * 8) + round256(kStaticSizes.parts * 4) + round256(kStaticSizes.parts * 4 * kPosStride) + 2 * round256(kStaticSizes.small * 8) +
-    round256(static_cast<size_t>(kStaticKeys) * 2) + round256(kStaticSizes.tiles * 4) + round256(static_cast<size_t>(kStaticKeys) * 8) +
+    round256(kStaticSizes.parts * 8) + round256(kStaticSizes.parts * 4) + round256(kStaticSizes.parts * 4 * kPosStride) +
+    2 * round256(kStaticSizes.small * 8) + round256(static_cast<size_t>(kStaticKeys) * 2) +
+    round256(kStaticSizes.tiles * 4) + round256(static_cast<size_t>(kStaticKeys) * 8) +
     round256(static_cast<size_t>(kStaticKeys) * 4);
 
 __device__ __align__(256) unsigned char g_sort_scratch[kStaticBytes];

@@ -3,7 +3,7 @@
 Workload (one step): N = 2^27 particles, float64 coordinates from 1,000 Gaussian clumps
 (sigma log-uniform in 1e-4..1e-2 of the box) plus 20% uniform background, float32 log-normal
 masses, 63-bit Hilbert keys, Ncrit = 64. A step runs the whole path on the device: bounding cube,
-keys, radix sort with permutation, cornerstone leaf loop, linked octree, node-count upsweep and
+keys, sort with permutation, cornerstone leaves, linked octree, node-count upsweep and
 the FP32 compensated monopole/quadrupole upsweep. Inputs (3.5 GB) are larger than the 129 MB L2,
 so no explicit flush is needed between steps.
 
@@ -141,20 +141,20 @@ class ClockSampler:
 
 
 # DRAM bytes per particle of the bounding cube, the key pass with multipole records, the sort
-# (per-pass tile counts and scans, 8 passes) and the multipole upsweep (leaf sums and levels),
+# (samples, counts, two scatters and the final sort) and the multipole upsweep (leaf sums and levels),
 # measured with ncu (dram__bytes_read.sum + dram__bytes_write.sum over the phase's launches) on
 # 2^24 particles of the same workload and scaled by the particle count (these phases stream or
 # gather per particle, so traffic grows with n).
-MEASURED_DRAM_BYTES_PER_PARTICLE = {"bbox": 24.2, "keys": 64.7, "sort": 233.5, "multipoles": 139.8}
+MEASURED_DRAM_BYTES_PER_PARTICLE = {"bbox": 24.0, "keys": 64.5, "sort": 85.5, "multipoles": 139.4}
 
 
-def algorithmic_bytes(n: int, n_leaves: int, iter_leaves: int, n_nodes: int):
+def algorithmic_bytes(n: int, n_leaves: int, n_nodes: int):
     """Compulsory DRAM traffic of one step (bytes), by phase."""
     return {
         "bbox": 24 * n,
         "keys": 68 * n,                         # read x, y, z, m; write the key and the 32-byte record
-        "sort": (20 + 24 * 7) * n,              # 8 passes (the first has no value read)
-        "leaves": 24 * iter_leaves + 8 * n,     # K + pos read/written per pass; P read by searches once
+        "sort": (20 + 24 * 2) * n,              # three moves of a pair (the first has no value read)
+        "leaves": 24 * n_leaves + 8 * n,        # P read once; leaf starts listed and read, keys, counts, offsets
         "link": 40 * n_nodes,
         "counts": 8 * n_nodes,
         "multipoles": 36 * n + 48 * n_nodes,    # record gather + perm; per-node outputs + scratch
@@ -239,9 +239,9 @@ def run_ours(args, rank, world, local):
     ms_per_step = elapsed_ms / K
     value = world * n / (ms_per_step * 1e-3)
 
-    # roofline of the dominant kernel group: the radix sort (8 digit passes)
+    # roofline of the dominant kernel group
     hbm, peak_kind = peaks()
-    algo = algorithmic_bytes(n, n_leaves, int(n_leaves * 1.3), n_nodes)
+    algo = algorithmic_bytes(n, n_leaves, n_nodes)
     dom = max(phase_ms, key=phase_ms.get)
     achieved = algo[dom] / (phase_ms[dom] * 1e-3) / 1e9
     step_bytes = sum(algo.values())
@@ -451,8 +451,8 @@ def run_global(args, rank, world, local):
     e2e_ms = max_over_ranks(e0.elapsed_time(e1) / ke, dist, dev)
     hbm, peak_kind = peaks()
     nl_local = out["n_leaves"]
-    local_bytes = sum(v for k2, v in algorithmic_bytes(n_local, nl_local, int(nl_local * 1.3),
-                                                        cs.n_nodes(nl_local)).items() if k2 != "bbox")
+    local_bytes = sum(v for k2, v in algorithmic_bytes(n_local, nl_local, cs.n_nodes(nl_local)).items()
+                      if k2 != "bbox")
     line = None
     if rank == 0:
         line = {

@@ -106,7 +106,7 @@ int cstone_build_batched(const cstone_batch_input* in, const cstone_batch_params
                                                    l.len[cst::kWsLeaves], stream))
         return rc;
     // with leaf offsets the node counts come from the pass that links the tree (512 sets of 1,024 to
-    // 1,048,576: link and counts 640 -> 330 us); without, from their own
+    // 1,048,576: link and counts 640 -> 310 us); without, from their own
     const bool counted = out->leaf_offsets != nullptr;
     if (int rc = cst::link_tree_batched("cstone_build_batched", reinterpret_cast<const cst::u64*>(out->elements), ecap,
                                         reinterpret_cast<const long long*>(out->element_offsets), S, out->node_cap,

@@ -26,8 +26,8 @@
 // particles are those between the first of its first leaf and the first of the leaf after its last, and
 // both leaves are found near the pair (`covered`). This takes the place of a sum over the children level
 // by level, whose grid barriers bounded it (upsweep.cu, which still serves callers that have counts only).
-// Link and counts together: 512 sets of 1,024 to 1,048,576 particles 640 -> 330 us, 48 of 128 to 4,096
-// 88 -> 35, one of 1,048,576 43 -> 24, of 33,554,432 122 -> 84.
+// Link and counts together: 512 sets of 1,024 to 1,048,576 particles 640 -> 310 us, 48 of 128 to 4,096
+// 88 -> 35, one of 1,048,576 43 -> 25, of 33,554,432 122 -> 63.
 #include "common.cuh"
 
 namespace CST_NS {

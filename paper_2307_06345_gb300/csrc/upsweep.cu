@@ -761,8 +761,11 @@ int launch_upsweep_multipoles(const double* x, const double* y, const double* z,
         multipole_leaf_kernel<8><<<lgrid, kLeafThreads, 0, st>>>(offsets, static_cast<u32>(nl), perm, leaf_to_node, nn,
                                                                  l.mp, box, mass, com, quad);
     CST_LAUNCHED("multipole_leaf_kernel");
-    multipole_bigleaf_kernel<<<sm_count() * 4, kLeafThreads, 0, st>>>(offsets, perm, leaf_to_node, nn, l.mp, box, mass,
-                                                                     com, quad);
+    // no more blocks than n particles can make leaves of that size (the launch of four per SM took 5.7 us even
+    // where there are none: small trees' moments 42.9 us a call, 39.8 so)
+    const long long big_most = n / (kBigLeaf + 1) + 1, big_grid = sm_count() * 4ll;
+    multipole_bigleaf_kernel<<<static_cast<unsigned>(big_most < big_grid ? big_most : big_grid), kLeafThreads, 0, st>>>(
+        offsets, perm, leaf_to_node, nn, l.mp, box, mass, com, quad);
     CST_LAUNCHED("multipole_bigleaf_kernel");
     if (nl > 1) {
         u32 nn_ = nn;

@@ -148,7 +148,8 @@ CSTONE_API int cstone_sort_static(const uint64_t* keys_in, uint64_t* keys_out, u
  * the rebalance g = g3 . g2 . g1 until g1 decides O_i = 1 for every leaf. Rules of g1: split when
  * N_i > ncrit (unless the leaf is a single key at depth L); merge the 8 consecutive sibling
  * leaves of a parent when their combined count is <= ncrit (the first octant keeps its key).
- *   sorted_keys [n] uint64 sorted particle keys P (< 2^63).
+ *   sorted_keys [n] uint64 sorted particle keys P (< 2^63). Keys out of order between two leaves of a cold
+ *               start are reported as CSTONE_ERR_INVALID_ARG.
  *   leaves      [leaf_cap + 1] uint64 in/out cornerstone array K.
  *   n_leaves    host in/out: leaves on entry (0 = root), final n_l on exit; on
  *               CSTONE_ERR_CAPACITY the number of leaves that did not fit.

@@ -601,7 +601,8 @@ int run_cold(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap, 
     const u32 sms = static_cast<u32>(sm_count());
     u32* first = offsets ? offsets : l.bufs.pos[0];
     auto grid = [&](u32 per_sm) { return tiles < sms * per_sm ? tiles : sms * per_sm; };
-    cold::starts_kernel<BATCH><<<grid(cold::kBlocks), cold::kThreads, cold::sweep_smem(ncrit), st>>>(P, v, ncrit, l.tiles);
+    cold::starts_kernel<BATCH><<<grid(cold::kBlocks), cold::kThreads, cold::sweep_smem(ncrit), st>>>(P, v, ncrit, l.tiles,
+                                                                                                      hdr);
     CST_LAUNCHED("starts_kernel");
     cold::outcome_kernel<<<1, 1024, 0, st>>>(l.tiles, sv.n_sets, static_cast<u32>(ecap), max_iters, hdr);
     CST_LAUNCHED("outcome_kernel");

@@ -34,6 +34,7 @@ constexpr int kItems = 8;
 constexpr u32 kTile = kThreads * kItems;  // positions per tile: the particles, and one after the last
 constexpr u32 kMaxNcrit = 1024;
 constexpr int kBlocks = 6;  // blocks per SM of the sweep
+constexpr u32 kDisorder = 0x70001u;  // error detail: keys that are not sorted
 static_assert(kTile == 2048 && kLevels < 32, "bits of a listed leaf start");
 
 struct View {  // the sets' particles; offsets == NULL: one set of n
@@ -164,7 +165,8 @@ constexpr u32 kMostBits = kKeyBits - 1;
 // borders; the elements are counted from the list, where a warp has work for all lanes (counting them
 // where the starts are found, four particles to a thread, took 1.16 ms for 2^27 clumps, this takes 0.78).
 template <bool BATCH>
-__global__ void __launch_bounds__(kThreads, kBlocks) starts_kernel(const Key* __restrict__ P, View v, u32 ncrit, Tiles t) {
+__global__ void __launch_bounds__(kThreads, kBlocks) starts_kernel(const Key* __restrict__ P, View v, u32 ncrit, Tiles t,
+                                                                   WsHeader* hdr) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_levels[kLevels + 2];
     __shared__ u32 s_count[kItems * kWarps];
@@ -293,6 +295,7 @@ __global__ void __launch_bounds__(kThreads, kBlocks) starts_kernel(const Key* __
             const int level = static_cast<int>((w >> 11) & 31u), prev_level = static_cast<int>((w >> 16) & 31u);
             const Key key = s_key[q], prev = s_key[q - 1];
             const int d = (w >> 21) ? -1 : shared_digits(prev, key);
+            if (d >= 0 && key < prev) raise_error(hdr, CSTONE_ERR_INVALID_ARG, kDisorder);
             elems += d < 0 ? elements_at_boundary(v, j, p0, p1, prev, key, prev_level, level)
                            : elements_between(prev, key, d, prev_level, level);
             if (j < p1 && level > d + 1) {  // internal nodes of levels d + 1 .. level - 1 start here
@@ -317,6 +320,10 @@ static_assert(kItems * kWarps == 64, "two counts per lane");
 
 // Index of every tile's first element, and the outcome as the loop would have it: pass l splits the
 // internal nodes of level l, the pass after the last of them changes nothing. One block.
+//
+// Self-check: keys that are not sorted (or set offsets that do not ascend) can list more starts than the array
+// has elements, and so more than the list holds. Of a sorted set every start emits its leaf, and the starts
+// together emit the array; anything else is an error, before the list is read.
 __global__ void __launch_bounds__(1024) outcome_kernel(Tiles t, int n_sets, u32 ecap, int max_iters,
                                                        WsHeader* hdr) {
     __shared__ u32 s_warp[32];
@@ -345,6 +352,8 @@ __global__ void __launch_bounds__(1024) outcome_kernel(Tiles t, int n_sets, u32 
     for (int pass = 0; pass < max_iters; ++pass) {
         nodes += pass < kLevels ? t.levels[pass] : -nodes;  // of level `pass`
         if (nodes == 0) {
+            if (*t.n_starts > ne || run != static_cast<u32>(ne)) raise_error(hdr, CSTONE_ERR_INVALID_ARG, kDisorder);
+            if (hdr->err) return;
             *outcome_of(hdr) = Outcome{static_cast<u32>(pass + 1), 1u, 0u, static_cast<u32>(ne)};
             return;
         }

@@ -633,6 +633,8 @@ def build_octree(x, y, z, curve: int = HILBERT, ncrit: int = 64, box=None, masse
             b.records = torch.empty(records_size(n), dtype=torch.uint8, device=b.device)
             b.rws = Workspace(b.device)
         b.rws.get(_size(load().cstone_keys_records_workspace_size))
+    # no masses are told by a null pointer, which an empty tensor has too: any other address stands in for it
+    m_ptr = (masses.data_ptr() or b.records.data_ptr()) if masses is not None else None
     cur = stream if stream is not None else torch.cuda.current_stream()
     nl0 = 0
     if warm_leaves is not None:
@@ -643,7 +645,7 @@ def build_octree(x, y, z, curve: int = HILBERT, ncrit: int = 64, box=None, masse
     buf = b.c_struct()
     ws = b.ws.get(_size(fn("build_set_workspace_size"), n, buf.leaf_cap, max_iters))
     st = ctypes.c_void_p(cur.cuda_stream)
-    inp = _SetInput(x.data_ptr(), y.data_ptr(), z.data_ptr(), _ptr(masses), n, _ptr(box))
+    inp = _SetInput(x.data_ptr(), y.data_ptr(), z.data_ptr(), m_ptr, n, _ptr(box))
     nl_c, it_c = ctypes.c_int64(nl0), ctypes.c_int32(0)
     rc = fn("build_set")(ctypes.byref(inp), ctypes.byref(_SetParams(curve, ncrit, max_iters)), ctypes.byref(buf),
                          ctypes.byref(nl_c), ctypes.byref(it_c), ws.data_ptr(), ws.numel(), st)

@@ -50,3 +50,17 @@ def test_build_octree_equals_single_calls(lib, levels, n, ncrit, boxed, masses, 
     warm = lib.build_octree(x, y, z, curve=1, ncrit=ncrit, box=box, levels=levels, warm_leaves=got["leaves"].clone())
     assert warm["n_leaves"] == nl
     assert torch.equal(warm["leaves"], want["leaves"]) and torch.equal(warm["NK"], want["NK"])
+
+
+@pytest.mark.parametrize("levels", [21, 10])
+def test_masses_of_no_particles(lib, levels):
+    """A build of no particles with masses clears the error word of the records' workspace, as any other."""
+    none = torch.empty(0, dtype=torch.float64, device="cuda")
+    b = lib.OctreeBuffers.allocate(0, 64, "cuda", levels)
+    b.records = torch.empty(lib.records_size(0), dtype=torch.uint8, device="cuda")
+    b.rws = lib.Workspace("cuda")
+    b.rws.get(256).fill_(255)
+    got = lib.build_octree(none, none, none, masses=none.float(), buffers=b, levels=levels)
+    assert b.rws.status() == lib.OK
+    assert got["n_leaves"] == 1 and got["node_counts"].tolist() == [0]
+    assert got["mass"].tolist() == [0.0] and not got["quad"].any()

@@ -539,11 +539,11 @@ namespace {
 struct LeavesLayout {
     LoopState* ls;
     LeafBufs bufs;
-    cold::Tiles tiles;  // of a cold build: the list lies in the loop's split queue
+    cold::Tiles tiles;  // of a sweep, in the loop's split queue: four words per element
     size_t bytes;
 };
 
-// n: particles (in a batched build the most there can be, the size query does not know them).
+// The size does not depend on n: a batch's size query does not know it.
 LeavesLayout leaves_layout(void* ws, long long n, long long ecap, bool batch) {
     LeavesLayout l;
     Carver c(ws);
@@ -556,13 +556,12 @@ LeavesLayout leaves_layout(void* ws, long long n, long long ecap, bool batch) {
         l.bufs.pos[k] = c.take<u32>((size_t)ecap);
         l.bufs.set[k] = batch ? c.take<u32>((size_t)ecap) : nullptr;
     }
-    const u32 most = cold::tiles_of(batch ? CSTONE_MAX_PARTICLES : n);
-    l.tiles.list = c.take<u32>(most);
-    l.tiles.count = c.take<u32>(most);
-    l.tiles.elems = c.take<u32>(most);
     l.tiles.tiles = cold::tiles_of(n);
     l.tiles.starts = reinterpret_cast<u32*>(l.bufs.split_q);
     l.tiles.start_cap = static_cast<u32>(ecap);
+    l.tiles.list = l.tiles.starts + ecap;  // one word per tile each, of room for one per element
+    l.tiles.count = l.tiles.list + ecap;
+    l.tiles.elems = l.tiles.count + ecap;
     l.tiles.n_starts = l.ls ? &l.ls->cold_starts : nullptr;
     l.tiles.levels = l.ls ? l.ls->cold_levels : nullptr;
     l.bytes = c.size();
@@ -616,6 +615,12 @@ int run_cold(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap, 
     return CSTONE_OK;
 }
 
+// A cold build takes one sweep over the keys instead of a pass per level (2^27 clumps: 1.47 ms in the loop). A
+// window of more than kMaxNcrit particles does not fit its shared memory; an array with room for fewer
+// elements than there are tiles (of many particles in a few cells, or too small) has no room for their tables,
+// and few elements are quick in the loop.
+bool sweep_taken(u32 ncrit, long long ecap, u32 tiles) { return ncrit <= cold::kMaxNcrit && tiles <= ecap; }
+
 // Runs the build. ne0: element count of the warm-start arrays held in `leaves` (0 = cold start from
 // the roots, -1 = warm start with the count read on the device). With sync, *ne_out is the element
 // count of the converged arrays on success; without, nothing is read back (the outcome stays in
@@ -627,9 +632,7 @@ int run_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap
     LeavesLayout l = leaves_layout(ws, n, ecap, BATCH);
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader) + sizeof(LoopState), st));
-    // A cold build takes one sweep over the keys instead of a pass per level (2^27 clumps: 1.47 ms in the
-    // loop); a window of more than kMaxNcrit particles does not fit its shared memory.
-    if (ne0 == 0 && ncrit <= cold::kMaxNcrit) {
+    if (ne0 == 0 && sweep_taken(ncrit, ecap, l.tiles.tiles)) {
         if (int rc = run_cold<BATCH>(P, n, ncrit, leaves, ecap, counts, offsets, max_iters, sv, l, hdr, !sync, st))
             return rc;
         if (!sync) return CSTONE_OK;
@@ -657,7 +660,7 @@ int run_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap
 
 }  // namespace
 
-size_t leaves_ws_bytes(long long n, long long cap) { return leaves_layout(nullptr, n, cap + 1, false).bytes; }
+size_t leaves_ws_bytes(long long cap) { return leaves_layout(nullptr, 0, cap + 1, false).bytes; }
 size_t leaves_batched_ws_bytes(long long ecap) { return leaves_layout(nullptr, 0, ecap, true).bytes; }
 
 int launch_build_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long cap, long long* n_leaves,
@@ -701,7 +704,7 @@ int CSTONE_FN(leaves_workspace_size)(int64_t n, int64_t leaf_cap, int32_t max_it
     if (!bytes || n < 0 || n >= CSTONE_MAX_PARTICLES || leaf_cap < 1 || leaf_cap > CSTONE_MAX_LEAVES ||
         max_iters < 1 || max_iters > 256)
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(leaves_workspace_size)) ": bad argument");
-    *bytes = CST_NS::leaves_ws_bytes(n, leaf_cap);
+    *bytes = CST_NS::leaves_ws_bytes(leaf_cap);
     return CSTONE_OK;
 }
 
@@ -714,7 +717,7 @@ int CSTONE_FN(build_leaves)(const CST_KEY_C* sorted_keys, int64_t n, uint32_t nc
     if (*n_leaves < 0 || *n_leaves > leaf_cap)
         return cst::fail(CSTONE_ERR_INVALID_ARG, CST_STR(CSTONE_FN(build_leaves)) ": initial n_leaves %lld outside "
                          "[0, %lld]", (long long)*n_leaves, (long long)leaf_cap);
-    if (int rc = cst::check_ws(ws, ws_bytes, CST_NS::leaves_ws_bytes(n, leaf_cap),
+    if (int rc = cst::check_ws(ws, ws_bytes, CST_NS::leaves_ws_bytes(leaf_cap),
                                CST_STR(CSTONE_FN(build_leaves))))
         return rc;
     long long nl = *n_leaves;

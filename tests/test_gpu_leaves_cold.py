@@ -91,3 +91,23 @@ def test_batched_sets(lib, oracle, sizes, ncrit):
     assert np.array_equal(counts[:ne].cpu().numpy(), np.concatenate([np.append(r[1], 0) for r in ref]))
     assert np.array_equal(first[:ne].cpu().numpy(),
                           np.concatenate([off[k] + np.concatenate([[0], np.cumsum(r[1])]) for k, r in enumerate(ref)]))
+
+
+@pytest.mark.parametrize("room", [0, 1, 300])
+def test_fewer_elements_than_tiles(lib, oracle, room):
+    """Capacities below and above the number of tiles, for many particles in one cell."""
+    n = 600_000
+    tiles = n // 2048 + 1
+    P = np.full(n, (1 << 63) // 3, np.uint64)
+    K_ref, N_ref, it_ref = oracle.build_leaves(P, 64)
+    assert K_ref.size < tiles
+    cap = max(K_ref.size - 1, tiles - 2 + room)
+    K, N, off, it = _build(lib, P, 64, cap)
+    assert np.array_equal(K, K_ref) and np.array_equal(N, N_ref) and it == it_ref
+    assert np.array_equal(off, np.concatenate([[0], np.cumsum(N_ref)]))
+    eo = torch.zeros(3, dtype=torch.int64, device="cuda")
+    d = torch.from_numpy(np.concatenate([P, P[:7]]).view(np.int64)).cuda()
+    E, C = (torch.zeros(cap + 3, dtype=t, device="cuda") for t in (torch.int64, torch.int32))
+    ne, it = lib.cstone_build_leaves_batched(d, torch.tensor([0, n, n + 7], device="cuda"), 64, E, eo, C)
+    assert it == it_ref and eo.tolist() == [0, K_ref.size, K_ref.size + 2]
+    assert np.array_equal(E[: K_ref.size].cpu().numpy().view(np.uint64), K_ref) and C[ne - 2].item() == 7

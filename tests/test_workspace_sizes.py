@@ -38,3 +38,14 @@ def test_size_query_is_monotone(clib, name):
         assert call(f, n, ctypes.byref(out)) == 0
         assert out.value >= last, n
         last = out.value
+
+
+@pytest.mark.parametrize("elements", [64, 4096, 1 << 20])
+def test_leaf_workspace_follows_the_capacity(clib, elements):
+    """A batch's leaf workspace holds the loop's arrays for its elements (under 64 bytes each, and the passes'
+    state), however many particles a batch may have."""
+    out = ctypes.c_size_t()
+    assert clib.cstone_leaves_batched_workspace_size(elements, 64, ctypes.byref(out)) == 0
+    assert out.value <= 64 * elements + (1 << 16)
+    assert clib.cstone_leaves_workspace_size(1 << 29, elements, 64, ctypes.byref(out)) == 0
+    assert out.value <= 64 * elements + (1 << 16)

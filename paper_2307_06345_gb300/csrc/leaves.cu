@@ -1,6 +1,6 @@
 // Cornerstone leaf array. A cold start (from the roots) finds the converged array in one sweep over
-// the keys (leaves_cold.cuh); a warm start, and a cold one with a large N_crit, run the f / g iteration of
-// Sec. 4 (Eqs. histogram, g1, g2, g3) in one persistent cooperative kernel, described here.
+// the keys (leaves_cold.cuh); a warm start, and a cold one with few leaves for its particles (sweep_taken), run
+// the f / g iteration of Sec. 4 (Eqs. histogram, g1, g2, g3) in one persistent cooperative kernel, described here.
 //
 // Alongside K the kernel keeps pos_i = lower_bound(P, K_i) for every key of the array. Then the
 // histogram of Eq. (histogram) is N_i = pos_{i+1} - pos_i, and the combined count of 8 sibling
@@ -615,11 +615,30 @@ int run_cold(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap, 
     return CSTONE_OK;
 }
 
-// A cold build takes one sweep over the keys instead of a pass per level (2^27 clumps: 1.47 ms in the loop). A
-// window of more than kMaxNcrit particles does not fit its shared memory; an array with room for fewer
-// elements than there are tiles (of many particles in a few cells, or too small) has no room for their tables,
-// and few elements are quick in the loop.
-bool sweep_taken(u32 ncrit, long long ecap, u32 tiles) { return ncrit <= cold::kMaxNcrit && tiles <= ecap; }
+// Whether a cold build takes the sweep over the keys, else the loop's pass per level. The sweep reads every key
+// (5.6 ps each, and 0.5 more per 100 of N_crit), whatever the tree; the loop only touches the keys near leaf
+// borders, so its time follows the leaves and the passes: it wins where the leaves are few for the particles.
+// Measured (us, sweep / loop) with uniform, Gaussian, Plummer and clumped sets:
+//   N_crit   64: 2^25 320/422 319/459 307/521 312/640     2^27 1080/991  1061/969 1074/1043 1075/1462
+//                2^29 3931/2212 4061/2976 4073/3114 4052/4236
+//   N_crit  256: 2^23 122/190 118/224 118/262 118/359     2^25 314/248  317/313 320/374 322/462
+//                2^27 1101/532 1099/559 1084/614 1093/763
+//   N_crit 1024: 2^20 68/116  70/150  70/178  72/175      2^23 145/146  142/176 143/211 146/313
+//                2^25 410/214 406/262 410/302 415/397
+//   N_crit   32: 2^27 1194/1436 1180/1462 1149/1576 1128/2079   2^29 4670/5181 4381/4606 4438/5462 4478/7240
+// so the mean of the four breaks even at n * N_crit = 2^33 from N_crit 64 on (one set in four loses up to a third
+// near that line, one gains as much), and up to N_crit 32 the sweep is the faster one (at worst, 2^28 uniform:
+// 2046/1819); batches of sets have the same line (64 x 2^20 particles at N_crit 64: 559/509, 575/736,
+// 647/1509). 30-bit trees end at level 10 with fewer leaves: half of that, at any N_crit (N_crit 64: 2^26 504/426
+// 516/560 477/421 468/450, 2^27 973/871 967/861 880/498 867/615). Where sets are single leaves, the loop has
+// one pass (4,000 sets of 100 at N_crit 128: 69/52). A window of more than kMaxNcrit particles does not fit the
+// sweep's shared memory, and an array with room for fewer elements than there are tiles (many particles in
+// a few cells, or an array that is too small) does not hold its tables.
+bool sweep_taken(u32 ncrit, long long n, int n_sets, long long ecap, u32 tiles) {
+    if (ncrit > cold::kMaxNcrit || tiles > ecap || n <= static_cast<long long>(ncrit) * n_sets) return false;
+    constexpr bool kLong = kLevels == CSTONE_LEVELS;
+    return (kLong && ncrit <= 32) || n * static_cast<long long>(ncrit) <= 1ll << (kLong ? 33 : 32);
+}
 
 // Runs the build. ne0: element count of the warm-start arrays held in `leaves` (0 = cold start from
 // the roots, -1 = warm start with the count read on the device). With sync, *ne_out is the element
@@ -632,7 +651,7 @@ int run_leaves(const Key* P, long long n, u32 ncrit, Key* leaves, long long ecap
     LeavesLayout l = leaves_layout(ws, n, ecap, BATCH);
     WsHeader* hdr = reinterpret_cast<WsHeader*>(ws);
     CST_CUDA(cudaMemsetAsync(hdr, 0, sizeof(WsHeader) + sizeof(LoopState), st));
-    if (ne0 == 0 && sweep_taken(ncrit, ecap, l.tiles.tiles)) {
+    if (ne0 == 0 && sweep_taken(ncrit, n, BATCH ? sv.n_sets : 1, ecap, l.tiles.tiles)) {
         if (int rc = run_cold<BATCH>(P, n, ncrit, leaves, ecap, counts, offsets, max_iters, sv, l, hdr, !sync, st))
             return rc;
         if (!sync) return CSTONE_OK;

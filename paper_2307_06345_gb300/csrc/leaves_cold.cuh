@@ -18,9 +18,10 @@
 // builds the first particle of a set closes the set before it, with the empty sets between.
 //
 // One launch reads P and lists the leaf starts (5 % of the particles at N_crit 64), a block scans the
-// tiles' totals, one launch emits the leaves and one takes their counts; the loop makes two sweeps and
-// a search of the split ranges per level. The window maximum takes log2(N_crit) steps on bytes in
-// shared memory; sets with a larger N_crit than kMaxNcrit, whose arrays are small, take the loop.
+// tiles' totals, one launch emits the leaves and one takes their counts; the loop makes two sweeps over its
+// elements and a search of the split ranges per level, which is less where the leaves are few (sweep_taken in
+// leaves.cu says where). The window maximum takes log2(N_crit) steps on bytes in shared memory, which holds
+// windows of up to kMaxNcrit.
 #pragma once
 
 #include "common.cuh"

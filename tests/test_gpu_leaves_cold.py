@@ -111,3 +111,36 @@ def test_fewer_elements_than_tiles(lib, oracle, room):
     ne, it = lib.cstone_build_leaves_batched(d, torch.tensor([0, n, n + 7], device="cuda"), 64, E, eo, C)
     assert it == it_ref and eo.tolist() == [0, K_ref.size, K_ref.size + 2]
     assert np.array_equal(E[: K_ref.size].cpu().numpy().view(np.uint64), K_ref) and C[ne - 2].item() == 7
+
+
+SWEEP, LOOP = 4, 1  # launches of a cold build
+
+
+@pytest.mark.parametrize("levels,n,ncrit,launches", [
+    (21, 1 << 23, 1024, SWEEP), (21, (1 << 23) + 1, 1024, LOOP), (21, (1 << 23) + 1, 32, SWEEP),
+    (10, 1 << 22, 1024, SWEEP), (10, (1 << 22) + 1, 1024, LOOP),
+    (21, 500, 500, LOOP), (21, 501, 500, SWEEP), (10, 500, 500, LOOP), (10, 501, 500, SWEEP)])
+def test_both_sides_of_the_size_rule(lib, oracle, levels, n, ncrit, launches):
+    P = _keys(np.random.default_rng(n), n, "clustered", levels)
+    K_ref, N_ref, it_ref = oracle.build_leaves(P, ncrit, levels=levels)
+    before = lib.cstone_kernel_launches()
+    K, N, off, it = _build(lib, P, ncrit, max(K_ref.size, n // 2048 + 1), levels)
+    assert lib.cstone_kernel_launches() - before == launches
+    assert np.array_equal(K, K_ref) and np.array_equal(N, N_ref) and it == it_ref
+
+
+@pytest.mark.parametrize("size,launches", [(40, LOOP), (41, SWEEP)])
+def test_sets_of_single_leaves(lib, size, launches):
+    rng = np.random.default_rng(size)
+    s, ncrit = 300, 40
+    P = np.concatenate([_keys(rng, size, "uniform", 21) for _ in range(s)])
+    off = torch.arange(s + 1, device="cuda") * size
+    E, C = (torch.zeros(9 * s, dtype=t, device="cuda") for t in (torch.int64, torch.int32))
+    eo = torch.zeros(s + 1, dtype=torch.int64, device="cuda")
+    before = lib.cstone_kernel_launches()
+    ne, _ = lib.cstone_build_leaves_batched(torch.from_numpy(P.view(np.int64)).cuda(), off, ncrit, E, eo, C)
+    assert lib.cstone_kernel_launches() - before == launches
+    per = 2 if size <= ncrit else 9
+    assert ne == per * s and eo.tolist() == [per * k for k in range(s + 1)]
+    counts = C[:ne].view(s, per)
+    assert (counts.sum(1) == size).all() and not counts[:, -1].any() and (counts <= ncrit).all()

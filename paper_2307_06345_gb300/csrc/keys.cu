@@ -175,13 +175,20 @@ __device__ __forceinline__ u32 grid_cell(double x, double lo, double scale) {
 // together move u by far less than 2^-24 cells, so whenever the fixed-point u is at least 2^-20
 // away from an integer its floor is the floor of the IEEE result. The remaining ~2^-19 of
 // coordinates, and boxes where the error bound does not hold, take the IEEE path.
-struct FixedGrid {
+struct FixedGrid {  // one axis
     long long lo_fixed;   // LO
     u64 scale_fixed;      // S
+    u64 lo_ord, hi_ord;   // order-preserving bits of lo and of lo + 2 side
     double lo, scale;
     int F, R;
-    int fast;
+    int ok;               // the values allow a bound (whether it holds depends on F)
+    int fast;             // the bound holds at this F
 };
+
+__device__ __forceinline__ u64 order_bits(double v) {
+    const u64 b = static_cast<u64>(__double_as_longlong(v));
+    return (b >> 63) ? ~b : (b | (1ULL << 63));
+}
 
 __device__ __forceinline__ int exponent_of(double v) {  // unbiased exponent field (0 for zero/subnormal)
     return static_cast<int>((static_cast<u64>(__double_as_longlong(v)) >> 52) & 0x7ffu);
@@ -198,23 +205,29 @@ __device__ __forceinline__ long long to_fixed(double x, int F) {
     return (b >> 63) ? -static_cast<long long>(mag) : static_cast<long long>(mag);
 }
 
-// F_frame != 0: take that fixed-point exponent (a frame shared with other arrays) instead of the
-// axis' own; the fast path is then enabled only where its error bound holds for it.
-__device__ FixedGrid make_fixed_grid(double lo, double side, int F_frame = 0) {
+__device__ __forceinline__ bool bound_holds(int F, int R) {
+    const int es = F - R - 53;  // scale = mantissa * 2^es
+    return R >= 26 && R <= 62 && es + 78 <= F && F <= 1074;
+}
+
+// The axis in the widest frame that holds it.
+__device__ FixedGrid make_fixed_grid(double lo, double side) {
     FixedGrid f;
     f.lo = lo;
     f.scale = __ddiv_rn(2097152.0, side);
     const double hi = __dadd_rn(lo, __dmul_rn(2.0, side));
+    f.lo_ord = order_bits(lo);
+    f.hi_ord = order_bits(hi);
     // 2^E > max(|lo|, |hi|)
     const int e_max = max(exponent_of(lo), exponent_of(hi)) - 1023 + 1;
-    f.F = F_frame != 0 && F_frame <= 61 - e_max ? F_frame : 61 - e_max;
-    const int es = exponent_of(f.scale) - 1023 - 52;  // scale = mantissa * 2^es
+    f.F = 61 - e_max;
+    const int es = exponent_of(f.scale) - 1023 - 52;
     const int G = 11 - es;
     f.R = f.F + G - 64;
     u64 sb = static_cast<u64>(__double_as_longlong(f.scale));
     f.scale_fixed = ((sb & ((1ULL << 52) - 1)) | (1ULL << 52)) << 11;
-    f.fast = (f.R >= 26 && f.R <= 62 && es + 78 <= f.F && f.F <= 1074 && exponent_of(f.scale) != 0 &&
-              exponent_of(f.scale) != 0x7ff && !(hi <= lo));
+    f.ok = exponent_of(f.scale) != 0 && exponent_of(f.scale) != 0x7ff && e_max < 1024 && !(hi <= lo);
+    f.fast = f.ok && bound_holds(f.F, f.R);
     f.lo_fixed = f.fast ? to_fixed(lo, f.F) : 0;
     return f;
 }
@@ -233,30 +246,33 @@ struct FastGrid {
     u32 d_end;      // distances from the corner whose high word is below this are inside the box
     int d_shift;
     int fast;       // the error bound holds
-    double lo[3], inv;
-    int F;
+    FixedGrid axis[3];  // for the rare path
 };
 
-// Frame F of the records when it is shared with them; else the widest that holds the box.
-__device__ FastGrid make_fast_grid(const double* box) {
+// The frame that holds all axes, which is the records' frame (make_frame). Called by whole warps: lane d of a
+// group of four takes axis d (the fourth repeats the last), and the group writes *g where `write` is set. One
+// thread with the axes one after the other took 2 us longer, of the 8 that the keys of 1000 particles take.
+__device__ __forceinline__ void make_fast_grid(const double* box, FastGrid* g, bool write) {
+    const u32 d = min(threadIdx.x & 3u, 2u);
     const double side = box[3];
-    const int F = make_frame(box).F;
-    FastGrid g;
-    g.fast = F <= 900;  // so that subnormal coordinates are zero in fixed point
-    FixedGrid f;
-    for (int d = 0; d < 3; ++d) {
-        f = make_fixed_grid(box[d], side, F);
-        g.fast = g.fast && f.fast && f.F == F;
-        g.neg_lo[d] = 0ULL - static_cast<u64>(f.lo_fixed);
-        g.lo[d] = f.lo;
+    const FixedGrid f = make_fixed_grid(box[d], side);
+    int F = f.F, ok = f.ok;
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) {
+        F = min(F, __shfl_xor_sync(0xffffffffu, F, o));
+        ok &= __shfl_xor_sync(0xffffffffu, ok, o);
     }
-    g.inv = f.scale;
-    g.F = F;
-    g.scale = f.R >= 32 ? f.scale_fixed >> (f.R - 32) : f.scale_fixed;
-    g.d_shift = f.R >= 32 ? 0 : 32 - f.R;
-    g.e_end = static_cast<u32>(9 + 1075 - F);
-    g.d_end = g.fast ? static_cast<u32>(static_cast<u64>(to_fixed(side, F)) >> 32) : 0u;
-    return g;
+    const int R = F + f.R - f.F;
+    const int fast = ok && bound_holds(F, R) && F <= 900;  // so that subnormal coordinates are zero in fixed point
+    if (!write || (threadIdx.x & 3u) == 3u) return;
+    g->axis[d] = f;
+    g->neg_lo[d] = fast ? 0ULL - static_cast<u64>(to_fixed(f.lo, F)) : 0ULL;
+    if (d != 0) return;
+    g->scale = R >= 32 ? f.scale_fixed >> (R - 32) : f.scale_fixed;
+    g->d_shift = R >= 32 ? 0 : 32 - R;
+    g->e_end = static_cast<u32>(9 + 1075 - F);
+    g->d_end = fast ? static_cast<u32>(static_cast<u64>(to_fixed(side, F)) >> 32) : 0u;
+    g->fast = fast;
 }
 
 // X = trunc(x * 2^F) and its distance d from the box's corner; returns the exponent field.
@@ -278,12 +294,38 @@ __device__ __forceinline__ u64 mul_high(u64 a, u64 b) {
     return static_cast<u64>(ah) * bh + ((static_cast<u64>(al) * bh) >> 32) + __umulhi(ah, bl);
 }
 
-// Cell of one coordinate on the rare path: IEEE inside the frame; beyond it (where only boxes without
-// the error bound would compute anything), by the sign.
-__device__ __noinline__ u32 cell_exact(double x, const FastGrid& g, int d) {
-    const u32 hi = static_cast<u32>(__double2hiint(x));
-    if (g.fast && ((hi >> 20) & 0x7ffu) >= g.e_end) return (hi >> 31) ? 0u : 2097151u;
-    return grid_cell(x, g.lo[d], g.inv);
+// Cell of one coordinate on the rare path, d its axis: in the shared frame once more, since mostly another axis of
+// the particle led here; beyond the box by the order of the bits; where another axis of the box lies too far out
+// for the shared frame (10^6 sides from the origin), in the axis' own; at the borders of cells and where no bound
+// holds by IEEE arithmetic (inside the box without grid_cell's comparisons, which run at the FP64 rate too).
+// 2^25 Morton keys with IEEE arithmetic on all three axes, and so: one axis of the box far out 957 -> 479 us, every
+// tenth particle outside the box 939 -> 463, all on the borders of cells 960 -> 784.
+__device__ __forceinline__ u32 cell_exact(double x, const FastGrid& g, int d) {
+    const FixedGrid& f = g.axis[d];
+    if (g.fast) {
+        u64 X, dist;
+        const u32 e = to_frame(x, g.neg_lo[d], g.e_end, X, dist);
+        const u64 u = mul_high(dist << g.d_shift, g.scale);
+        if (e < g.e_end && static_cast<u32>(dist >> 32) < g.d_end && static_cast<u32>(u) + 0x1000u >= 0x2000u)
+            return static_cast<u32>(u >> 32);
+    }
+    if (!f.fast) return grid_cell(x, f.lo, f.scale);
+    const u64 o = order_bits(x);
+    if (o <= f.lo_ord) return 0u;
+    if (o >= f.hi_ord) return 2097151u;
+    if (!g.fast) {
+        const u64 u = __umul64hi(static_cast<u64>(to_fixed(x, f.F) - f.lo_fixed), f.scale_fixed);
+        const u32 frac20 = static_cast<u32>(u >> (f.R - 20)) & 0xfffffu;
+        const u64 c = u >> f.R;
+        if (frac20 != 0u && frac20 != 0xfffffu) return c > 2097151ULL ? 2097151u : static_cast<u32>(c);
+    }
+    return min(__double2uint_rz(__dmul_rn(__dsub_rn(x, f.lo), f.scale)), 2097151u);
+}
+
+// The three cells of a particle on the rare path, 21 bits each.
+__device__ __noinline__ u64 cells_exact(double px, double py, double pz, const FastGrid& g) {
+    return cell_exact(px, g, 0) | (static_cast<u64>(cell_exact(py, g, 1)) << 21) |
+           (static_cast<u64>(cell_exact(pz, g, 2)) << 42);
 }
 
 // Cells of a particle; X gets its fixed-point coordinates where the grid is fast. Returns whether all
@@ -307,9 +349,10 @@ __device__ __forceinline__ bool cells_of(const FastGrid& g, double px, double py
         sure = in && dh < g.d_end && frac >= 0x2000u;  // 2^-20 cells or more from every border
     }
     if (!sure) {
-        c[0] = cell_exact(px, g, 0);
-        c[1] = cell_exact(py, g, 1);
-        c[2] = cell_exact(pz, g, 2);
+        const u64 cells = cells_exact(px, py, pz, g);
+        c[0] = static_cast<u32>(cells) & 0x1fffffu;
+        c[1] = static_cast<u32>(cells >> 21) & 0x1fffffu;
+        c[2] = static_cast<u32>(cells >> 42);
     }
     return in;
 }
@@ -414,7 +457,7 @@ __global__ void __launch_bounds__(kKeyThreads, 3) keys_kernel(const double* __re
     __shared__ KeySmem sm;
     extern __shared__ unsigned short table[];  // kTableBytes<TL> for Hilbert keys
     if (CURVE == CSTONE_HILBERT) compose_table<TL>(sm, table, one);
-    if (threadIdx.x == 0) sm.grid = make_fast_grid(box);
+    if (threadIdx.x < 32) make_fast_grid(box, &sm.grid, threadIdx.x < 4);
     __syncthreads();
     auto encode = [&](double px, double py, double pz) -> Key {
         u32 c[3];
@@ -460,7 +503,7 @@ __global__ void __launch_bounds__(kKeyThreads, 2)
     __shared__ FixedFrame s_frame;
     extern __shared__ unsigned short table[];  // kTableBytes<TL> for Hilbert keys
     if (CURVE == CSTONE_HILBERT) compose_table<TL>(sm, table, one);
-    if (threadIdx.x == 0) sm.grid = make_fast_grid(box);
+    if (threadIdx.x < 32) make_fast_grid(box, &sm.grid, threadIdx.x < 4);
     if (threadIdx.x == 32) s_frame = make_frame(box);
     __syncthreads();
     const FixedFrame fr = s_frame;
@@ -689,8 +732,9 @@ __global__ void __cluster_dims__(kBoxCluster, 1, 1) __launch_bounds__(kBoxThread
 }
 
 __global__ void keys_batched_setup_kernel(const double* __restrict__ boxes, int n_sets, FastGrid* grids) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n_sets; i += gridDim.x * blockDim.x)
-        grids[i] = make_fast_grid(boxes + 4 * i);
+    const int set = static_cast<int>((blockIdx.x * blockDim.x + threadIdx.x) >> 2);  // four lanes per set
+    const int at = min(set, n_sets - 1);
+    make_fast_grid(boxes + 4 * at, grids + at, set < n_sets);
 }
 
 // A block takes a stretch of consecutive tiles of particles. Where a tile lies in one set, which one load
@@ -729,7 +773,8 @@ __global__ void __launch_bounds__(kKeyThreads, 3) keys_batched_kernel(const doub
             first = __ldg(set_offsets + set);
             end = __ldg(set_offsets + set + 1);
             __syncthreads();  // the table, and the previous set's grids
-            if (threadIdx.x == 0) sm.grid = grids[set];
+            if (threadIdx.x < sizeof(FastGrid) / 8)
+                reinterpret_cast<u64*>(&sm.grid)[threadIdx.x] = __ldg(reinterpret_cast<const u64*>(grids + set) + threadIdx.x);
             __syncthreads();
         }
         const bool whole = t0 >= first && t1 <= end;
@@ -782,7 +827,7 @@ int launch_keys_batched(const double* x, const double* y, const double* z, const
                         long long n, const double* boxes, int curve, Key* keys, void* ws, cudaStream_t st) {
     Carver c(ws);
     FastGrid* grids = c.take<FastGrid>((size_t)n_sets);
-    keys_batched_setup_kernel<<<(n_sets + 127) / 128, 128, 0, st>>>(boxes, n_sets, grids);
+    keys_batched_setup_kernel<<<(n_sets + 31) / 32, 128, 0, st>>>(boxes, n_sets, grids);
     CST_LAUNCHED("keys_batched_setup_kernel");
     if (n == 0) return CSTONE_OK;
     const HilbertTable& tab = hilbert_table();

@@ -738,7 +738,8 @@ __global__ void keys_batched_setup_kernel(const double* __restrict__ boxes, int 
 }
 
 // A block takes a stretch of consecutive tiles of particles. Where a tile lies in one set, which one load
-// shows, its grids are read from shared memory, else every particle looks its set up.
+// shows, its grid is read from shared memory, else every particle looks its set up; so does every particle
+// of sets that are smaller than a tile on average (by_tile is 0), instead of a search before its own.
 constexpr int kBatchItems = 2;
 constexpr int kBatchTile = kKeyThreads * kBatchItems;
 
@@ -747,31 +748,33 @@ __global__ void __launch_bounds__(kKeyThreads, 3) keys_batched_kernel(const doub
                                                                      const double* __restrict__ y,
                                                                      const double* __restrict__ z,
                                                                      const long long* __restrict__ set_offsets, int n_sets,
-                                                                     long long n, const FastGrid* __restrict__ grids,
+                                                                     long long n, int by_tile, const FastGrid* __restrict__ grids,
                                                                      Key* __restrict__ keys,
                                                                      const __grid_constant__ HilbertTable one) {
     __shared__ KeySmem sm;
     extern __shared__ unsigned short table[];  // kTableBytes<TL> for Hilbert keys
     if (CURVE == CSTONE_HILBERT) compose_table<TL>(sm, table, one);
-    const long long tiles = (n + kBatchTile - 1) / kBatchTile;
-    const long long b0 = tiles * blockIdx.x / gridDim.x, b1 = tiles * (blockIdx.x + 1) / gridDim.x;
-    int set = -1;                  // set of the tile's first particle
-    long long first = 0, end = 0;  // its particles
-    for (long long tile = b0; tile < b1; ++tile) {
-        const long long t0 = tile * kBatchTile, t1 = min(t0 + kBatchTile, n);
+    const u32 tiles = static_cast<u32>((n + kBatchTile - 1) / kBatchTile);
+    const u32 b0 = static_cast<u32>(static_cast<u64>(tiles) * blockIdx.x / gridDim.x);
+    const u32 b1 = static_cast<u32>(static_cast<u64>(tiles) * (blockIdx.x + 1) / gridDim.x);
+    int set = 0;              // set of the tile's first particle
+    u32 first = 0, end = 0;   // its particles
+    if (!by_tile) __syncthreads();  // the table
+    for (u32 tile = b0; tile < b1; ++tile) {
+        const u32 t0 = tile * kBatchTile, t1 = min(t0 + kBatchTile, static_cast<u32>(n));
         double p[kBatchItems][3];
 #pragma unroll
         for (int k = 0; k < kBatchItems; ++k) {
-            const long long i = t0 + k * kKeyThreads + threadIdx.x;
+            const u32 i = t0 + k * kKeyThreads + threadIdx.x;
             const bool on = i < t1;
             p[k][0] = on ? __ldcg(x + i) : 0.0;
             p[k][1] = on ? __ldcg(y + i) : 0.0;
             p[k][2] = on ? __ldcg(z + i) : 0.0;
         }
-        if (t0 >= end) {  // the same in every thread
+        if (by_tile && t0 >= end) {  // the same in every thread
             set = set_of(set_offsets, n_sets, t0);
-            first = __ldg(set_offsets + set);
-            end = __ldg(set_offsets + set + 1);
+            first = static_cast<u32>(__ldg(set_offsets + set));
+            end = static_cast<u32>(__ldg(set_offsets + set + 1));
             __syncthreads();  // the table, and the previous set's grids
             if (threadIdx.x < sizeof(FastGrid) / 8)
                 reinterpret_cast<u64*>(&sm.grid)[threadIdx.x] = __ldg(reinterpret_cast<const u64*>(grids + set) + threadIdx.x);
@@ -780,7 +783,7 @@ __global__ void __launch_bounds__(kKeyThreads, 3) keys_batched_kernel(const doub
         const bool whole = t0 >= first && t1 <= end;
 #pragma unroll
         for (int k = 0; k < kBatchItems; ++k) {
-            const long long i = t0 + k * kKeyThreads + threadIdx.x;
+            const u32 i = t0 + k * kKeyThreads + threadIdx.x;
             u32 c[3];
             u64 X[3];
             if (whole || (i >= first && i < end))
@@ -809,6 +812,14 @@ const HilbertDecodeTable& hilbert_decode_table() {
     return dec;
 }
 
+// Dynamic shared memory beyond the default limit (48 KB with the static part) for the three-level table.
+template <class Kernel>
+int allow_table(Kernel kernel, size_t smem) {
+    if (smem > kTableBytes<2>)
+        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+    return CSTONE_OK;
+}
+
 size_t keys_batched_ws_bytes(int n_sets) {
     Carver c(nullptr);
     c.take<FastGrid>((size_t)n_sets);
@@ -831,11 +842,12 @@ int launch_keys_batched(const double* x, const double* y, const double* z, const
     CST_LAUNCHED("keys_batched_setup_kernel");
     if (n == 0) return CSTONE_OK;
     const HilbertTable& tab = hilbert_table();
+    const int by_tile = n >= static_cast<long long>(n_sets) * kBatchTile ? 1 : 0;
     const long long want = (n + kBatchTile - 1) / kBatchTile, most = (long long)sm_count() * kKeyBlocks;
     const unsigned grid = static_cast<unsigned>(want < most ? want : most);
     auto launch = [&](auto kernel, size_t smem) -> int {
-        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-        kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, set_offsets, n_sets, n, grids, keys, tab);
+        if (int rc = allow_table(kernel, smem)) return rc;
+        kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, set_offsets, n_sets, n, by_tile, grids, keys, tab);
         CST_LAUNCHED("keys_batched_kernel");
         return CSTONE_OK;
     };
@@ -853,7 +865,7 @@ int launch_keys(const double* x, const double* y, const double* z, long long n, 
     const bool vec = ((reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) | reinterpret_cast<uintptr_t>(z) |
                        reinterpret_cast<uintptr_t>(keys)) & 15u) == 0;
     auto launch = [&](auto kernel, size_t smem) -> int {
-        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        if (int rc = allow_table(kernel, smem)) return rc;
         kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, n, box, keys, tab);
         CST_LAUNCHED("keys_kernel");
         return CSTONE_OK;
@@ -878,7 +890,7 @@ int launch_keys_records(const double* x, const double* y, const double* z, const
     const long long want = (n + per - 1) / per, most = (long long)sm_count() * kKeyBlocks;
     const unsigned grid = static_cast<unsigned>(want < most ? want : most);
     auto launch = [&](auto kernel, size_t smem) -> int {
-        CST_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+        if (int rc = allow_table(kernel, smem)) return rc;
         kernel<<<grid, kKeyThreads, smem, st>>>(x, y, z, m, n, box, keys, rec, hdr, tab);
         CST_LAUNCHED("keys_records_kernel");
         return CSTONE_OK;

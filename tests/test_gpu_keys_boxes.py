@@ -49,10 +49,11 @@ def test_single_set(lib, oracle, name, levels):
             assert np.array_equal(got, oracle.keys(x, y, z, box, curve, levels=levels)), (n, curve)
 
 
+# sets of a tile of 1024 particles on average or more, and of fewer: looked up by tile, and by particle
+@pytest.mark.parametrize("sizes", [(5, 1023, 0, 1024, 3000, 1, 2, 700, 4097), (5, 1023, 0, 1024, 2000, 1, 2, 64, 1100)])
 @pytest.mark.parametrize("curve", [0, 1])
-def test_sets_with_boxes_of_their_own(lib, oracle, curve):
+def test_sets_with_boxes_of_their_own(lib, oracle, curve, sizes):
     rng = np.random.default_rng(curve)
-    sizes = [5, 1023, 0, 1024, 3000, 1, 2, 700, 4097]
     off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
     parts = [[c[:n] for c in _particles(rng, max(n, 64), *BOXES[b])] for n, b in zip(sizes, BOXES)]
     x, y, z = (np.concatenate([p[d] for p in parts]) for d in range(3))

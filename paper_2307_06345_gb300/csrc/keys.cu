@@ -633,13 +633,15 @@ __device__ __forceinline__ int set_of(const long long* __restrict__ set_offsets,
 // Bounding cube of every set: one cluster of kBoxCluster blocks per set (a large set is read by
 // kBoxCluster SMs, not one); each block reduces its share of the set, and the cluster's first block
 // combines the blocks' results from their shared memory (distributed shared memory of the cluster).
-// Bound by loads in flight and by clusters, which start only where 16 blocks are free: pairs of particles by
-// 16-byte loads (512 sets, 77 million particles: 446 -> 399 us); more in flight per thread (405 to 425), 512
-// threads (559) or clusters of 8 (391, with 512 threads; the small sets' 10.7 -> 11.3) gained nothing more.
+// Bound by loads in flight and by clusters, which start only where 16 blocks are free: six blocks per SM (with 44
+// registers and five, 500 sets of 2 or 2,000 particles took 68 and 76 us; so 60 and 66). Large sets are read in
+// pairs of particles by 16-byte loads (512 sets of 1,024 to 1,048,576: 457 -> 406 us; 4 of 4 million 474 -> 328); more
+// in flight per thread, 512 threads or clusters of 8 gained nothing more. Sets of at most two particles per thread
+// are read one by one, since the pairs' odd ends would be a second round of loads.
 constexpr int kBoxCluster = 16;  // a non-portable cluster size, allowed per kernel at launch
 constexpr int kBoxThreads = 256;
 
-__global__ void __cluster_dims__(kBoxCluster, 1, 1) __launch_bounds__(kBoxThreads)
+__global__ void __cluster_dims__(kBoxCluster, 1, 1) __launch_bounds__(kBoxThreads, 6)
     bbox_batched_kernel(const double* __restrict__ x, const double* __restrict__ y, const double* __restrict__ z,
                         const long long* __restrict__ set_offsets, double* __restrict__ boxes) {
     __shared__ long long s_lo[kBoxThreads / 32][3], s_hi[kBoxThreads / 32][3];
@@ -657,9 +659,10 @@ __global__ void __cluster_dims__(kBoxCluster, 1, 1) __launch_bounds__(kBoxThread
     };
     const long long first = static_cast<long long>(rank) * kBoxThreads + threadIdx.x;
     constexpr long long kStep = static_cast<long long>(kBoxCluster) * kBoxThreads;
+    constexpr long long kPairsFrom = 2 * kStep;
     const uintptr_t bases = reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y) |
                             reinterpret_cast<uintptr_t>(z);
-    if ((bases & 15u) == 0) {  // pairs of particles of even index, and the odd ones at the set's ends
+    if ((bases & 15u) == 0 && b - a > kPairsFrom) {  // pairs of particles of even index, and the odd ones at the set's ends
         const long long q1 = b >> 1;
         for (long long q = ((a + 1) >> 1) + first; q < q1; q += kStep) {
             double2 v[3];

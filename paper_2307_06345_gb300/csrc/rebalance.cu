@@ -230,20 +230,23 @@ __device__ __forceinline__ bool outside_focus(Key start, Key size, Key f_start, 
     return f_end <= f_start || start + size <= f_start || start >= f_end;
 }
 
-// r_min^2 of the cube [c, c + edge)^3 against the focus tiles held in shared memory, by a whole warp
-// (each lane takes every 32nd tile); all ones for an empty focus.
+// Squared distance of the cube [c, c + edge)^3 from a focus tile (corner and edge).
+__device__ __forceinline__ u64 tile_distance(const u32 c[3], u32 edge, const u32 t[4]) {
+    u64 r2 = 0;
+#pragma unroll
+    for (int d = 0; d < 3; ++d) {
+        const u32 a1 = c[d] + edge, b0 = t[d], b1 = b0 + t[3];
+        const u32 gap = b0 > a1 ? b0 - a1 : (c[d] > b1 ? c[d] - b1 : 0u);
+        r2 += static_cast<u64>(gap) * gap;
+    }
+    return r2;
+}
+
+// r_min^2 of the cube against the focus tiles held in shared memory, by a whole warp (each lane takes every 32nd
+// tile).
 __device__ __forceinline__ u64 warp_distance(const u32 c[3], u32 edge, const u32 (*tc)[4], int nt) {
     u64 best = ~0ULL;
-    for (int t = threadIdx.x & 31; t < nt; t += 32) {
-        u64 r2 = 0;
-#pragma unroll
-        for (int d = 0; d < 3; ++d) {
-            const u32 a1 = c[d] + edge, b0 = tc[t][d], b1 = b0 + tc[t][3];
-            const u32 gap = b0 > a1 ? b0 - a1 : (c[d] > b1 ? c[d] - b1 : 0u);
-            r2 += static_cast<u64>(gap) * gap;
-        }
-        best = r2 < best ? r2 : best;
-    }
+    for (int t = threadIdx.x & 31; t < nt; t += 32) best = min(best, tile_distance(c, edge, tc[t]));
     const u32 hi = __reduce_min_sync(0xffffffffu, static_cast<u32>(best >> 32));
     const u32 low = static_cast<u32>(best >> 32) == hi ? static_cast<u32>(best) : 0xffffffffu;
     const u32 lo = __reduce_min_sync(0xffffffffu, low);
@@ -254,7 +257,11 @@ __device__ __forceinline__ u64 warp_distance(const u32 c[3], u32 edge, const u32
 // outside F and one for every parent of eight siblings outside F (its siblings in the warp share the
 // answer), and (l / theta)^2 is tabulated by level: a thread per eight leaves that went through all
 // focus tiles itself, for every sibling, with two FP64 operations each, took 177 us for 2.3e5 leaves
-// and 100 tiles on GB300 (FP64 division is a few operations per SM and clock).
+// and 100 tiles on GB300 (FP64 division is a few operations per SM and clock). With a few tiles, or none, every
+// lane goes through them itself: the warp would take as long for one of its lanes as a lane for all of them.
+// A step of 2.4e6 leaves and one tile: 166 us with a thread per eight leaves, 203 by warps, 116 so.
+constexpr int kFewTiles = 8;
+template <bool FEW>
 __global__ void __launch_bounds__(kThreads) focus_ops_kernel(const Key* __restrict__ K, const u32* __restrict__ N,
                                                              u32 nl, u32 ncrit, const __grid_constant__ FocusParams fp,
                                                              const __grid_constant__ HilbertDecodeTable dt,
@@ -306,25 +313,36 @@ __global__ void __launch_bounds__(kThreads) focus_ops_kernel(const Key* __restri
                 }
             }
         }
-        if (ask_leaf || (ask_parent && leader == lane)) key_cell(ke, fp.curve, s_dec, c);
+        if (fp.n_tiles > 0 && (ask_leaf || (ask_parent && leader == lane))) key_cell(ke, fp.curve, s_dec, c);
     }
     u32 far_leaf = 0, far_parent = 0;  // bit per lane: the MAC accepts its leaf; the parent it asks for
-    for (int kind = 0; kind < 2; ++kind) {
-        u32 todo = __ballot_sync(0xffffffffu, kind == 0 ? ask_leaf : ask_parent && leader == lane);
-        while (todo != 0u) {
-            const int l = __ffs(todo) - 1;
-            todo &= todo - 1u;
-            const int lv = __shfl_sync(0xffffffffu, level, l) - kind;
-            const u32 edge = 1u << (kLevels - lv);
-            u32 q[3];
+    if (FEW) {
+        auto is_far = [&](int lv) -> bool {
+            const u32 edge = 1u << (kLevels - lv), q[3] = {c[0] & ~(edge - 1u), c[1] & ~(edge - 1u), c[2] & ~(edge - 1u)};
+            u64 r2 = ~0ULL;
+            for (int t = 0; t < fp.n_tiles; ++t) r2 = min(r2, tile_distance(q, edge, s_tile[t]));
+            return fp.n_tiles == 0 || __ull2double_rn(r2) > s_reach[lv];  // an empty focus accepts every node
+        };
+        far_leaf = __ballot_sync(0xffffffffu, ask_leaf && is_far(level));
+        far_parent = __ballot_sync(0xffffffffu, ask_parent && leader == lane && is_far(level - 1));
+    } else {
+        for (int kind = 0; kind < 2; ++kind) {
+            u32 todo = __ballot_sync(0xffffffffu, kind == 0 ? ask_leaf : ask_parent && leader == lane);
+            while (todo != 0u) {
+                const int l = __ffs(todo) - 1;
+                todo &= todo - 1u;
+                const int lv = __shfl_sync(0xffffffffu, level, l) - kind;
+                const u32 edge = 1u << (kLevels - lv);
+                u32 q[3];
 #pragma unroll
-            for (int d = 0; d < 3; ++d) q[d] = __shfl_sync(0xffffffffu, c[d], l) & ~(edge - 1u);
-            const u64 r2 = warp_distance(q, edge, s_tile, fp.n_tiles);
-            const bool far = fp.n_tiles == 0 || __ull2double_rn(r2) > s_reach[lv];  // an empty focus accepts every node
-            if (kind == 0)
-                far_leaf |= far ? 1u << l : 0u;
-            else
-                far_parent |= far ? 1u << l : 0u;
+                for (int d = 0; d < 3; ++d) q[d] = __shfl_sync(0xffffffffu, c[d], l) & ~(edge - 1u);
+                const u64 r2 = warp_distance(q, edge, s_tile, fp.n_tiles);
+                const bool far = __ull2double_rn(r2) > s_reach[lv];
+                if (kind == 0)
+                    far_leaf |= far ? 1u << l : 0u;
+                else
+                    far_parent |= far ? 1u << l : 0u;
+            }
         }
     }
     u32 op = 0;
@@ -399,8 +417,9 @@ int launch_rebalance(const Key* K, const u32* N, long long nl, u32 ncrit, Key* K
                                                         static_cast<char*>(ws)), st));
     if (focus) {
         const unsigned blocks = static_cast<unsigned>((nl + 1 + kThreads - 1) / kThreads);
-        focus_ops_kernel<<<blocks, kThreads, 0, st>>>(K, N, static_cast<u32>(nl), ncrit, *focus,
-                                                        hilbert_decode_table(), l.O, l.tile_sums, l.st);
+        auto* ops = focus->n_tiles <= kFewTiles ? focus_ops_kernel<true> : focus_ops_kernel<false>;
+        ops<<<blocks, kThreads, 0, st>>>(K, N, static_cast<u32>(nl), ncrit, *focus, hilbert_decode_table(), l.O, l.tile_sums,
+                                         l.st);
         CST_LAUNCHED("focus_ops_kernel");
     } else {
         rebalance_ops_kernel<<<l.ntiles, kThreads, 0, st>>>(K, N, static_cast<u32>(nl), ncrit, l.O, l.tile_sums,

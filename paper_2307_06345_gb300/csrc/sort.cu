@@ -268,23 +268,20 @@ __device__ __forceinline__ u32 bin_add(u32* bins, u32 b) {  // the pair's rank i
     return (b & 1u) ? was >> 16 : was & 0xffffu;
 }
 
-// How a set of pairs is binned: the leading nb of the `top` low bits in which the keys' distances
-// from the base differ, followed by leading bits of the value where that is fewer than nb; equal keys
-// by the leading nb of the `vtop` low bits in which their values differ.
+// How a set of pairs is binned: by the leading nb of the `top` low bits in which the keys' distances from the
+// base differ, followed, where those are fewer than nb, by the leading ones of the `vtop` low bits in which the
+// values differ. (The values of a part that lies among equal keys are close together: bins by the leading bits
+// of any index would all but one stay empty, and the part take another step.)
 struct BinMap {
     int top, vtop, nb;
-    __device__ __forceinline__ u32 bin(Key d, u32 v, int idx_bits) const {
+    __device__ __forceinline__ u32 bin(Key d, u32 v) const {
         if (top >= nb) {
             const Key low = d & (~static_cast<Key>(0) >> (kWordBits - top));
             return static_cast<u32>(low >> (top - nb));
         }
-        if (top > 0) {
-            const int up = nb - top;
-            const u32 low = static_cast<u32>(d) & ((1u << top) - 1u);
-            return (low << up) | (v >> max(0, idx_bits - up));
-        }
+        const int up = nb - top;  // bits left for the value
         const u32 low = vtop >= 32 ? v : v & ((1u << vtop) - 1u);
-        return low >> max(0, vtop - nb);
+        return ((static_cast<u32>(d) & ((1u << top) - 1u)) << up) | (low >> max(0, vtop - up));
     }
 };
 
@@ -305,14 +302,14 @@ __device__ __forceinline__ u32 rank_in_bin(const Smem& sm, Key k, u32 v, u32 b0,
 
 // Sorts m <= THREADS * ITEMS pairs: load(e, key, value) gives pair e, out(position, key, value)
 // takes each at its place in the sorted order. Every load comes before any out. No key may be
-// below base; idx_bits bounds the values.
+// below base.
 //
 // The first step bins all pairs, m <= bins < 2 m. A pair whose bin holds at most kHeavy pairs is
 // ranked there by comparison and leaves; the larger bins are the groups of the next step, which
 // bins all of them at once, each over its own differing bits, and so on. A step takes four bits
 // or more off a group's keys (or values), so the steps end.
 template <int THREADS, int ITEMS, class Load, class Out>
-__device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, int idx_bits, Load load, Out out) {
+__device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, Load load, Out out) {
     const u32 tid = threadIdx.x;
     const int lane = tid & 31, warp = tid >> 5;
     const u16* starts = reinterpret_cast<const u16*>(sm.bins);  // little-endian halves
@@ -344,12 +341,31 @@ __device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, i
 #pragma unroll
         for (int w = 0; w < THREADS / 32; ++w) ored |= sm.red[w];
         map.top = bit_length(ored);
-        map.vtop = idx_bits;
+        map.vtop = 0;
         // the usual case needs no mask (the distances have `top` bits) and nothing of the values
         const bool plain = map.top >= map.nb;
         const int sh = map.top - map.nb;
+        if (!plain) {  // the values are loaded once more: with this branch on registers the usual case is 1 % slower
+            if (tid == 0) {
+                sm.diff[0][0] = val[0];
+                sm.diff[2][0] = 0u;
+            }
+            __syncthreads();
+            u32 differ = 0;
+#pragma unroll 1
+            for (u32 e = tid; e < m; e += THREADS) {
+                Key k;
+                u32 v;
+                load(e, k, v);
+                differ |= v ^ sm.diff[0][0];
+            }
+            differ = __reduce_or_sync(0xffffffffu, differ);
+            if (lane == 0) atomicOr(&sm.diff[2][0], differ);
+            __syncthreads();
+            map.vtop = 32 - __clz(static_cast<int>(sm.diff[2][0]));
+        }
         auto bin_of = [&](Key k, u32 v) -> u32 {
-            return plain ? static_cast<u32>((k - base) >> sh) : map.bin(k - base, v, idx_bits);
+            return plain ? static_cast<u32>((k - base) >> sh) : map.bin(k - base, v);
         };
         // unconditional, so that a thread's atomics are in flight together (with a test per slot the
         // kernel is a fifth slower): a slot without a pair adds nothing to a word of its lane
@@ -462,7 +478,7 @@ __device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, i
             const u32 e = tid + i * THREADS;
             if (e < left) {
                 const u32 g = group_of(e);
-                const u32 b = (sm.first[g] >> 16) + map_of(g).bin(key[i] - base, val[i], idx_bits);
+                const u32 b = (sm.first[g] >> 16) + map_of(g).bin(key[i] - base, val[i]);
                 at[i] = b | (bin_add(sm.bins, b) << 16);
             }
         }
@@ -486,7 +502,7 @@ __device__ void block_sort(BlockSortSmem<THREADS, ITEMS>& sm, u32 m, Key base, i
             const u32 s0 = group[g] & 0xffffu, s = s0 + e - (sm.first[g] & 0xffffu);
             const Key k = sm.K[s];
             const u32 v = sm.V[s];
-            const u32 o = sm.first[g] >> 16, b = o + map.bin(k - base, v, idx_bits);
+            const u32 o = sm.first[g] >> 16, b = o + map.bin(k - base, v);
             const u32 b0 = s0 + starts[b] - starts[o], b1 = s0 + starts[b + 1] - starts[o];
             // equal pairs, which only overlapping segments could give, cannot be split
             if (b1 - b0 <= kHeavy || (map.top == 0 && map.vtop == 0))
@@ -517,8 +533,8 @@ __device__ __forceinline__ u32 hash32(u32 x) {  // Wang's integer mix (public do
 // A sort of one set starts here (single = its keys, else 0): its tables have one bucket, and the
 // launch that lists segments is not needed.
 template <int SRC>
-__global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Buckets b, Tables t, int idx_bits, u32 single,
-                                                                 int rounds, WsHeader* hdr) {
+__global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Buckets b, Tables t, u32 single, int rounds,
+                                                                 WsHeader* hdr) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BigSmem& sm = *reinterpret_cast<BigSmem*>(smem_raw);
     if (single != 0) {  // one block
@@ -546,7 +562,7 @@ __global__ void __launch_bounds__(kBigThreads) sort_sample_kernel(Pairs p, Bucke
         const Key* keys = keys_of<SRC>(p);
         const Key base = b.base[k];
         block_sort<kBigThreads, kBigItems>(
-            sm, ns, base, idx_bits,
+            sm, ns, base,
             [&](u32 e, Key& key, u32& val) {
                 const u32 lo = static_cast<u32>(static_cast<u64>(e) * size / ns);
                 const u32 hi = static_cast<u32>(static_cast<u64>(e + 1) * size / ns);
@@ -819,7 +835,7 @@ __global__ void __launch_bounds__(kThreads, CSTONE_SORT_MIN_BLOCKS) sort_scatter
 
 // ---------------------------------------------------------------------------- final sort
 // Every listed part, one block each, from wherever it is to its place in the output.
-__global__ void __launch_bounds__(kSmallThreads, kSmallBlocks) sort_small_kernel(Pairs p, Tables t, int idx_bits) {
+__global__ void __launch_bounds__(kSmallThreads, kSmallBlocks) sort_small_kernel(Pairs p, Tables t) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SmallSmem& sm = *reinterpret_cast<SmallSmem*>(smem_raw);
     const u32 count = *t.n_small;
@@ -829,7 +845,7 @@ __global__ void __launch_bounds__(kSmallThreads, kSmallBlocks) sort_small_kernel
         const Key* keys = src == kInput ? p.in : (src == kBufA ? p.a : p.b);
         const u32* vals = src == kBufA ? p.va : p.vb;
         block_sort<kSmallThreads, kSmallItems>(
-            sm, m, t.small_base[k], idx_bits,
+            sm, m, t.small_base[k],
             [&](u32 e, Key& key, u32& val) {
                 key = __ldcg(keys + start + e);
                 val = src == kInput ? start + e : __ldcg(vals + start + e);
@@ -846,7 +862,7 @@ __global__ void __launch_bounds__(kSmallThreads, kSmallBlocks) sort_small_kernel
 // in shared memory, then merged pairwise between the part's ranges of the two buffers. LAST: the
 // buffer that the last round wrote.
 template <int LAST>
-__global__ void __launch_bounds__(kBigThreads) sort_rest_kernel(Pairs p, Buckets b, int idx_bits) {
+__global__ void __launch_bounds__(kBigThreads) sort_rest_kernel(Pairs p, Buckets b) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     BigSmem& sm = *reinterpret_cast<BigSmem*>(smem_raw);
     const u32 count = *b.count;
@@ -864,7 +880,7 @@ __global__ void __launch_bounds__(kBigThreads) sort_rest_kernel(Pairs p, Buckets
             Key* ko = (in_b ? p.b : p.a) + start + c;
             u32* vo = (in_b ? p.vb : p.va) + start + c;
             block_sort<kBigThreads, kBigItems>(
-                sm, m, base, idx_bits,
+                sm, m, base,
                 [&](u32 e, Key& key, u32& val) {
                     key = __ldcg(k0 + c + e);
                     val = __ldcg(v0 + c + e);
@@ -1316,13 +1332,13 @@ SortLayout sort_layout(void* ws, long long n, int n_segs) {
 
 template <int SRC>
 int run_round(const Pairs& p, const SortLayout& l, const Buckets& cur, const Buckets& next, long long max_big,
-              int idx_bits, u32 single, int rounds, WsHeader* hdr, cudaStream_t st) {
+              u32 single, int rounds, WsHeader* hdr, cudaStream_t st) {
     const int sms = sm_count();
     const int smem = static_cast<int>(sizeof(BigSmem)), ssmem = static_cast<int>(sizeof(ScatterSmem));
     CST_CUDA(cudaFuncSetAttribute(sort_sample_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     CST_CUDA(cudaFuncSetAttribute(sort_scatter_kernel<SRC>, cudaFuncAttributeMaxDynamicSharedMemorySize, ssmem));
     const int bgrid = static_cast<int>(max_big < 2 * sms ? max_big : 2 * sms);
-    sort_sample_kernel<SRC><<<bgrid, kBigThreads, smem, st>>>(p, cur, l.t, idx_bits, single, rounds, hdr);
+    sort_sample_kernel<SRC><<<bgrid, kBigThreads, smem, st>>>(p, cur, l.t, single, rounds, hdr);
     CST_LAUNCHED("sort_sample_kernel");
     sort_count_kernel<SRC><<<sms * kCountBlocks, kThreads, 0, st>>>(p, cur, l.t);
     CST_LAUNCHED("sort_count_kernel");
@@ -1345,8 +1361,6 @@ int run_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, const lo
     if (!seg_offsets && digits::taken(n)) return digits::run(keys_in, keys_out, perm, n, ws, st);
     const int rounds = rounds_for(n);
     const Pairs p{keys_in, l.keys_a, l.vals_a, keys_out, perm};
-    int idx_bits = 1;
-    while ((1ll << idx_bits) < n) ++idx_bits;
     const u32 single = !seg_offsets && rounds > 0 ? static_cast<u32>(n) : 0u;
     if (single == 0) {
         sort_init_kernel<<<1, 1024, 0, st>>>(seg_offsets, n_segs, n, rounds, l.t, hdr);
@@ -1356,29 +1370,27 @@ int run_sort(const Key* keys_in, Key* keys_out, u32* perm, long long n, const lo
     const long long cap = static_cast<long long>(sort_sizes(n, n_segs).big);
     const long long cap1 = cap < n_segs ? cap : n_segs;
     if (rounds >= 1) {
-        if (int rc = run_round<kInput>(p, l, l.t.big[0], l.t.big[1], cap1, idx_bits, single, rounds, hdr, st)) return rc;
+        if (int rc = run_round<kInput>(p, l, l.t.big[0], l.t.big[1], cap1, single, rounds, hdr, st)) return rc;
     }
     if (rounds == 2) {
         sort_prefix_kernel<<<1, 1024, 0, st>>>(l.t.big[1], l.t.big[0].count, 1);
         CST_LAUNCHED("sort_prefix_kernel");
-        if (int rc = run_round<kBufA>(p, l, l.t.big[1], l.t.big[0], cap, idx_bits, 0u, 1, hdr, st)) return rc;
+        if (int rc = run_round<kBufA>(p, l, l.t.big[1], l.t.big[0], cap, 0u, 1, hdr, st)) return rc;
     }
     const int sms = sm_count();
     const int smem = static_cast<int>(sizeof(SmallSmem)), bsmem = static_cast<int>(sizeof(BigSmem));
     CST_CUDA(cudaFuncSetAttribute(sort_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const long long want = static_cast<long long>(sort_sizes(n, n_segs).small);
     const unsigned sgrid = static_cast<unsigned>(want < kSmallBlocks * sms ? want : kSmallBlocks * sms);
-    sort_small_kernel<<<sgrid, kSmallThreads, smem, st>>>(p, l.t, idx_bits);
+    sort_small_kernel<<<sgrid, kSmallThreads, smem, st>>>(p, l.t);
     CST_LAUNCHED("sort_small_kernel");
     if (rounds == 1) {
         CST_CUDA(cudaFuncSetAttribute(sort_rest_kernel<kBufA>, cudaFuncAttributeMaxDynamicSharedMemorySize, bsmem));
-        sort_rest_kernel<kBufA><<<(unsigned)(cap < 2 * sms ? cap : 2 * sms), kBigThreads, bsmem, st>>>(p, l.t.big[1],
-                                                                                                        idx_bits);
+        sort_rest_kernel<kBufA><<<(unsigned)(cap < 2 * sms ? cap : 2 * sms), kBigThreads, bsmem, st>>>(p, l.t.big[1]);
         CST_LAUNCHED("sort_rest_kernel");
     } else if (rounds == 2) {
         CST_CUDA(cudaFuncSetAttribute(sort_rest_kernel<kBufB>, cudaFuncAttributeMaxDynamicSharedMemorySize, bsmem));
-        sort_rest_kernel<kBufB><<<(unsigned)(cap < 2 * sms ? cap : 2 * sms), kBigThreads, bsmem, st>>>(p, l.t.big[0],
-                                                                                                        idx_bits);
+        sort_rest_kernel<kBufB><<<(unsigned)(cap < 2 * sms ? cap : 2 * sms), kBigThreads, bsmem, st>>>(p, l.t.big[0]);
         CST_LAUNCHED("sort_rest_kernel");
     }
     return CSTONE_OK;

@@ -1,5 +1,6 @@
 """Sorts whose parts are hard for the last step: keys in fewer bits than it has bins (the values decide, over the
-bits in which they differ)."""
+bits in which they differ), and sets whose first sample misses nearly every key, so that the second round's parts
+are larger than a block sorts at once and are merged in global memory."""
 import numpy as np
 import pytest
 import torch
@@ -31,3 +32,22 @@ def test_keys_of_few_bits(lib, n, values):
     _check(lib, k + np.uint64(77), levels=10)
     off = np.array([0, n // 3, n // 3 + 40, n - 3000 if n > 9000 else n // 2, n], np.int64)
     _check(lib, k, off=off)
+
+
+@pytest.mark.parametrize("n", [2_000_003, 8_000_003])  # merges of chunks of 8192: none and one; one and two
+def test_first_sample_misses_the_set(lib, n):
+    full = -(-n // 1536)
+    parts = max(min(int(np.sqrt(np.float32(full))) + 1, 256), min(-(-full // 384), 512))
+    ns = parts * min(32, 8192 // parts)
+    e = np.arange(ns, dtype=np.uint64)
+    lo, hi = e * np.uint64(n) // np.uint64(ns), (e + np.uint64(1)) * np.uint64(n) // np.uint64(ns)
+    with np.errstate(over="ignore"):
+        x = e.astype(np.uint32)  # the sample's integer hash of e
+        x = (x ^ np.uint32(61)) ^ (x >> np.uint32(16))
+        x = x * np.uint32(9)
+        x = x ^ (x >> np.uint32(4))
+        x = x * np.uint32(0x27D4EB2D)
+        x = x ^ (x >> np.uint32(15))
+    k = np.random.default_rng(n).integers(1 << 40, 1 << 63, n, dtype=np.uint64)
+    k[(lo + x.astype(np.uint64) % (hi - lo)).astype(np.int64)] = e
+    _check(lib, k)

@@ -13,8 +13,9 @@
 // flip of a level is the parity of the Gray-coded third axis above it. Tracking (permutation,
 // flips, parity) as a state gives 48 reachable states. The host builds the one-level table
 // (state, octant) -> (digit, next state) once and passes it to the kernels as a by-value
-// parameter (no device memory or symbol upload); each block composes it into a three-level table
-// in shared memory, so a 21-level key takes 7 lookups.
+// parameter (no device memory or symbol upload); each block composes it into a table of several levels
+// in shared memory: three from 2^22 particles on, so that a 21-level key takes 7 lookups, and two below
+// (11 lookups), where composing the larger table would take longer than the keys.
 #include <mutex>
 
 #include <cooperative_groups.h>
@@ -357,8 +358,8 @@ __device__ __forceinline__ bool cells_of(const FastGrid& g, double px, double py
     return in;
 }
 
-// Every third bit of a word: bit b of the low 10 bits to bit 3b. The multiplications run beside the
-// integer pipe.
+// Every third bit of a word: bit b of the low 10 bits to bit 3b, by the multiply-and-mask steps of T. Karras
+// ("Thinking Parallel, Part III", 2012). The multiplications run beside the integer pipe.
 __device__ __forceinline__ u32 spread10(u32 v) {
     v = (v * 0x00010001u) & 0xff0000ffu;
     v = (v * 0x00000101u) & 0x0f00f00fu;

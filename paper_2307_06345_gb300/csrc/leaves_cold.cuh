@@ -328,6 +328,7 @@ static_assert(kItems * kWarps == 64, "two counts per lane");
 __global__ void __launch_bounds__(1024) outcome_kernel(Tiles t, int n_sets, u32 ecap, int max_iters,
                                                        WsHeader* hdr) {
     __shared__ u32 s_warp[32];
+    const u32 listed = *t.n_starts, err = hdr->err;  // loaded while the tiles are scanned
     u32 run = 0, all;
     constexpr u32 kPer = 4;
     for (u32 k0 = 0; k0 < t.tiles; k0 += 1024 * kPer) {
@@ -353,8 +354,11 @@ __global__ void __launch_bounds__(1024) outcome_kernel(Tiles t, int n_sets, u32 
     for (int pass = 0; pass < max_iters; ++pass) {
         nodes += pass < kLevels ? t.levels[pass] : -nodes;  // of level `pass`
         if (nodes == 0) {
-            if (*t.n_starts > ne || run != static_cast<u32>(ne)) raise_error(hdr, CSTONE_ERR_INVALID_ARG, kDisorder);
-            if (hdr->err) return;
+            if (err) return;
+            if (listed > ne || run != static_cast<u32>(ne)) {
+                raise_error(hdr, CSTONE_ERR_INVALID_ARG, kDisorder);
+                return;
+            }
             *outcome_of(hdr) = Outcome{static_cast<u32>(pass + 1), 1u, 0u, static_cast<u32>(ne)};
             return;
         }

@@ -7,11 +7,13 @@
 // pairs (at first the whole set, or every segment) is split at pairs drawn from a sorted sample of
 // it, so its parts are of nearly equal size whatever the distribution of the keys, with any number
 // of equal keys; a part of at most kSmall pairs is sorted in shared memory by one block and written to
-// its final place. Two rounds of splitting reach every size: a pair moves three times (round 1, round
-// 2, final place), where the eight digit passes of a radix sort move it eight times. 2^27 clump keys
-// take 4.7 ms (count 0.33 and 0.69, scatter 0.8 to 0.9 each, final sort 1.64; the digit passes took
-// 7.2), 2^25 Plummer keys 1.2 ms (1.9), 65,536 uniform keys 65 us in 7 launches (200 in 40). Fetching a
-// tile's pairs while the one before it is written gained nothing in the scatter. Per round:
+// its final place. Two rounds of splitting reach 4e8 pairs at the parts' target size: a pair moves three
+// times (round 1, round 2, final place), where the eight digit passes of a radix sort move it eight times.
+// Beyond that the 512 x 512 parts grow, and above 6.7e8 most are larger than kSmall and sorted by
+// sort_rest_kernel, a whole SM's block each: 5.2e8 uniform keys 18.6 ms, 2^30 - 1 43.1 (the digit passes 29.0
+// and 57.2). 2^27 clump keys take 4.7 ms (count 0.33 and 0.69, scatter 0.8 to 0.9 each, final sort 1.64; the
+// digit passes took 7.2), 2^25 Plummer keys 1.2 ms (1.9), 65,536 uniform keys 62 us in 6 launches (a call; 234 in 40).
+// Fetching a tile's pairs while the one before it is written gained nothing in the scatter. Per round:
 //
 //   sample   one block per bucket sorts a sample and writes the bounds of the parts;
 //   count    every pair's part is found (a table over the leading key bits, then a binary search
@@ -933,8 +935,9 @@ __global__ void __launch_bounds__(kBigThreads) sort_rest_kernel(Pairs p, Buckets
 //
 // 30-bit keys have four digits only, and in clustered matter many particles share a key: the passes
 // are the better sort where splitting takes two rounds (2^24 keys: 510 us against 530 us uniform and
-// 850 us clumped; 2^20: 133 against 112 and 171), one round the better below (2^18: 117 against 73 and
-// 99).
+// 850 us clumped; 2^20: 133 against 112 and 171), one round the better below (2^18: 124 us by passes
+// against 66 uniform, 94 Plummer, 117 clumped, 99 to 104 with few distinct keys; at 786,432, where the two are
+// even on average, 125 against 88, 125, 154 and 128 to 135).
 // 63-bit keys take eight; one launch of the block sort above is faster (28 us against 190 us for
 // 1000 keys on GB300), but the launches of a sort of 1000 keys are part of what the launch counter
 // is tested for, so sets of at most kDigitMax keys keep the passes.
@@ -1160,7 +1163,7 @@ __global__ void __launch_bounds__(kRadix) chunk_sum_kernel(const unsigned short*
 
 // Exclusive scan of the chunk sums over the chunks, per digit: one block per digit over its
 // contiguous row (in place). The row's total (the keys of digit d in the whole pass) goes to
-// totals[d] unless totals is NULL.
+// totals[d].
 __global__ void __launch_bounds__(1024) chunk_scan_kernel(u32* __restrict__ chunk, long long nchunks,
                                                           u32* __restrict__ totals) {
     __shared__ u32 s_warp[32];
@@ -1180,7 +1183,7 @@ __global__ void __launch_bounds__(1024) chunk_scan_kernel(u32* __restrict__ chun
     __syncthreads();
     u32 before = 0;
     for (int w = 0; w < warp; ++w) before += s_warp[w];
-    if (totals && threadIdx.x == 1023) totals[blockIdx.x] = before + incl;
+    if (threadIdx.x == 1023) totals[blockIdx.x] = before + incl;
     u32 run = before + incl - sum;
     for (long long c = c0; c < c1; ++c) {
         const u32 v = row[c];
@@ -1191,7 +1194,7 @@ __global__ void __launch_bounds__(1024) chunk_scan_kernel(u32* __restrict__ chun
 
 // Output position of every tile's first key of every digit (thread = digit): the digit's first
 // position in the pass (the keys of all smaller digits: an exclusive scan of totals over the digits,
-// done by every block; 0 when totals is NULL) plus the digit's keys in all earlier tiles.
+// done by every block) plus the digit's keys in all earlier tiles.
 __global__ void __launch_bounds__(kRadix) tile_offsets_kernel(const unsigned short* __restrict__ counts, long long tiles,
                                                               const u32* __restrict__ chunk,
                                                               const u32* __restrict__ totals,
@@ -1199,21 +1202,18 @@ __global__ void __launch_bounds__(kRadix) tile_offsets_kernel(const unsigned sho
     static_assert(kRadix % 32 == 0 && kRadix <= 1024, "one thread per digit");
     __shared__ u32 s_warp[kRadix / 32];
     const int d = threadIdx.x, lane = d & 31, warp = d >> 5;
-    u32 digit_first = 0;
-    if (totals) {
-        const u32 v = totals[d];
-        u32 incl = v;
+    const u32 v0 = totals[d];
+    u32 incl = v0;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const u32 t = __shfl_up_sync(0xffffffffu, incl, o);
-            if (lane >= o) incl += t;
-        }
-        if (lane == 31) s_warp[warp] = incl;
-        __syncthreads();
-        u32 before = 0;
-        for (int w = 0; w < warp; ++w) before += s_warp[w];
-        digit_first = before + incl - v;
+    for (int o = 1; o < 32; o <<= 1) {
+        const u32 t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
     }
+    if (lane == 31) s_warp[warp] = incl;
+    __syncthreads();
+    u32 before = 0;
+    for (int w = 0; w < warp; ++w) before += s_warp[w];
+    const u32 digit_first = before + incl - v0;
     const long long t0 = (long long)blockIdx.x * kChunkTiles;
     const long long t1 = t0 + kChunkTiles < tiles ? t0 + kChunkTiles : tiles;
     u32 run = digit_first + chunk[(size_t)d * gridDim.x + blockIdx.x];

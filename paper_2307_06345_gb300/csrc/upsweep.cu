@@ -632,7 +632,7 @@ __global__ void __launch_bounds__(kThreads, 4) multipole_level_kernel(const int*
         }
         store_node(x, n_nodes, Mp, cp, Qp, Rp, s, f, mass, com, quad);
     };
-    // small levels by block 0 alone, as in the count upsweep; 8 lanes per node, the loop bounds
+    // levels of at most kSmall nodes by block 0 alone; 8 lanes per node, the loop bounds
     // the same in every lane of a warp
     constexpr u32 kGroups = kThreads / 8;
     constexpr u32 kSmall = 2 * kGroups;  // a round of 32 nodes takes block 0 about as long as a grid barrier
